@@ -194,7 +194,8 @@ __global__ void __launch_bounds__(256, 3) k_assemble(MeshView m, const int32_t *
             if (lane >= d) incl += t;
         }
         const int npairs = __shfl_sync(0xffffffffu, incl, 31);
-        if (lane <= nK) sm.poff[lane] = incl - box;  // lane nK holds the total
+        if (lane < nK) sm.poff[lane] = incl - box;
+        if (lane == 0) sm.poff[nK] = npairs;  // nK may be 32: no lane of its own
         __syncwarp();
         const bool table = npairs <= BallSmem<real>::kPairCap;  // warp-uniform
         // 3. every pair's weight once, spread over all lanes; then each

@@ -479,3 +479,30 @@ def test_error_statuses(bc):
     with pytest.raises(bc.BcharError) as e:
         bc.Mesh(wl.coords, -wl.phi)
     assert e.value.name == "INVALID_ARG"
+
+
+def test_cells_of_32_balls_match_oracle(bc):
+    """Cells of the largest ball count (4 x 4 x 2 = 32, one per lane of a
+    warp): widths 2 : 2 : 1 give every second cell 32 balls.  The last ball's
+    candidates end at the row's total, which no lane of its own holds."""
+    x = np.cumsum([0.0, 0.25, 0.25, 0.25, 0.25])
+    z = np.cumsum([0.0, 0.125, 0.2, 0.125, 0.2, 0.125, 0.225])
+    wl = inputs.workload("deform3d_128", n=4)
+    coords = [x, x, z / z[-1]]
+    phi = np.random.Generator(np.random.PCG64(8)).uniform(0.1, 0.3, 4 * 4 * 6)
+    om = oracle.Mesh(coords, phi)
+    assert oracle.ball_counts(om).max() == 32
+    faces = inputs.deform3d_faces(coords)
+    c = np.random.Generator(np.random.PCG64(9)).uniform(size=om.nc)
+    mesh = bc.Mesh(coords, phi, bc.default_options())
+    import torch
+    mesh.set_velocity(faces)
+    c_in = torch.tensor(c, device="cuda")
+    c_out = torch.empty_like(c_in)
+    info = mesh.step(wl.dt, c_in, c_out)
+    ref = oracle.step(om, faces, wl.dt, c)
+    e0 = _row_rel_err(_csr(mesh, 0), ref["A0"])
+    assert np.mean(e0 <= 1e-10) >= 0.99
+    assert np.abs(c_out.cpu().numpy() - ref["c"]).sum() / np.abs(ref["c"]).sum() <= 1e-5
+    assert abs(info["mass_after"] - info["mass_before"]) <= 1e-12 * info["mass_before"]
+    mesh.close()
