@@ -220,11 +220,12 @@ enum {
 /* Measurement aid: replay the kernel of one stage `reps` times on the data of
  * the last step, on the handle's stream, and return the mean duration of one
  * launch in milliseconds (CUDA events around the replays).  CG_MATVEC, UPDATE,
- * SMOOTH and VCYCLE are replayed from one CUDA graph of `reps` launches
+ * SMOOTH and SCALING are replayed from one CUDA graph of `reps` launches
  * (captured on a private stream), so that host launch overhead is not
- * measured; SCALING too (it writes the scaling factors, which the step no
- * longer needs).  VCYCLE (a chain of kernels, one per pass and level) needs a
- * step that built the multigrid hierarchy, like SMOOTH.  The replays do
+ * measured (SCALING writes the scaling factors, which the step no longer
+ * needs).  VCYCLE (one launch per application, which loads the hierarchy's rows
+ * before the cycle) needs a step that built the multigrid hierarchy, like
+ * SMOOTH.  The replays do
  * not change the result of the last step (exports stay valid) except that
  * BCHAR_STAGE_TRACK overwrites the tracked balls with the same values.
  * Errors: INVALID_ARG (no step yet, bad stage, reps < 1), CUDA. */

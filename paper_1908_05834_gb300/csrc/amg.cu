@@ -1,114 +1,87 @@
-// Aggregation multigrid preconditioner for the minimisation's linear system.
+// The aggregation-multigrid hierarchy of the minimisation's linear system,
+// built by one cooperative kernel.
 //
-// The system (A-hat A-hat^T + W) y = F of the penalised minimisation is, after
-// flipping the sign of the column unknowns (S = diag(1 rows, -1 columns)), the
-// M-matrix L = [[D_r, -W], [-W^T, D_c]] + diag(w): a weighted graph Laplacian
-// of the bipartite row/column graph (edge weights a_ij^2) plus a small
-// positive shift.  Its conditioning is poor on two counts: mesh-scale smooth
-// modes, and weak links (near-tangent ball overlaps give a_ij that are orders
-// of magnitude below the row's main entries).  A cluster of nodes held to the
-// rest only by weak links has a near-null mode (constant on the cluster); the
-// coarse levels keep that mode only if no aggregate straddles the weak links.
-// So the aggregation follows strong links alone:
+// The system is the symmetric M-matrix L = diag(ex) + graph Laplacian of
+// weights w > 0 on the finest level's nodes (the columns of A once the rows are
+// eliminated, schur.cu; or rows and columns), a level's operator being kept as
+// (diagonal, weights): L = dg - W, dg_i = ex_i + sum_j w_ij.  The excess ex
+// (the shift) is carried separately because it is down to ~1e-14 of the
+// weights and differences of diagonals would cancel it away.
+//
+// The conditioning is poor on two counts: mesh-scale smooth modes, and weak
+// links (near-tangent ball overlaps).  A cluster of nodes held to the rest only
+// by weak links has a near-null mode (constant on the cluster); the coarse
+// levels keep that mode only if no aggregate straddles the weak links.  So the
+// aggregation follows strong links alone:
 //   - an edge is strong when its weight is at least kStrength sqrt(d_i d_j);
-//   - each level pairs every node with its heaviest strong neighbour when the
+//   - each level pairs every node with its top-ranked strong neighbour when the
 //     choice is mutual (kHandshakes rounds, each among the nodes still
-//     unpaired); a node left unpaired joins the aggregate of its heaviest
-//     strong neighbour when that one is paired, else stays single;
-//   - a node without any off-diagonal entry (a whole connected component
-//     that has collapsed into one node, or an isolated row or column) leaves
-//     the hierarchy: its equation is solved exactly by the smoother (weight 1
-//     instead of kOmega) and it has no coarse counterpart;
-//   - so does a node whose off-diagonal weights sum to at most kDominant of
-//     its diagonal (a constraint held by its shift: in the minimisation's late
-//     iterations, one priced by the linear part of the penalty, or one whose
-//     entries all sit at a bound).  The smoother alone reduces its error by
-//     about that ratio per sweep, and left in, such nodes stall the coarsening
-//     (they have no strong neighbour, so every level keeps them as singletons
-//     and the coarsest level stays large).  Its edges to the nodes that stay
-//     are carried into their coarse shift, so the coarse operator is still the
-//     Galerkin product;
-//   - coarsening stops when a level would keep more than kStall of its
-//     remaining nodes, or has at most kCoarsest of them;
-//   - the coarse operator is the Galerkin product P^T L P for the piecewise-
-//     constant P of the aggregates (coarse edge = sum of fine edges between
-//     two aggregates).  Its diagonal is formed as the coarse node's excess
-//     (the sum of its members' shifts) plus the sum of its coarse edge
-//     weights, not as member diagonals minus internal edges: the shift is
-//     ~1e-14 of the edge weights and the subtraction would cancel it away;
-//   - a symmetric V-cycle (one damped-Jacobi sweep before and after the
-//     coarse correction, Jacobi sweeps on the coarsest level) is applied as
-//     the preconditioner of the conjugate gradients; per level it takes three
-//     kernels (pre-smoothing fused with the residual, restriction,
-//     prolongation fused with post-smoothing).
-// Every sum runs in a fixed order, so the hierarchy and its application are
-// deterministic.
+//     unpaired); a node left unpaired joins the aggregate of its top-ranked
+//     neighbour when that edge carries kAttach of its diagonal, else stays single;
+//   - a node whose off-diagonal weights sum to at most kDominant of its
+//     diagonal (a constraint held by its shift) leaves the hierarchy: the
+//     smoother alone reduces its error by about that ratio per sweep, and left
+//     in, such nodes stall the coarsening.  Its edges to the nodes that stay are
+//     carried into their coarse shift, so the coarse operator is the Galerkin
+//     product P^T L P for the piecewise-constant P of the aggregates;
+//   - coarsening stops at kDense nodes (that level's inverse is formed), when a
+//     level would keep more than kStall of its remaining nodes, or when the
+//     arrays are full.
+// Neighbours are ranked by (binary exponent of the weight, symmetric hash of
+// the edge): by the exact weight, the weights of smooth flows grow along the
+// strong chains of the graph, every node points the same way and almost no
+// choice is mutual.
+//
+// Why one kernel: a level takes about twenty-five dependent passes of a few
+// microseconds; launched one by one, with the level sizes read back by the
+// host, a build took 1.5 to 3 ms on meshes of 10^3 to 6 x 10^4 cells, and an
+// interior point builds 15 to 75 of them.  Here seven passes per level run
+// between grid barriers (pairing ranks fused with the attachment and leaving
+// tests, the leader decisions evaluated in one pass from the ranks, one pass
+// per coarse row instead of count and fill), the sizes stay on the device, and
+// levels of at most kBlockEntries entries are built by block 0 alone between
+// block barriers.  The arithmetic does not depend on where a row is stored
+// (block shares of the entry arrays are claimed by an atomic cursor), and every
+// sum runs in a fixed order: the hierarchy is deterministic.
 #include <math.h>
+#include <stddef.h>
 
 #include "amg.cuh"
 #include "device.cuh"
+#include "gridbar.cuh"
 
 namespace bchar {
 
-#define GRID_STRIDE(i, n)                                                                    \
-    for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < (n); \
-         i += static_cast<int64_t>(gridDim.x) * blockDim.x)
-
-constexpr int kCoarseCap = 384;       // neighbours a coarse node may collect before merging
-constexpr int64_t kCoarsest = 128;    // stop coarsening at this many nodes
-constexpr int64_t kOneBlock = 4096;   // levels up to this size are cycled by one block
-constexpr int kMaxLevels = 40;
-constexpr int kHandshakes = 4;        // matching rounds per level
+constexpr int kHandshakes = 2;        // matching rounds (four gave the same iteration counts)
 constexpr double kStall = 0.9;        // stop coarsening when a level keeps this fraction of nodes
-constexpr double kOmega = 0.9;        // Jacobi damping (rows with off-diagonal entries)
 constexpr double kStrength = 0.1;     // strong edge: w_ij >= kStrength sqrt(d_i d_j)
 constexpr double kAttach = 0.25;      // a leftover node follows an edge carrying this share of its diagonal
-constexpr double kDominant = 0.25;    // a node leaves the hierarchy when its off-diagonal sum is this share of its diagonal
-constexpr int kCoarsestSweeps = 40;   // sweeps of a one-block coarsest level
-constexpr int64_t kFuseBelow = 1 << 19;  // levels smaller than this fuse prolongation with smoothing
-constexpr int kLargeCoarsestSweeps = 20;
-constexpr int kDominantSweeps = 4;
+constexpr double kDominant = 0.25;    // a node leaves when its off-diagonal sum is this share of its diagonal
+// Jacobi damping of rows with off-diagonal entries: on the eliminated system
+// 0.7, 0.8, 0.9 took 2 595, 2 545, 2 676 iterations on a 128^2 stretched step and
+// 827, 810, 839 on a porous 24^3 one; 1.0 and above does not converge.
+constexpr double kOmega = 0.8;
+constexpr int kLargeSweeps = 20;      // Jacobi sweeps of a coarsest level that is not solved by its inverse
+constexpr int kDominantSweeps = 4;    // the same when all of its nodes are diagonally dominant
 
-// ---------------------------------------------------------------- level 0
+constexpr int kWarpRaw = 256;                          // entries of a coarse row merged by one warp
+constexpr int kBlockRaw = kWarpRaw * (kBuildThreads / 32);  // by the whole block
+constexpr size_t kBuildSmem = static_cast<size_t>(kBlockRaw) * (sizeof(unsigned long long) + sizeof(double));
 
-// Row node l < nc: its entries come from row l of A (columns nc + j);
-// column node nc + j: from column j (rows i).  Values -a_ij^2.
-__global__ void k_level0_ptr(int64_t nc, int64_t nnz, const int64_t *row_ptr, const int64_t *col_ptr,
-                             int64_t *ptr0) {
-    dep_enter();
-    GRID_STRIDE(l, 2 * nc + 1) ptr0[l] = l <= nc ? row_ptr[l] : nnz + col_ptr[l - nc];
-}
-
-__global__ void k_level0_fill(int64_t nc, const int64_t *row_ptr, const int32_t *col, const int64_t *col_ptr,
-                              const int32_t *csc_row, const double *a2, const double *a2c, const int64_t *ptr0,
-                              int32_t *col0, double *val0) {
-    dep_enter();
-    GRID_STRIDE(l, 2 * nc) {
-        int64_t dst = ptr0[l];
-        if (l < nc) {
-            for (int64_t e = row_ptr[l]; e < row_ptr[l + 1]; ++e, ++dst) {
-                col0[dst] = static_cast<int32_t>(nc + col[e]);
-                val0[dst] = -a2[e];
-            }
-        } else {
-            const int64_t j = l - nc;
-            for (int64_t p = col_ptr[j]; p < col_ptr[j + 1]; ++p, ++dst) {
-                col0[dst] = csc_row[p];
-                val0[dst] = -a2c[p];
-            }
-        }
-    }
-}
-
-// ---------------------------------------------------------------- matching
-//
-// Neighbours are ranked by (weight class, edge hash): the class is the binary
-// exponent of the weight, so weights within a factor of two rank equal and a
-// symmetric hash of the edge decides between them.  Ranking by the exact
-// weight fails on smooth flows: the weights then grow monotonically along the
-// strong chains of the graph, every node points the same way and almost no
-// choice is mutual (on a uniform 261^2 mesh one level kept 92 % of its nodes).
-// Equal classes with hashed order put local maxima everywhere.
+struct BuildArgs {
+    HierView v;
+    int n0;          // nodes and entries of the finest level
+    int64_t e0;
+    int schur;       // 1: columns with the rows eliminated, 0: rows and columns
+    int64_t nc;
+    const int64_t *col_ptr;
+    const int32_t *csc_row;
+    const double *a2, *a2c, *diag, *exc;  // the bipartite system: weights by row and by column, 2 n_c diagonals and shifts
+    const double *g, *t;                  // a2 / sqrt(diag_row) per entry; exc / diag per row
+    const uint32_t *cs;                   // first contribution of each entry of the finest level
+    const int2 *pair;                     // contributions: two entries of one row of A
+    int32_t *best0, *best1, *partner, *att, *lead, *pos, *agg, *cnt, *cap;  // n0 each
+};
 
 __device__ __forceinline__ uint32_t edge_hash(int64_t i, int64_t j) {
     const uint64_t a = static_cast<uint64_t>(i < j ? i : j), b = static_cast<uint64_t>(i < j ? j : i);
@@ -121,1026 +94,751 @@ __device__ __forceinline__ uint32_t edge_hash(int64_t i, int64_t j) {
     return static_cast<uint32_t>(x);
 }
 
-// Is neighbour j (weight w > 0) ranked above the current best (class bc, hash bh, index b)?
-// The class is the exponent field of w's bits (monotone in w, read without
-// the FP64 pipe).
-__device__ __forceinline__ bool ranks_above(int64_t i, int32_t j, double w, int32_t b, int bc, uint32_t bh, int &cls,
-                                            uint32_t &hs) {
-    cls = static_cast<int>((__double_as_longlong(w) >> 52) & 0x7ff);
-    hs = edge_hash(i, j);
-    return b < 0 || cls > bc || (cls == bc && (hs > bh || (hs == bh && j < b)));
+// Rank of an edge: exponent field of the weight, then the hash.
+__device__ __forceinline__ unsigned long long edge_rank(int i, int j, double w) {
+    const unsigned long long cls = (static_cast<unsigned long long>(__double_as_longlong(w)) >> 52) & 0x7ffull;
+    return (cls << 32) | edge_hash(i, j);
 }
 
-// leave[i] = 1 when node i leaves the hierarchy: no off-diagonal entry, or
-// off-diagonal weights summing to at most kDominant d_i.
-__global__ void k_leaving(int64_t n, const int64_t *ptr, const int32_t *col, const double *val, const double *diag,
-                          int32_t *leave) {
-    dep_enter();
-    GRID_STRIDE(i, n) {
-        double w = 0.0;
-        for (int64_t e = ptr[i]; e < ptr[i + 1]; ++e)
-            if (col[e] != i) w -= val[e];
-        leave[i] = (ptr[i + 1] == ptr[i] || w <= kDominant * diag[i]) ? 1 : 0;
+// The higher-ranked of (key, j) and (k2, j2); j < 0 is none; ties go to the smaller node.
+__device__ __forceinline__ void take_higher(unsigned long long &key, int &j, unsigned long long k2, int j2) {
+    if (j2 >= 0 && (j < 0 || k2 > key || (k2 == key && j2 < j))) {
+        key = k2;
+        j = j2;
     }
 }
 
-// Top-ranked strong neighbour (off-diagonal weight w_ij = -l_ij > 0 with
-// w_ij >= kStrength sqrt(d_i d_j)) among the nodes that stay; with only_free,
-// among neighbours that are still unpaired.
-__global__ void k_heaviest(int64_t n, const int64_t *ptr, const int32_t *col, const double *val, const double *diag,
-                           const int32_t *leave, const int32_t *partner, int only_free, int32_t *best) {
-    dep_enter();
-    GRID_STRIDE(i, n) {
-        int32_t b = -1;
-        int bc = 0;
-        uint32_t bh = 0;
-        if (!leave[i] && (!only_free || partner[i] < 0)) {
-            const double di = diag[i];
-            for (int64_t e = ptr[i]; e < ptr[i + 1]; ++e) {
-                const int32_t j = col[e];
-                if (j == i || leave[j]) continue;
-                if (only_free && partner[j] >= 0) continue;
-                const double w = -val[e];
-                // strong: w >= kStrength sqrt(d_i d_j), compared squared (no FP64 square root)
-                if (!(w > 0.0) || !(w * w >= (kStrength * kStrength) * (di * diag[j]))) continue;
-                int cls;
-                uint32_t hs;
-                if (ranks_above(i, j, w, b, bc, bh, cls, hs)) {
-                    b = j;
-                    bc = cls;
-                    bh = hs;
+__device__ __forceinline__ bool leaves(const HierView &v, int64_t k) {
+    return v.rl[k] == 0 || v.ex[k] >= (1.0 - kDominant) * v.dg[k];
+}
+
+// Exclusive scan of one int per thread over the block (kBuildThreads); tmp: 33 ints of shared memory.
+__device__ __forceinline__ int block_scan(int x, int *tmp, int &total) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int incl = x;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    __syncthreads();  // tmp may still be read from the previous call
+    if (lane == 31) tmp[wid] = incl;
+    __syncthreads();
+    if (wid == 0) {
+        int t = tmp[lane], s = t;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int q = __shfl_up_sync(0xffffffffu, s, o);
+            if (lane >= o) s += q;
+        }
+        tmp[lane] = s - t;
+        if (lane == 31) tmp[32] = s;
+    }
+    __syncthreads();
+    total = tmp[32];
+    return tmp[wid] + incl - x;
+}
+
+__device__ __forceinline__ double warp_sum(double s) {
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
+// ---- the finest level's values: LPR lanes per row
+
+template <int LPR> __device__ void level0_values(const BuildArgs &a, int i0, int i1) {
+    const int lane = threadIdx.x & 31, sub = lane % LPR;
+    const HierView &v = a.v;
+    for (int r0 = i0 + static_cast<int>(threadIdx.x >> 5) * (32 / LPR); r0 < i1; r0 += blockDim.x / LPR) {
+        const int i = r0 + lane / LPR;
+        const bool ok = i < i1;
+        double s = 0.0, x = 0.0;
+        int len = 0;
+        if (ok) {
+            const int64_t e0 = v.rs[i];
+            len = v.rl[i];
+            if (a.schur) {
+                for (int e = sub; e < len; e += LPR) {
+                    double w = 0.0;
+                    const uint32_t k1 = a.cs[e0 + e + 1];
+                    for (uint32_t k = a.cs[e0 + e]; k < k1; ++k) {
+                        const int2 p = a.pair[k];
+                        w += a.g[p.x] * a.g[p.y];
+                    }
+                    v.ew[e0 + e] = w;
+                    s += w;
+                }
+                for (int64_t p = a.col_ptr[i] + sub; p < a.col_ptr[i + 1]; p += LPR) x += a.a2c[p] * a.t[a.csc_row[p]];
+            } else {
+                const bool row = i < a.nc;
+                const int64_t src = row ? e0 : a.col_ptr[i - a.nc];  // the row entries come first, in CSR order
+                for (int e = sub; e < len; e += LPR) v.ew[e0 + e] = row ? a.a2[src + e] : a.a2c[src + e];
+            }
+        }
+        for (int o = LPR / 2; o > 0; o >>= 1) {
+            s += __shfl_xor_sync(0xffffffffu, s, o);
+            x += __shfl_xor_sync(0xffffffffu, x, o);
+        }
+        if (ok && sub == 0) {
+            const double ex = a.schur ? a.exc[a.nc + i] + x : a.exc[i];
+            const double d = a.schur ? ex + s : a.diag[i];
+            v.ex[i] = ex;
+            v.dg[i] = d;
+            v.om[i] = (len == 0 ? 1.0 : kOmega) / d;
+        }
+    }
+}
+
+// ---- one matching round (LPR lanes per node of the level at node offset noff)
+
+template <int LPR>
+__device__ void rank_round(const BuildArgs &a, int64_t noff, int n, int i0, int i1, int round, const int32_t *bprev,
+                           int32_t *bcur) {
+    const HierView &v = a.v;
+    const int lane = threadIdx.x & 31, sub = lane % LPR;
+    volatile int32_t *partner = a.partner;
+    for (int r0 = i0 + static_cast<int>(threadIdx.x >> 5) * (32 / LPR); r0 < i1; r0 += blockDim.x / LPR) {
+        const int i = r0 + lane / LPR;
+        const bool ok = i < i1;
+        unsigned long long key = 0, akey = 0;
+        int bj = -1, aj = -1, mate = -3;
+        double wmax = 0.0, di = 0.0;
+        if (ok) {
+            di = v.dg[noff + i];
+            if (round == 0) {
+                mate = leaves(v, noff + i) ? -3 : -1;
+            } else {
+                mate = partner[i];
+                if (mate == -1) {  // did the previous round's choices meet?
+                    const int b = bprev[i];
+                    if (b >= 0 && bprev[b] == i) mate = b;
+                }
+            }
+            const bool open = mate == -1;
+            if (open) {
+                const int64_t e0 = v.rs[noff + i];
+                const int len = v.rl[noff + i];
+                for (int e = sub; e < len; e += LPR) {
+                    const int j = v.ecol[e0 + e];
+                    const double w = v.ew[e0 + e];
+                    if (!(w > 0.0)) continue;
+                    if (round == 0) {
+                        if (leaves(v, noff + j)) continue;
+                    } else {
+                        if (partner[j] != -1) continue;
+                        const int b = bprev[j];
+                        if (b >= 0 && bprev[b] == j) continue;
+                    }
+                    const unsigned long long k = edge_rank(i, j, w);
+                    if (round == 0) {
+                        wmax = fmax(wmax, w);
+                        take_higher(akey, aj, k, j);
+                    }
+                    // strong: w >= kStrength sqrt(d_i d_j), compared squared
+                    if (w * w >= (kStrength * kStrength) * (di * v.dg[noff + j])) take_higher(key, bj, k, j);
                 }
             }
         }
-        best[i] = b;
-    }
-}
-
-__global__ void k_handshake(int64_t n, const int32_t *best, int32_t *partner) {
-    dep_enter();
-    GRID_STRIDE(i, n) {
-        if (partner[i] >= 0) continue;
-        const int32_t b = best[i];
-        if (b >= 0 && best[b] == i) partner[i] = b;
-    }
-}
-
-// Attachment target of every node that stays: its top-ranked neighbour over
-// all edges to nodes that stay when the node's heaviest such edge carries at
-// least kAttach of its own diagonal, else -1.  The test is one-sided on
-// purpose: a leaf hanging off a hub by an edge that is strong for the leaf
-// (most of its diagonal) but weak for the hub should follow the hub.
-__global__ void k_attach_target(int64_t n, const int64_t *ptr, const int32_t *col, const double *val,
-                                const double *diag, const int32_t *leave, int32_t *att) {
-    dep_enter();
-    GRID_STRIDE(i, n) {
-        int32_t b = -1;
-        int bc = 0;
-        uint32_t bh = 0;
-        double wmax = 0.0;
-        for (int64_t e = leave[i] ? ptr[i + 1] : ptr[i]; e < ptr[i + 1]; ++e) {
-            const int32_t j = col[e];
-            if (j == i || leave[j]) continue;
-            const double w = -val[e];
-            if (!(w > 0.0)) continue;
-            wmax = fmax(wmax, w);
-            int cls;
-            uint32_t hs;
-            if (ranks_above(i, j, w, b, bc, bh, cls, hs)) {
-                b = j;
-                bc = cls;
-                bh = hs;
+        for (int o = LPR / 2; o > 0; o >>= 1) {
+            take_higher(key, bj, __shfl_xor_sync(0xffffffffu, key, o), __shfl_xor_sync(0xffffffffu, bj, o));
+            if (round == 0) {
+                take_higher(akey, aj, __shfl_xor_sync(0xffffffffu, akey, o), __shfl_xor_sync(0xffffffffu, aj, o));
+                wmax = fmax(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
             }
         }
-        att[i] = (b >= 0 && wmax >= kAttach * diag[i]) ? b : -1;
-    }
-}
-
-// Leaders, first pass.  A node that leaves the hierarchy gets leader -1
-// (no coarse node; counted in *isolated); a paired node, the smaller node of
-// its pair; an unpaired node whose attachment target is paired joins that
-// pair; every other node is left open (-2) for the second pass.
-__global__ void k_leaders1(int64_t n, const int32_t *leave, const int32_t *partner, const int32_t *att,
-                           int32_t *leader, int *isolated) {
-    dep_enter();
-    GRID_STRIDE(i, n) {
-        int32_t lead = -2;
-        if (leave[i]) {
-            atomicAdd(isolated, 1);
-            lead = -1;
-        } else if (partner[i] >= 0) {
-            const int32_t p = partner[i];
-            lead = i < p ? static_cast<int32_t>(i) : p;
-        } else {
-            const int32_t t = att[i];
-            if (t >= 0 && partner[t] >= 0) {
-                const int32_t q = partner[t];
-                lead = t < q ? t : q;
+        if (ok && sub == 0) {
+            bcur[i] = bj;
+            partner[i] = mate;
+            if (round == 0) {
+                // one-sided on purpose: a leaf hanging off a hub by an edge that is most of
+                // its own diagonal but little of the hub's should follow the hub
+                a.att[i] = (aj >= 0 && wmax >= kAttach * di) ? aj : -1;
+                a.cnt[i] = 0;
+                a.cap[i] = 0;
             }
         }
-        leader[i] = lead;
     }
 }
 
-// want[i]: the attachment target of an open node when that target is open
-// too, else -1.
-__global__ void k_want(int64_t n, const int32_t *att, const int32_t *leader, int32_t *want) {
-    dep_enter();
-    GRID_STRIDE(i, n) {
-        const int32_t t = att[i];
-        want[i] = (leader[i] == -2 && t >= 0 && leader[t] == -2) ? t : -1;
-    }
+// ---- leaders, from the ranks: -1 leaves; a paired node's is the smaller of
+// the pair; an unpaired node attached to a paired one joins that pair; of the
+// others, two attached to each other pair up, one attached to a node that is
+// itself not attached to an open node joins it, the rest lead themselves.
+
+__device__ __forceinline__ int mate_of(const BuildArgs &a, const int32_t *best, int i) {
+    const int p = a.partner[i];
+    if (p != -1) return p;
+    const int b = best[i];
+    return b >= 0 && best[b] == i ? b : -1;
 }
 
-// Leaders, second pass over the open nodes: two nodes that want each other
-// pair up (the smaller leads); a node that wants a node wanting nothing joins
-// it; every other open node leads itself.  Each leader leads itself, so
-// aggregates have no chains.  is_leader flags the leaders for the scan.
-__global__ void k_leaders2(int64_t n, const int32_t *want, int32_t *leader, int32_t *is_leader) {
-    dep_enter();
-    GRID_STRIDE(i, n) {
-        int32_t lead = leader[i];
-        if (lead == -2) {
-            const int32_t t = want[i];
-            if (t < 0)
-                lead = static_cast<int32_t>(i);
-            else if (want[t] == i)
-                lead = i < t ? static_cast<int32_t>(i) : t;
-            else if (want[t] < 0)
-                lead = t;
-            else
-                lead = static_cast<int32_t>(i);
-            leader[i] = lead;
-        }
-        is_leader[i] = lead == i ? 1 : 0;
+__device__ __forceinline__ int lead_first(const BuildArgs &a, const int32_t *best, int i) {
+    const int p = mate_of(a, best, i);
+    if (p == -3) return -1;
+    if (p >= 0) return min(i, p);
+    const int t = a.att[i];
+    if (t >= 0) {
+        const int q = mate_of(a, best, t);
+        if (q >= 0) return min(t, q);
     }
+    return -2;
 }
 
-__global__ void k_aggregates(int64_t n, const int32_t *leader, const int64_t *leader_pos, int32_t *agg,
-                             int32_t *count) {
-    dep_enter();
-    GRID_STRIDE(i, n) {
-        if (leader[i] < 0) {
-            agg[i] = -1;
-            continue;
-        }
-        const int32_t I = static_cast<int32_t>(leader_pos[leader[i]]);
-        agg[i] = I;
-        atomicAdd(&count[I], 1);
-    }
+__device__ __forceinline__ int wanted(const BuildArgs &a, const int32_t *best, int i) {  // i is open
+    const int t = a.att[i];
+    return t >= 0 && lead_first(a, best, t) == -2 ? t : -1;
 }
 
-__global__ void k_members_fill(int64_t n, const int32_t *agg, const int64_t *mptr, int32_t *fill, int32_t *mlist) {
-    dep_enter();
-    GRID_STRIDE(i, n) {
-        const int32_t I = agg[i];
-        if (I < 0) continue;
-        mlist[mptr[I] + atomicAdd(&fill[I], 1)] = static_cast<int32_t>(i);
-    }
+__device__ __forceinline__ int leader_of(const BuildArgs &a, const int32_t *best, int i) {
+    const int l = lead_first(a, best, i);
+    if (l != -2) return l;
+    const int t = wanted(a, best, i);
+    if (t < 0) return i;
+    const int b = wanted(a, best, t);
+    if (b == i) return min(i, t);
+    return b < 0 ? t : i;
 }
 
-// Members of each aggregate in increasing node order (small insertion sort).
-__global__ void k_members_sort(int64_t nco, const int64_t *mptr, int32_t *mlist) {
-    dep_enter();
-    GRID_STRIDE(I, nco) {
-        const int64_t b = mptr[I], e = mptr[I + 1];
-        for (int64_t p = b + 1; p < e; ++p) {
-            const int32_t v = mlist[p];
-            int64_t q = p;
-            while (q > b && mlist[q - 1] > v) {
-                mlist[q] = mlist[q - 1];
-                --q;
-            }
-            mlist[q] = v;
-        }
-    }
+// ---- coarse rows
+
+__device__ __forceinline__ int pow2_at_least(int n) {
+    int p = 32;
+    while (p < n) p <<= 1;
+    return p;
 }
 
-// ---------------------------------------------------------------- Galerkin coarse operator
-
-// Collect, sort and merge the coarse neighbours of coarse node I (internal
-// edges drop out of the Laplacian).  Returns the number of distinct
-// neighbours (or -1 on overflow); *eI receives the coarse excess.
-__device__ int coarse_row(int64_t I, const int64_t *mptr, const int32_t *mlist, const int64_t *ptr,
-                          const int32_t *col, const double *val, const double *exc, const int32_t *agg, int32_t *cbuf,
-                          double *vbuf, double *eI) {
-    int cnt = 0;
-    double e_sum = 0.0;
-    for (int64_t k = mptr[I]; k < mptr[I + 1]; ++k) {
-        const int32_t m = mlist[k];
-        e_sum += exc[m];
-        for (int64_t e = ptr[m]; e < ptr[m + 1]; ++e) {
-            const int32_t J = agg[col[e]];
-            if (J == I) continue;  // internal edge
-            if (J < 0) {           // an edge to a node without coarse counterpart: part of the coarse shift
-                e_sum -= val[e];
-                continue;
-            }
-            // insertion into the sorted buffer, merging equal columns
-            int pos = cnt;
-            while (pos > 0 && cbuf[pos - 1] > J) --pos;
-            if (pos > 0 && cbuf[pos - 1] == J) {
-                vbuf[pos - 1] += val[e];
-                continue;
-            }
-            if (cnt == kCoarseCap) return -1;
-            for (int q = cnt; q > pos; --q) {
-                cbuf[q] = cbuf[q - 1];
-                vbuf[q] = vbuf[q - 1];
-            }
-            cbuf[pos] = J;
-            vbuf[pos] = val[e];
-            ++cnt;
-        }
-    }
-    *eI = e_sum;
-    return cnt;
-}
-
-// Short coarse rows (2D): one thread per coarse node, merging by insertion.
-__global__ void k_coarse_count_thread(int64_t nco, const int64_t *mptr, const int32_t *mlist, const int64_t *ptr,
-                                      const int32_t *col, const double *val, const double *exc, const int32_t *agg,
-                                      int32_t *rowcnt, int *overflow) {
-    dep_enter();
-    int32_t cbuf[kCoarseCap];
-    double vbuf[kCoarseCap];
-    GRID_STRIDE(I, nco) {
-        double e;
-        const int c = coarse_row(I, mptr, mlist, ptr, col, val, exc, agg, cbuf, vbuf, &e);
-        if (c < 0) {
-            atomicOr(overflow, 1);
-            rowcnt[I] = 0;
-        } else {
-            rowcnt[I] = c;
-        }
-    }
-}
-
-__global__ void k_coarse_fill_thread(int64_t nco, const int64_t *mptr, const int32_t *mlist, const int64_t *ptr,
-                                     const int32_t *col, const double *val, const double *exc, const int32_t *agg,
-                                     const int64_t *cptr, int32_t *ccol, double *cval, double *cdiag, double *cexc) {
-    dep_enter();
-    int32_t cbuf[kCoarseCap];
-    double vbuf[kCoarseCap];
-    GRID_STRIDE(I, nco) {
-        double e;
-        const int c = coarse_row(I, mptr, mlist, ptr, col, val, exc, agg, cbuf, vbuf, &e);
-        const int64_t dst = cptr[I];
-        double d = e;
-        for (int k = 0; k < c; ++k) {
-            ccol[dst + k] = cbuf[k];
-            cval[dst + k] = vbuf[k];
-            d -= vbuf[k];
-        }
-        cdiag[I] = d;
-        cexc[I] = e;
-    }
-}
-
-// The same rows built by one warp per coarse node I: the members' entries are
-// gathered into shared memory in arrival order (members in order, then each
-// member's entries), sorted by (J, arrival), and each run of equal J is summed
-// by one lane in arrival order -- the order in which the insertion above adds
-// them, so the coarse operator is the same bit for bit.  A row with more than
-// kMergeCap raw entries is built by the warp's first lane with coarse_row.
-constexpr int kMergeCap = 512;
-constexpr int kMergeWarps = 4;  // warps per block
-struct MergeSmem {
-    int32_t key[kMergeCap];
-    int32_t pos[kMergeCap];
-    double val[kMergeCap];
-};
-
-// Gathers row I into sm; returns the raw entry count (> kMergeCap: not all
-// gathered) and the coarse excess in *eI (valid in every lane).
-__device__ int gather_row(int64_t I, const int64_t *mptr, const int32_t *mlist, const int64_t *ptr, const int32_t *col,
-                          const double *val, const double *exc, const int32_t *agg, MergeSmem &sm, double *eI) {
-    const int lane = threadIdx.x & 31;
-    int n = 0;
-    double e_sum = 0.0;
-    for (int64_t k = mptr[I]; k < mptr[I + 1]; ++k) {
-        const int32_t m = mlist[k];
-        e_sum += exc[m];
-        const int64_t b = ptr[m], e = ptr[m + 1];
-        for (int64_t base = b; base < e; base += 32) {
-            const int64_t idx = base + lane;
-            const int32_t J = idx < e ? agg[col[idx]] : I;
-            const bool keep = J != I && J >= 0;
-            // edges to nodes without coarse counterpart join the shift, added in entry order
-            // (the order of coarse_row)
-            const double shift = J < 0 ? -val[idx] : 0.0;
-            if (__any_sync(0xffffffffu, J < 0))
-                for (int q = 0; q < 32; ++q) e_sum += __shfl_sync(0xffffffffu, shift, q);
-            const unsigned mask = __ballot_sync(0xffffffffu, keep);
-            const int at = n + __popc(mask & ((1u << lane) - 1u));
-            if (keep && at < kMergeCap) {
-                sm.key[at] = J;
-                sm.pos[at] = at;
-                sm.val[at] = val[idx];
-            }
-            n += __popc(mask);
-        }
-    }
-    *eI = e_sum;
-    __syncwarp();
-    return n;
-}
-
-// Sorts the first n gathered entries by (key, pos) (bitonic, padded to a
-// power of two with keys that sort last).
-__device__ void sort_row(MergeSmem &sm, int n) {
-    const int lane = threadIdx.x & 31;
-    int P = 32;
-    while (P < n) P <<= 1;
-    for (int i = n + lane; i < P; i += 32) {
-        sm.key[i] = 0x7fffffff;
-        sm.pos[i] = 0x7fffffff;
-        sm.val[i] = 0.0;
-    }
-    __syncwarp();
-    for (int k = 2; k <= P; k <<= 1) {
+// Sorts keys[0, P) ascending with nt threads (tid in [0, nt)); sync() orders them.
+template <class Sync> __device__ void bitonic(unsigned long long *keys, int P, int tid, int nt, Sync sync) {
+    for (int k = 2; k <= P; k <<= 1)
         for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = lane; i < P; i += 32) {
+            for (int i = tid; i < P; i += nt) {
                 const int l = i ^ j;
                 if (l > i) {
-                    const bool up = (i & k) == 0;
-                    const bool greater = sm.key[i] > sm.key[l] || (sm.key[i] == sm.key[l] && sm.pos[i] > sm.pos[l]);
-                    if (greater == up) {
-                        const int32_t tk = sm.key[i], tp = sm.pos[i];
-                        const double tv = sm.val[i];
-                        sm.key[i] = sm.key[l];
-                        sm.pos[i] = sm.pos[l];
-                        sm.val[i] = sm.val[l];
-                        sm.key[l] = tk;
-                        sm.pos[l] = tp;
-                        sm.val[l] = tv;
+                    const unsigned long long x = keys[i], y = keys[l];
+                    if ((x > y) == ((i & k) == 0)) {
+                        keys[i] = y;
+                        keys[l] = x;
                     }
                 }
             }
-            __syncwarp();
+            sync();
         }
-    }
 }
 
-// Runs of equal keys in the sorted entries: calls out(r, key, sum) once per
-// run (r = run index, runs in key order; the sum in arrival order); returns
-// the number of runs.
-template <class F> __device__ int merge_runs(const MergeSmem &sm, int n, F out) {
+// Merges the sorted entries (key: coarse node << 32 | arrival; all ones: none)
+// into the coarse row I, summing equal nodes in arrival order; one warp.
+__device__ void merge_row(const HierView &v, int64_t noff2, int I, const unsigned long long *keys, const double *vals,
+                          int n, double ex, int &len) {
     const int lane = threadIdx.x & 31;
+    const int64_t dst = v.rs[noff2 + I];
     int runs = 0;
+    double d = 0.0;
     for (int base = 0; base < n; base += 32) {
         const int i = base + lane;
-        const bool start = i < n && (i == 0 || sm.key[i] != sm.key[i - 1]);
+        const unsigned long long k = i < n ? keys[i] : ~0ull;
+        const int J = static_cast<int>(k >> 32);
+        const bool start = k != ~0ull && (i == 0 || static_cast<int>(keys[i - 1] >> 32) != J);
         const unsigned mask = __ballot_sync(0xffffffffu, start);
         if (start) {
-            const int r = runs + __popc(mask & ((1u << lane) - 1u));
-            double sum = sm.val[i];
-            for (int q = i + 1; q < n && sm.key[q] == sm.key[i]; ++q) sum += sm.val[q];
-            out(r, sm.key[i], sum);
+            double s = vals[k & 0xffffffffull];
+            for (int q = i + 1; q < n && static_cast<int>(keys[q] >> 32) == J && keys[q] != ~0ull; ++q)
+                s += vals[keys[q] & 0xffffffffull];
+            const int64_t at = dst + runs + __popc(mask & ((1u << lane) - 1u));
+            v.ecol[at] = J;
+            v.ew[at] = s;
+            d += s;
         }
         runs += __popc(mask);
     }
-    return runs;
-}
-
-__global__ void __launch_bounds__(32 * kMergeWarps) k_coarse_count(int64_t nco, const int64_t *mptr,
-                                                                   const int32_t *mlist, const int64_t *ptr,
-                                                                   const int32_t *col, const double *val,
-                                                                   const double *exc, const int32_t *agg,
-                                                                   int32_t *rowcnt, int *overflow) {
-    dep_enter();
-    __shared__ MergeSmem sm_all[kMergeWarps];
-    MergeSmem &sm = sm_all[threadIdx.x >> 5];
-    const int lane = threadIdx.x & 31;
-    const int64_t nwarps = static_cast<int64_t>(gridDim.x) * kMergeWarps;
-    for (int64_t I = blockIdx.x * static_cast<int64_t>(kMergeWarps) + (threadIdx.x >> 5); I < nco; I += nwarps) {
-        double e;
-        const int n = gather_row(I, mptr, mlist, ptr, col, val, exc, agg, sm, &e);
-        int c;
-        if (n == 0) {
-            c = 0;
-        } else if (n <= kMergeCap) {
-            sort_row(sm, n);
-            c = merge_runs(sm, n, [](int, int32_t, double) {});
-        } else {
-            c = 0;
-            if (lane == 0) {
-                int32_t cbuf[kCoarseCap];
-                double vbuf[kCoarseCap];
-                c = coarse_row(I, mptr, mlist, ptr, col, val, exc, agg, cbuf, vbuf, &e);
-            }
-            c = __shfl_sync(0xffffffffu, c, 0);
-        }
-        if (lane == 0) {
-            if (c < 0) {
-                atomicOr(overflow, 1);
-                rowcnt[I] = 0;
-            } else {
-                rowcnt[I] = c;
-            }
-        }
-        __syncwarp();
+    d = warp_sum(d) + ex;
+    if (lane == 0) {
+        v.rl[noff2 + I] = runs;
+        v.dg[noff2 + I] = d;
+        v.ex[noff2 + I] = ex;
+        v.om[noff2 + I] = (runs == 0 ? 1.0 : kOmega) / d;
     }
+    len = runs;
 }
 
-__global__ void __launch_bounds__(32 * kMergeWarps) k_coarse_fill(int64_t nco, const int64_t *mptr,
-                                                                  const int32_t *mlist, const int64_t *ptr,
-                                                                  const int32_t *col, const double *val,
-                                                                  const double *exc, const int32_t *agg,
-                                                                  const int64_t *cptr, int32_t *ccol, double *cval,
-                                                                  double *cdiag, double *cexc) {
-    dep_enter();
-    __shared__ MergeSmem sm_all[kMergeWarps];
-    MergeSmem &sm = sm_all[threadIdx.x >> 5];
+// Puts the cnt members at own[0, cnt) in node order (one warp).
+__device__ void sort_members(int32_t *own, int cnt) {
     const int lane = threadIdx.x & 31;
-    const int64_t nwarps = static_cast<int64_t>(gridDim.x) * kMergeWarps;
-    for (int64_t I = blockIdx.x * static_cast<int64_t>(kMergeWarps) + (threadIdx.x >> 5); I < nco; I += nwarps) {
-        double e;
-        const int n = gather_row(I, mptr, mlist, ptr, col, val, exc, agg, sm, &e);
-        const int64_t dst = cptr[I];
-        int c;
-        if (n <= kMergeCap) {
-            sort_row(sm, n);
-            c = merge_runs(sm, n, [&](int r, int32_t J, double v) {
-                ccol[dst + r] = J;
-                cval[dst + r] = v;
-            });
-        } else {
-            c = 0;
-            if (lane == 0) {
-                int32_t cbuf[kCoarseCap];
-                double vbuf[kCoarseCap];
-                c = coarse_row(I, mptr, mlist, ptr, col, val, exc, agg, cbuf, vbuf, &e);
-                for (int k = 0; k < c; ++k) {
-                    ccol[dst + k] = cbuf[k];
-                    cval[dst + k] = vbuf[k];
-                }
-            }
-            c = __shfl_sync(0xffffffffu, c, 0);
-        }
+    if (cnt <= 32) {
+        const int m = lane < cnt ? own[lane] : 0x7fffffff;
+        int rank = 0;
+        for (int q = 0; q < cnt; ++q) rank += __shfl_sync(0xffffffffu, m, q) < m ? 1 : 0;
         __syncwarp();
-        if (lane == 0) {  // the diagonal from the merged entries, in their order
-            double d = e;
-            for (int k = 0; k < c; ++k) d -= cval[dst + k];
-            cdiag[I] = d;
-            cexc[I] = e;
+        if (lane < cnt) own[rank] = m;
+    } else if (lane == 0) {
+        for (int p = 1; p < cnt; ++p) {
+            const int m = own[p];
+            int q = p;
+            for (; q > 0 && own[q - 1] > m; --q) own[q] = own[q - 1];
+            own[q] = m;
         }
-        __syncwarp();
     }
+    __syncwarp();
 }
 
-// The coarse operator of one level: warp per row where the finer level's rows
-// are wide (the per-thread insertion then works in local memory), thread per
-// row where they are short (a warp's sort would cost more than the merge).
-static bool wide_rows(const AmgLevel &F) { return F.nnz > 8 * F.n; }
-
-static void coarse_count(bchar_mesh_t m, const AmgLevel &F, const AmgLevel &C, int64_t ncoarse, const double *fexc,
-                         int32_t *rowcnt, int *overflow) {
-    AmgLevel &Fm = const_cast<AmgLevel &>(F);
-    AmgLevel &Cm = const_cast<AmgLevel &>(C);
-    if (wide_rows(F))
-        launch_dep(k_coarse_count, blocks_for(ncoarse * 32, 32 * kMergeWarps), 32 * kMergeWarps, m->stream, 
-            ncoarse, ptr<int64_t>(Cm.mptr), ptr<int32_t>(Cm.mlist), ptr<int64_t>(Fm.ptr), ptr<int32_t>(Fm.col),
-            ptr<double>(Fm.val), fexc, ptr<int32_t>(Fm.agg), rowcnt, overflow);
-    else
-        launch_dep(k_coarse_count_thread, blocks_for(ncoarse, 128), 128, m->stream, 
-            ncoarse, ptr<int64_t>(Cm.mptr), ptr<int32_t>(Cm.mlist), ptr<int64_t>(Fm.ptr), ptr<int32_t>(Fm.col),
-            ptr<double>(Fm.val), fexc, ptr<int32_t>(Fm.agg), rowcnt, overflow);
-    ++m->launches;
+// Coarse row I (raw <= kWarpRaw entries over its members), by one warp.
+__device__ int coarse_row_warp(const BuildArgs &a, int64_t noff, int64_t noff2, int I, int raw, unsigned long long *keys,
+                               double *vals) {
+    const HierView &v = a.v;
+    const int lane = threadIdx.x & 31;
+    const int cnt = v.gc[noff2 + I];
+    int32_t *own = v.own + noff + v.gs[noff2 + I];
+    sort_members(own, cnt);
+    double ex = 0.0;
+    int done = 0;  // entries of the members before this batch of 32
+    for (int m0 = 0; m0 < cnt; m0 += 32) {
+        const int m = m0 + lane < cnt ? own[m0 + lane] : -1;
+        const int len = m >= 0 ? v.rl[noff + m] : 0;
+        const int64_t e0 = m >= 0 ? v.rs[noff + m] : 0;
+        if (m >= 0) ex += v.ex[noff + m];
+        int incl = len;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        const int tot = __shfl_sync(0xffffffffu, incl, 31);
+        const int nm = min(32, cnt - m0);
+        for (int base = 0; base < tot; base += 32) {
+            const int t = base + lane;
+            int k = 0;  // the member holding raw entry t
+            for (int q = 0; q < nm - 1; ++q) k += t >= __shfl_sync(0xffffffffu, incl, q) ? 1 : 0;
+            const int before = __shfl_sync(0xffffffffu, incl - len, k);
+            const int64_t e = __shfl_sync(0xffffffffu, e0, k) + (t - before);
+            if (t < tot) {
+                const int J = a.agg[v.ecol[e]];
+                const double w = v.ew[e];
+                if (J < 0) ex += w;  // an edge to a node without coarse counterpart joins the shift
+                keys[done + t] = (J < 0 || J == I) ? ~0ull
+                                                   : (static_cast<unsigned long long>(static_cast<unsigned>(J)) << 32) |
+                                                         static_cast<unsigned>(done + t);
+                vals[done + t] = w;
+            }
+        }
+        done += tot;
+    }
+    ex = warp_sum(ex);
+    const int P = pow2_at_least(raw);
+    for (int i = raw + lane; i < P; i += 32) keys[i] = ~0ull;
+    __syncwarp();
+    bitonic(keys, P, lane, 32, [] { __syncwarp(); });
+    int len;
+    merge_row(v, noff2, I, keys, vals, raw, ex, len);
+    __syncwarp();
+    return len;
 }
 
-static void coarse_fill(bchar_mesh_t m, const AmgLevel &F, AmgLevel &C, int64_t ncoarse, const double *fexc) {
-    AmgLevel &Fm = const_cast<AmgLevel &>(F);
-    if (wide_rows(F))
-        launch_dep(k_coarse_fill, blocks_for(ncoarse * 32, 32 * kMergeWarps), 32 * kMergeWarps, m->stream, 
-            ncoarse, ptr<int64_t>(C.mptr), ptr<int32_t>(C.mlist), ptr<int64_t>(Fm.ptr), ptr<int32_t>(Fm.col),
-            ptr<double>(Fm.val), fexc, ptr<int32_t>(Fm.agg), ptr<int64_t>(C.ptr), ptr<int32_t>(C.col),
-            ptr<double>(C.val), ptr<double>(C.diag), ptr<double>(C.exc));
-    else
-        launch_dep(k_coarse_fill_thread, blocks_for(ncoarse, 128), 128, m->stream, 
-            ncoarse, ptr<int64_t>(C.mptr), ptr<int32_t>(C.mlist), ptr<int64_t>(Fm.ptr), ptr<int32_t>(Fm.col),
-            ptr<double>(Fm.val), fexc, ptr<int32_t>(Fm.agg), ptr<int64_t>(C.ptr), ptr<int32_t>(C.col),
-            ptr<double>(C.val), ptr<double>(C.diag), ptr<double>(C.exc));
-    ++m->launches;
+// A wider coarse row (raw <= kBlockRaw), by the whole block.
+__device__ int coarse_row_block(const BuildArgs &a, int64_t noff, int64_t noff2, int I, int raw,
+                                unsigned long long *keys, double *vals, double *ex_sm) {
+    const HierView &v = a.v;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    __syncthreads();
+    if (wid == 0) {
+        const int cnt = v.gc[noff2 + I];
+        int32_t *own = v.own + noff + v.gs[noff2 + I];
+        sort_members(own, cnt);
+        double ex = 0.0;
+        int done = 0;
+        for (int k = 0; k < cnt; ++k) {
+            const int m = own[k];
+            const int len = v.rl[noff + m];
+            const int64_t e0 = v.rs[noff + m];
+            if (lane == 0) ex += v.ex[noff + m];
+            for (int e = lane; e < len; e += 32) {
+                const int J = a.agg[v.ecol[e0 + e]];
+                const double w = v.ew[e0 + e];
+                if (J < 0) ex += w;
+                keys[done + e] = (J < 0 || J == I) ? ~0ull
+                                                   : (static_cast<unsigned long long>(static_cast<unsigned>(J)) << 32) |
+                                                         static_cast<unsigned>(done + e);
+                vals[done + e] = w;
+            }
+            done += len;
+        }
+        ex = warp_sum(ex);
+        if (lane == 0) *ex_sm = ex;
+    }
+    const int P = pow2_at_least(raw);
+    for (int i = raw + threadIdx.x; i < P; i += blockDim.x) keys[i] = ~0ull;
+    __syncthreads();
+    bitonic(keys, P, threadIdx.x, blockDim.x, [] { __syncthreads(); });
+    int len = 0;
+    if (wid == 0) merge_row(v, noff2, I, keys, vals, raw, *ex_sm, len);
+    __syncthreads();
+    return len;  // valid in warp 0
 }
 
-// ---------------------------------------------------------------- V-cycle kernels
+// ---- the coarsest level's inverse
 //
-// The V-cycle runs in FP64 on a copy of each level's operator divided by a
-// fixed scale (the square of the largest |K|_phi, so that the entries sit near
-// 1).  An FP32 V-cycle costs less per application but loses the modes the
-// preconditioner exists for: a cluster held by a shift ~1e-10 of its diagonal
-// has a residual that cancels below FP32 rounding in b - L x, and the
-// conjugate gradients then need more than twice the iterations (measured on
-// the 1024^2 and 128^3 workloads), which costs more than FP64 saves.  The
-// kernels are templates on the precision all the same.
-
-template <class T> __global__ void k_scaled_copy(int64_t n, const double *in, T *out, double inv_scale) {
-    dep_enter();
-    GRID_STRIDE(i, n) out[i] = static_cast<T>(in[i] * inv_scale);
-}
-
-// Relaxation weight of row i: kOmega, or 1 for a row without off-diagonal
-// entries (then one sweep solves its equation exactly).
-__device__ __forceinline__ double row_weight(const int64_t *ptr, int64_t i) {
-    return ptr[i + 1] == ptr[i] ? 1.0 : kOmega;
-}
-
-// w_i = omega_i / (diag_i / scale): kOmega, or 1 for a row without
-// off-diagonal entries (one sweep then solves its equation exactly)
-template <class T>
-__global__ void k_scaled_inv(int64_t n, const int64_t *ptr, const double *diag, T *out, double inv_scale) {
-    dep_enter();
-    GRID_STRIDE(i, n) out[i] = static_cast<T>(row_weight(ptr, i) / (diag[i] * inv_scale));
-}
-
-// b = S res (S: +1 rows, -1 columns), in the V-cycle's precision
-template <class T> __global__ void k_flip_in(int64_t nc, const double *res, T *b, const CgState *st) {
-    dep_enter();
-    if (st && st->converged) return;
-    GRID_STRIDE(l, 2 * nc) b[l] = static_cast<T>(l < nc ? res[l] : -res[l]);
-}
-
-// z = S x / scale, in FP64
-template <class T> __global__ void k_flip_out(int64_t nc, const T *x, double inv_scale, double *z, const CgState *st) {
-    dep_enter();
-    if (st && st->converged) return;
-    GRID_STRIDE(l, 2 * nc) {
-        const double v = static_cast<double>(x[l]) * inv_scale;
-        z[l] = l < nc ? v : -v;
+// Elimination without subtractions: with weights w and excess ex the pivot is
+// ex_k + sum_{j > k} w_kj, and eliminating k adds w_ik w_kj / d_k to w_ij and
+// w_ik ex_k / d_k to ex_i -- sums of positive terms, so a shift of 1e-14 of the
+// weights keeps its relative precision.  L = (I - F) with F >= 0 gives
+// inv = sum_k M_k M_k^T / d_k, M = (I - F)^{-1}, again sums of positive terms.
+__device__ void dense_inverse(const HierView &v, int64_t noff, int n, double *sm) {
+    double(*w)[kDense + 1] = reinterpret_cast<double(*)[kDense + 1]>(sm);
+    double(*M)[kDense + 1] = w + kDense;
+    double *ex = &M[kDense][0], *d = ex + kDense;
+    const int i = threadIdx.x >> 5, j = threadIdx.x & 31;  // kBuildThreads = kDense^2
+    w[i][j] = 0.0;
+    M[i][j] = 0.0;
+    __syncthreads();
+    if (i < n) {
+        const int64_t e0 = v.rs[noff + i];
+        const int len = v.rl[noff + i];
+        for (int e = j; e < len; e += 32) w[i][v.ecol[e0 + e]] = v.ew[e0 + e];
+        if (j == 0) ex[i] = v.ex[noff + i];
     }
-}
-
-// z = S x / scale, with the per-block partial sums of z.res and z.rp that
-// the conjugate gradients need next (one pass instead of two)
-template <class T>
-__global__ void k_flip_out_dots(int64_t nc, const T *x, double inv_scale, double *z, const double *res,
-                                const double *rp, double *pa, double *pb, const CgState *st) {
-    dep_enter();
-    if (st && st->converged) return;
-    double a = 0.0, b = 0.0;
-    GRID_STRIDE(l, 2 * nc) {
-        const double v = static_cast<double>(x[l]) * inv_scale;
-        const double zl = l < nc ? v : -v;
-        z[l] = zl;
-        a += zl * res[l];
-        b += zl * rp[l];
-    }
-    a = block_sum(a);
-    b = block_sum(b);
-    if (threadIdx.x == 0) {
-        pa[blockIdx.x] = a;
-        pb[blockIdx.x] = b;
-    }
-}
-
-
-// The smoothers multiply by w_i = omega_i / diag_i, formed once per build
-// (k_scaled_inv): a division per node (and, in the pre-smoothing, per entry)
-// would cost far more, in FP64 above all.
-
-// x = w b
-template <class T> __global__ void k_jacobi0(int64_t n, const T *dinv, const T *b, T *x, const CgState *st) {
-    dep_enter();
-    if (st && st->converged) return;
-    GRID_STRIDE(i, n) x[i] = dinv[i] * b[i];
-}
-
-// x_out = x + w (b - L x)
-template <class T>
-__global__ void k_jacobi(int64_t n, const int64_t *ptr, const int32_t *col, const T *val, const T *diag,
-                         const T *dinv, const T *x, const T *b, T *x_out, const CgState *st) {
-    dep_enter();
-    if (st && st->converged) return;
-    GRID_STRIDE(i, n) {
-        const int64_t e0 = ptr[i], e1 = ptr[i + 1];
-        T s = diag[i] * x[i];
-        for (int64_t e = e0; e < e1; ++e) s += val[e] * x[col[e]];
-        x_out[i] = x[i] + dinv[i] * (b[i] - s);
-    }
-}
-
-// Pre-smoothing from zero and the residual in one pass: x = w b, r = b - L x
-// (a neighbour's x_j = w_j b_j is formed exactly as its owner forms it).
-template <class T>
-__global__ void k_presmooth_residual(int64_t n, const int64_t *ptr, const int32_t *col, const T *val, const T *diag,
-                                     const T *dinv, const T *b, T *x, T *r, const CgState *st) {
-    dep_enter();
-    if (st && st->converged) return;
-    GRID_STRIDE(i, n) {
-        const int64_t e0 = ptr[i], e1 = ptr[i + 1];
-        const T bi = b[i];
-        const T xi = dinv[i] * bi;
-        x[i] = xi;
-        T s = diag[i] * xi;
-        for (int64_t e = e0; e < e1; ++e) {
-            const int32_t j = col[e];
-            s += val[e] * (dinv[j] * b[j]);
+    __syncthreads();
+    for (int k = 0; k < n; ++k) {
+        if (i == 0) {
+            double s = j > k && j < n ? w[k][j] : 0.0;
+            s = warp_sum(s);
+            if (j == 0) d[k] = ex[k] + s;
         }
-        r[i] = bi - s;
-    }
-}
-
-// Prolongation and post-smoothing in one pass: with x' = x + xc[agg] (the
-// coarse correction; nothing for a node without a coarse counterpart),
-// x_out = x' + w (b - L x').  A neighbour's x'_j is formed as its owner forms it.
-template <class T>
-__global__ void k_prolong_smooth(int64_t n, const int64_t *ptr, const int32_t *col, const T *val, const T *diag,
-                                 const T *dinv, const int32_t *agg, const T *xc, const T *x, const T *b, T *x_out,
-                                 const CgState *st) {
-    dep_enter();
-    if (st && st->converged) return;
-    GRID_STRIDE(i, n) {
-        const int64_t e0 = ptr[i], e1 = ptr[i + 1];
-        const int32_t I = agg[i];
-        const T xi = I >= 0 ? x[i] + xc[I] : x[i];
-        T s = diag[i] * xi;
-        for (int64_t e = e0; e < e1; ++e) {
-            const int32_t j = col[e];
-            const int32_t J = agg[j];  // < 0: a neighbour that left the hierarchy
-            s += val[e] * (J >= 0 ? x[j] + xc[J] : x[j]);
-        }
-        x_out[i] = xi + dinv[i] * (b[i] - s);
-    }
-}
-
-template <class T>
-__global__ void k_restrict(int64_t nco, const int64_t *mptr, const int32_t *mlist, const T *r, T *bc,
-                           const CgState *st) {
-    dep_enter();
-    if (st && st->converged) return;
-    GRID_STRIDE(I, nco) {
-        T s = 0;
-        for (int64_t k = mptr[I]; k < mptr[I + 1]; ++k) s += r[mlist[k]];
-        bc[I] = s;
-    }
-}
-
-template <class T> __global__ void k_prolong(int64_t n, const int32_t *agg, const T *xc, T *x, const CgState *st) {
-    dep_enter();
-    if (st && st->converged) return;
-    GRID_STRIDE(i, n) {
-        const int32_t I = agg[i];
-        if (I >= 0) x[i] += xc[I];
-    }
-}
-
-// The levels small enough for one block (n <= kOneBlock each), from the
-// first of them down to the coarsest and back, in one launch: the same
-// arithmetic per node as the per-level kernels above (pre-smoothing fused with
-// the residual, restriction, kCoarsestSweeps sweeps on the coarsest level,
-// prolongation fused with post-smoothing), with a block barrier between the
-// passes instead of a kernel boundary.  On a fine mesh the hierarchy has a
-// handful of such levels, each of which otherwise costs three launches of a
-// few microseconds that do almost no work.
-template <class T> struct SmallLevel {
-    int64_t n;
-    const int64_t *ptr;
-    const int32_t *col;
-    const T *val, *diag, *dinv;
-    const int32_t *agg;    // node -> aggregate of the next level (levels above the coarsest)
-    const int64_t *mptr;   // members (nodes of the previous level) of each node of this level
-    const int32_t *mlist;
-    T *x, *x2, *b, *r;
-};
-
-template <class T>
-__global__ void __launch_bounds__(1024) k_small_cycle(const SmallLevel<T> *Ls, int nl, const CgState *st) {
-    dep_enter();
-    if (st && st->converged) return;
-    for (int l = 0; l + 1 < nl; ++l) {  // down
-        const SmallLevel<T> &L = Ls[l];
-        for (int64_t i = threadIdx.x; i < L.n; i += blockDim.x) {
-            const int64_t e0 = L.ptr[i], e1 = L.ptr[i + 1];
-            const T bi = L.b[i];
-            const T xi = L.dinv[i] * bi;
-            L.x[i] = xi;
-            T sum = L.diag[i] * xi;
-            for (int64_t e = e0; e < e1; ++e) {
-                const int32_t j = L.col[e];
-                sum += L.val[e] * (L.dinv[j] * L.b[j]);
+        __syncthreads();
+        const double dk = d[k], wik = w[i][k], wkj = w[k][j], exk = ex[k];
+        __syncthreads();
+        if (i > k && i < n) {
+            const double f = wik / dk;
+            if (j > k && j < n && j != i) w[i][j] += f * wkj;
+            if (j == k) {
+                ex[i] += f * exk;
+                w[i][k] = f;  // F below the diagonal
             }
-            L.r[i] = bi - sum;
-        }
-        __syncthreads();
-        const SmallLevel<T> &C = Ls[l + 1];
-        for (int64_t I = threadIdx.x; I < C.n; I += blockDim.x) {
-            T sum = 0;
-            for (int64_t k = C.mptr[I]; k < C.mptr[I + 1]; ++k) sum += L.r[C.mlist[k]];
-            C.b[I] = sum;
         }
         __syncthreads();
     }
-    {  // coarsest
-        const SmallLevel<T> &L = Ls[nl - 1];
-        for (int64_t i = threadIdx.x; i < L.n; i += blockDim.x)
-            L.x[i] = L.dinv[i] * L.b[i];
+    if (i == 0)  // column j of M, by lane j
+        for (int r = 0; r < n; ++r) {
+            double s = r == j ? 1.0 : 0.0;
+            for (int k = j; k < r; ++k) s += w[r][k] * M[k][j];
+            if (j < n) M[r][j] = r >= j ? s : 0.0;
+        }
+    __syncthreads();
+    if (i < n && j < n) {
+        double s = 0.0;
+        for (int k = max(i, j); k < n; ++k) s += M[k][i] * M[k][j] / d[k];
+        v.H->inv[i * kDense + j] = s;
+    }
+}
+
+// ---- the build
+
+template <int LPR> __global__ void __launch_bounds__(kBuildThreads, 1) k_amg_build(BuildArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    unsigned long long *keys = reinterpret_cast<unsigned long long *>(smem);
+    double *vals = reinterpret_cast<double *>(smem + sizeof(unsigned long long) * kBlockRaw);
+    __shared__ int pre[2][kMaxCtas + 1];
+    __shared__ int tmp[33];
+    __shared__ int s_base[2];
+    __shared__ unsigned long long s_ebase;
+    __shared__ double s_ex;
+    __shared__ int s_wide[kBuildThreads];
+    const HierView &v = a.v;
+    Hier *H = v.H;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    int nb = gridDim.x, b = blockIdx.x;
+    GridBar bar(&H->bar[0], &H->err, gridDim.x);
+
+    int n = a.n0;
+    int64_t noff = 0, nnz = a.e0;
+    int block_nodes = 0;  // nodes of the levels built by block 0 alone
+    {
+        const int ch = (n + nb - 1) / nb;
+        level0_values<LPR>(a, min(n, b * ch), min(n, (b + 1) * ch));
+        if (b == 0 && tid == 0) H->ecur = static_cast<unsigned long long>(a.e0);
+    }
+    if (!bar.sync()) return;
+    int l = 0, sweeps = kLargeSweeps;
+    for (;; ++l) {
+        if (nb > 1 && nnz <= kBlockEntries && n <= kBlockNodes) {
+            if (b != 0) return;  // block 0 finishes the hierarchy alone
+            nb = 1;
+            bar.nb = 1;
+        }
+        const int grid = nb > 1 ? 1 : 0;
+        if (b == 0 && tid == 0) {
+            H->L[l].noff = noff;
+            H->L[l].n = n;
+            H->L[l].nmem = 0;
+            H->L[l].nnz = nnz;
+            H->L[l].grid = l == 0 ? 1 : grid;
+        }
+        if (!grid && l > 0) block_nodes += n;
+        if (n <= kDense || l + 1 == kMaxLevels) break;
+        const int ch = (n + nb - 1) / nb;
+        const int i0 = min(n, b * ch), i1 = min(n, i0 + ch);
+        rank_round<LPR>(a, noff, n, i0, i1, 0, nullptr, a.best0);
+        if (!bar.sync()) return;
+        int32_t *bp = a.best0, *bc = a.best1;
+        for (int r = 1; r < kHandshakes; ++r) {
+            rank_round<LPR>(a, noff, n, i0, i1, r, bp, bc);
+            if (!bar.sync()) return;
+            int32_t *t = bp;
+            bp = bc;
+            bc = t;
+        }
+        // leaders and, per block, their number and that of the leaving nodes
+        int run = 0, lrun = 0;
+        for (int base = i0; base < i1; base += kBuildThreads) {
+            const int i = base + tid;
+            int lead = -2, flags = 0;
+            if (i < i1) {
+                lead = leader_of(a, bp, i);
+                flags = lead == i ? 1 : (lead == -1 ? 1 << 16 : 0);
+            }
+            int tot;
+            const int at = block_scan(flags, tmp, tot);
+            if (i < i1) {
+                a.lead[i] = lead;
+                a.pos[i] = lead == i ? run + (at & 0xffff) : lrun + (at >> 16);
+            }
+            run += tot & 0xffff;
+            lrun += tot >> 16;
+        }
+        if (tid == 0) {
+            H->ctasum[0][b] = run;
+            H->ctasum[1][b] = lrun;
+        }
+        if (!bar.sync()) return;
+        // their prefixes over the blocks
+        if (wid < 2) {
+            int carry = 0;
+            for (int base = 0; base < nb; base += 32) {
+                const int q = base + lane;
+                const int x = q < nb ? *reinterpret_cast<volatile int *>(&H->ctasum[wid][q]) : 0;
+                int incl = x;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += t;
+                }
+                if (q < nb) pre[wid][q] = carry + incl - x;
+                carry += __shfl_sync(0xffffffffu, incl, 31);
+            }
+            if (lane == 0) pre[wid][nb] = carry;
+        }
         __syncthreads();
-        for (int k = 0; k < kCoarsestSweeps; ++k) {
-            const T *xi = (k & 1) ? L.x2 : L.x;
-            T *xo = (k & 1) ? L.x : L.x2;
-            for (int64_t i = threadIdx.x; i < L.n; i += blockDim.x) {
-                T sum = L.diag[i] * xi[i];
-                for (int64_t e = L.ptr[i]; e < L.ptr[i + 1]; ++e) sum += L.val[e] * xi[L.col[e]];
-                xo[i] = xi[i] + L.dinv[i] * (L.b[i] - sum);
+        const int nco = pre[0][nb], nlv = pre[1][nb], active = n - nlv;
+        const int64_t noff2 = noff + n;
+        if (active == 0) sweeps = kDominantSweeps;
+        if (active == 0 || nco < 1 || nco >= active * kStall || noff2 + nco > v.capn ||
+            (!grid && l > 0 && block_nodes + nco > kBlockTotalNodes))
+            break;
+        // aggregates: members are counted and their raw entries added up
+        for (int i = i0 + tid; i < i1; i += kBuildThreads) {
+            const int L = a.lead[i];
+            int I = -1;
+            if (L < 0) {
+                v.own[noff + active + pre[1][b] + a.pos[i]] = i;
+            } else {
+                I = pre[0][L / ch] + a.pos[L];
+                atomicAdd(&a.cnt[I], 1);
+                atomicAdd(&a.cap[I], v.rl[noff + i]);
+            }
+            a.agg[i] = I;
+        }
+        if (!bar.sync()) return;
+        // per block of coarse nodes: where their members and entries go
+        const int ch2 = (nco + nb - 1) / nb;
+        const int g0 = min(nco, b * ch2), g1 = min(nco, g0 + ch2);
+        int mtot = 0;
+        int64_t etot = 0;
+        for (int pass = 0; pass < 2; ++pass) {  // totals first, then the places
+            int m = 0;
+            int64_t e = 0;
+            for (int base = g0; base < g1; base += kBuildThreads) {
+                const int I = base + tid;
+                const int c = I < g1 ? a.cnt[I] : 0, cp = I < g1 ? a.cap[I] : 0;
+                int ct, et;
+                const int ca = block_scan(c, tmp, ct);
+                const int ea = block_scan(cp, tmp, et);
+                if (pass == 1 && I < g1) {
+                    v.gs[noff2 + I] = s_base[0] + m + ca;
+                    v.gc[noff2 + I] = c;
+                    v.rs[noff2 + I] = static_cast<int64_t>(s_ebase) + e + ea;
+                    a.cnt[I] = 0;  // from here on the members placed so far
+                }
+                m += ct;
+                e += et;
+            }
+            if (pass == 0) {
+                mtot = m;
+                etot = e;
+                __syncthreads();
+                if (tid == 0) {
+                    s_base[0] = static_cast<int>(atomicAdd(&H->mcur[l], static_cast<unsigned>(mtot)));
+                    s_ebase = atomicAdd(&H->ecur, static_cast<unsigned long long>(etot));
+                    if (s_ebase + etot > static_cast<unsigned long long>(v.cape)) atomicExch(&H->overflow, 1);
+                    Seg s;
+                    s.m0 = s_base[0];
+                    s.mlen = mtot;
+                    s.l0 = active + pre[1][b];
+                    s.llen = pre[1][b + 1] - pre[1][b];
+                    s.g0 = g0;
+                    s.glen = g1 - g0;
+                    v.seg[l * kMaxCtas + b] = s;
+                }
+                __syncthreads();
+            }
+        }
+        if (!bar.sync()) return;
+        if (*reinterpret_cast<volatile int *>(&H->overflow)) break;  // the finer level stays the coarsest
+        for (int i = i0 + tid; i < i1; i += kBuildThreads) {
+            const int I = a.agg[i];
+            if (I >= 0) v.own[noff + v.gs[noff2 + I] + atomicAdd(&a.cnt[I], 1)] = i;
+        }
+        if (!bar.sync()) return;
+        // coarse rows: one warp each, the wide ones by the whole block
+        int got = 0, nwide = 0;
+        for (int base = g0; base < g1; base += kBuildThreads) {
+            const int cnt_here = min(kBuildThreads, g1 - base);
+            __syncthreads();
+            if (tid == 0) s_base[1] = 0;
+            __syncthreads();
+            for (int q = wid; q < cnt_here; q += kBuildThreads / 32) {
+                const int I = base + q;
+                const int raw = a.cap[I];
+                if (raw <= kWarpRaw)
+                    got += coarse_row_warp(a, noff, noff2, I, raw, keys + wid * kWarpRaw, vals + wid * kWarpRaw);
+                else if (lane == 0)
+                    s_wide[atomicAdd(&s_base[1], 1)] = I;
             }
             __syncthreads();
-        }
-    }
-    for (int l = nl - 2; l >= 0; --l) {  // up
-        const SmallLevel<T> &L = Ls[l];
-        const T *xc = l + 1 == nl - 1 ? Ls[l + 1].x : Ls[l + 1].x2;
-        for (int64_t i = threadIdx.x; i < L.n; i += blockDim.x) {
-            const int64_t e0 = L.ptr[i], e1 = L.ptr[i + 1];
-            const int32_t I = L.agg[i];
-            const T xi = I >= 0 ? L.x[i] + xc[I] : L.x[i];
-            T sum = L.diag[i] * xi;
-            for (int64_t e = e0; e < e1; ++e) {
-                const int32_t j = L.col[e];
-                const int32_t J = L.agg[j];
-                sum += L.val[e] * (J >= 0 ? L.x[j] + xc[J] : L.x[j]);
+            nwide = s_base[1];
+            for (int q = 0; q < nwide; ++q) {
+                const int I = s_wide[q];
+                const int raw = a.cap[I];
+                if (raw > kBlockRaw) {  // block-uniform
+                    if (tid == 0) {
+                        v.rl[noff2 + I] = 0;
+                        v.dg[noff2 + I] = v.ex[noff2 + I] = v.om[noff2 + I] = 1.0;
+                        atomicExch(&H->overflow, 1);
+                    }
+                    continue;
+                }
+                const int len = coarse_row_block(a, noff, noff2, I, raw, keys, vals, &s_ex);
+                if (wid == 0) got += len;
             }
-            L.x2[i] = xi + L.dinv[i] * (L.b[i] - sum);
         }
-        __syncthreads();
+        if (lane == 0 && got) atomicAdd(&H->nnzacc[l + 1], static_cast<unsigned long long>(got));
+        if (!bar.sync()) return;
+        if (*reinterpret_cast<volatile int *>(&H->overflow)) break;
+        if (b == 0 && tid == 0) H->L[l].nmem = active;
+        nnz = static_cast<int64_t>(*reinterpret_cast<volatile unsigned long long *>(&H->nnzacc[l + 1]));
+        n = nco;
+        noff = noff2;
+    }
+    // level l is the coarsest
+    if (b != 0) return;
+    const int dense = n <= kDense ? 1 : 0;
+    if (dense) dense_inverse(v, noff, n, reinterpret_cast<double *>(smem));
+    if (tid == 0) {
+        H->nlev = l + 1;
+        H->dense = dense;
+        H->sweeps = sweeps;
+        if (l > 0 && nb > 1) H->L[l].grid = 1;
     }
 }
 
-// ---------------------------------------------------------------- host side
+// ---- host side
 
-void amg_release(Amg &amg) {
-    for (AmgLevel &L : amg.levels) {
-        Buf *all[] = {&L.ptr, &L.col, &L.val, &L.diag, &L.exc, &L.agg, &L.mptr, &L.mlist, &L.x, &L.x2, &L.b, &L.r,
-                      &L.dval, &L.ddiag, &L.ddinv};
-        for (Buf *b : all) release(*b);
-    }
-    amg.levels.clear();
-    release(amg.tmp);
-    release(amg.small_d);
+int solve_grid(int64_t e0) {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (sms < 1) sms = 1;
+    if (sms > kMaxCtas) sms = kMaxCtas;
+    // one block per ~800 entries: the FP64 pipe takes about 1.7 products per
+    // clock and SM, so a pass then costs ~500 clocks against ~2 300 for the barrier
+    // after it; up to one block's worth of work needs no grid barrier at all
+    int64_t g = e0 / 800;
+    if (e0 <= 6000) g = 1;
+    return static_cast<int>(g < 1 ? 1 : (g > sms ? sms : g));
 }
 
-static bool level_vectors(bchar_mesh_t m, AmgLevel &L) {
-    // x holds n + 1 entries: it doubles as the int64 scan output while coarsening
-    return ensure(m, L.x, sizeof(double) * (L.n + 1)) && ensure(m, L.x2, sizeof(double) * L.n) &&
-           ensure(m, L.b, sizeof(double) * L.n) && ensure(m, L.r, sizeof(double) * L.n);
+template <typename... P, typename... A>
+static void launch_cooperative(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
-static bool amg_scaled_copies(bchar_mesh_t m, Amg &amg);
-
-// The one-block levels: every level from the first with at most kOneBlock
-// nodes down to the coarsest (levels shrink, so they are a suffix), when the
-// coarsest is one of them.  Their descriptors go to the device once per build.
-static bool small_descriptors(bchar_mesh_t m, Amg &amg) {
-    int from = amg.nlev;
-    while (from > 0 && amg.levels[from - 1].n <= kOneBlock) --from;
-    amg.small_from = from;
-    const int nl = amg.nlev - from;
-    if (nl == 0) return true;
-    std::vector<SmallLevel<double>> hd(nl);
-    for (int k = 0; k < nl; ++k) {
-        AmgLevel &L = amg.levels[from + k];
-        const bool last = from + k == amg.nlev - 1;
-        const bool first = k == 0;
-        hd[k] = {L.n, ptr<int64_t>(L.ptr), ptr<int32_t>(L.col), ptr<double>(L.dval), ptr<double>(L.ddiag), ptr<double>(L.ddinv),
-                 last ? nullptr : ptr<int32_t>(L.agg), first ? nullptr : ptr<int64_t>(L.mptr),
-                 first ? nullptr : ptr<int32_t>(L.mlist), ptr<double>(L.x), ptr<double>(L.x2), ptr<double>(L.b),
-                 ptr<double>(L.r)};
-    }
-    if (!ensure(m, amg.small_d, sizeof(SmallLevel<double>) * nl)) return false;
-    // a pageable source: the copy has read it when the call returns
-    cudaMemcpyAsync(amg.small_d.p, hd.data(), sizeof(SmallLevel<double>) * nl, cudaMemcpyHostToDevice, m->stream);
-    return true;
+HierView hier_view(bchar_mesh_t m) {
+    Amg &A = m->amg;
+    HierView v{};
+    v.H = ptr<Hier>(A.hier);
+    v.seg = ptr<Seg>(A.seg);
+    v.capn = A.capn;
+    v.cape = A.cape;
+    v.rs = ptr<int64_t>(A.rs);
+    v.rl = ptr<int32_t>(A.rl);
+    v.dg = ptr<double>(A.dg);
+    v.ex = ptr<double>(A.ex);
+    v.om = ptr<double>(A.om);
+    v.x = ptr<double>(A.x);
+    v.b = ptr<double>(A.b);
+    v.own = ptr<int32_t>(A.own);
+    v.gs = ptr<int32_t>(A.gs);
+    v.gc = ptr<int32_t>(A.gc);
+    v.ecol = ptr<int32_t>(A.ecol);
+    v.ew = ptr<double>(A.ew);
+    return v;
 }
 
-bool amg_build(bchar_mesh_t m, Amg &amg) {
-    cudaStream_t s = m->stream;
-    const int64_t nc = m->nc, nnz = m->nnz;
-    if (amg.levels.empty()) amg.levels.resize(1);
-    amg.nlev = 1;
-    amg.large_sweeps = kLargeCoarsestSweeps;
-    AmgLevel &L0 = amg.levels[0];
-    L0.n = 2 * nc;
-    L0.nnz = 2 * nnz;
-    if (!ensure(m, L0.ptr, sizeof(int64_t) * (L0.n + 1)) || !ensure(m, L0.col, sizeof(int32_t) * L0.nnz) ||
-        !ensure(m, L0.val, sizeof(double) * L0.nnz) || !level_vectors(m, L0))
-        return false;
-    L0.diag_ext = ptr<double>(m->diag);
-    L0.exc_ext = ptr<double>(m->qexc);
-    launch_dep(k_level0_ptr, blocks_for(L0.n + 1), kThreads, s, nc, nnz, ptr<int64_t>(m->row_ptr), ptr<int64_t>(m->col_ptr),
-                                                           ptr<int64_t>(L0.ptr));
-    launch_dep(k_level0_fill, blocks_for(L0.n), kThreads, s, nc, ptr<int64_t>(m->row_ptr), ptr<int32_t>(m->col),
-                                                        ptr<int64_t>(m->col_ptr), ptr<int32_t>(m->csc_row),
-                                                        ptr<double>(m->a2), ptr<double>(m->a2c),
-                                                        ptr<int64_t>(L0.ptr), ptr<int32_t>(L0.col),
-                                                        ptr<double>(L0.val));
-    m->launches += 2;
-    while (amg.nlev < kMaxLevels) {
-        AmgLevel &F = amg.levels[amg.nlev - 1];
-        if (F.n <= kCoarsest) break;
-        const double *fexc = F.exc_ext ? F.exc_ext : ptr<double>(F.exc);
-        const double *fdg = F.diag_ext ? F.diag_ext : ptr<double>(F.diag);
-        if (!ensure(m, amg.tmp, sizeof(int32_t) * 6 * F.n + 64) || !ensure(m, F.agg, sizeof(int32_t) * F.n))
-            return false;
-        int32_t *best = ptr<int32_t>(amg.tmp);
-        int32_t *partner = best + F.n;
-        int32_t *att = partner + F.n;     // attachment targets
-        int32_t *want = att + F.n;
-        int32_t *leader = want + F.n;
-        int32_t *flag = leader + F.n;     // leader flags, later member counts / fill / row counts
-        int *overflow = reinterpret_cast<int *>(flag + F.n);
-        int *isolated = overflow + 1;
-        const int bl = blocks_for(F.n);
-        cudaMemsetAsync(partner, 0xff, sizeof(int32_t) * F.n, s);
-        cudaMemsetAsync(overflow, 0, 2 * sizeof(int), s);
-        // the want array holds the leave flags until k_want overwrites them
-        launch_dep(k_leaving, bl, kThreads, s, F.n, ptr<int64_t>(F.ptr), ptr<int32_t>(F.col), ptr<double>(F.val), fdg,
-                   want);
-        ++m->launches;
-        for (int round = 0; round < kHandshakes; ++round) {
-            launch_dep(k_heaviest, bl, kThreads, s, F.n, ptr<int64_t>(F.ptr), ptr<int32_t>(F.col), ptr<double>(F.val),
-                                               fdg, want, partner, round > 0, best);
-            launch_dep(k_handshake, bl, kThreads, s, F.n, best, partner);
-            m->launches += 2;
-        }
-        launch_dep(k_attach_target, bl, kThreads, s, F.n, ptr<int64_t>(F.ptr), ptr<int32_t>(F.col), ptr<double>(F.val), fdg,
-                                                want, att);
-        launch_dep(k_leaders1, bl, kThreads, s, F.n, want, partner, att, leader, isolated);
-        launch_dep(k_want, bl, kThreads, s, F.n, att, leader, want);
-        launch_dep(k_leaders2, bl, kThreads, s, F.n, want, leader, flag);
-        m->launches += 4;
-        // leader positions: scan of the leader flags (int32 -> int64), reuse the
-        // per-level x buffer as int64 scratch (it holds n + 1 entries)
-        int64_t *pos = reinterpret_cast<int64_t *>(ptr<double>(F.x));
-        scan_i32_to_i64(m, flag, pos, F.n);
-        // The coarse level is laid out for U = F.n coarse nodes, a bound on their
-        // number nco, so that its members and row counts are formed before nco is
-        // read back: nodes nco..U-1 have no members and empty rows.  One read-back
-        // per level then returns nco, the isolated nodes and the coarse entries.
-        if (static_cast<int>(amg.levels.size()) <= amg.nlev) amg.levels.resize(amg.nlev + 1);
-        AmgLevel &Fr = amg.levels[amg.nlev - 1];  // re-fetch after resize
-        AmgLevel &C = amg.levels[amg.nlev];
-        const int64_t U = Fr.n;
-        C.n = U;
-        C.diag_ext = nullptr;
-        C.exc_ext = nullptr;
-        if (!ensure(m, C.mptr, sizeof(int64_t) * (U + 1)) || !ensure(m, C.mlist, sizeof(int32_t) * Fr.n) ||
-            !ensure(m, C.ptr, sizeof(int64_t) * (U + 1)) || !ensure(m, C.diag, sizeof(double) * U) ||
-            !ensure(m, C.exc, sizeof(double) * U) || !level_vectors(m, C))
-            return false;
-        // aggregates: map, member counts -> pointers, members sorted by node
-        cudaMemsetAsync(flag, 0, sizeof(int32_t) * U, s);
-        launch_dep(k_aggregates, bl, kThreads, s, Fr.n, leader, pos, ptr<int32_t>(Fr.agg), flag);
-        scan_i32_to_i64(m, flag, ptr<int64_t>(C.mptr), U);
-        cudaMemsetAsync(flag, 0, sizeof(int32_t) * U, s);
-        launch_dep(k_members_fill, bl, kThreads, s, Fr.n, ptr<int32_t>(Fr.agg), ptr<int64_t>(C.mptr), flag,
-                                               ptr<int32_t>(C.mlist));
-        launch_dep(k_members_sort, blocks_for(U), kThreads, s, U, ptr<int64_t>(C.mptr), ptr<int32_t>(C.mlist));
-        m->launches += 3;
-        int32_t *rowcnt = flag;
-        coarse_count(m, Fr, C, U, fexc, rowcnt, overflow);
-        scan_i32_to_i64(m, rowcnt, ptr<int64_t>(C.ptr), U);
-        int64_t nco = 0, cnnz = 0;
-        int niso = 0, ovf = 0;
-        cudaMemcpyAsync(&nco, pos + Fr.n, sizeof nco, cudaMemcpyDeviceToHost, s);
-        cudaMemcpyAsync(&niso, isolated, sizeof niso, cudaMemcpyDeviceToHost, s);
-        cudaMemcpyAsync(&cnnz, ptr<int64_t>(C.ptr) + U, sizeof cnnz, cudaMemcpyDeviceToHost, s);
-        cudaMemcpyAsync(&ovf, overflow, sizeof ovf, cudaMemcpyDeviceToHost, s);
-        if (cudaStreamSynchronize(s) != cudaSuccess) return false;
-        m->launches += 1;
-        const int64_t active = Fr.n - niso;  // nodes that would have a coarse counterpart
-        // a coarsest level whose nodes have all left the hierarchy is diagonally
-        // dominant (ratio <= kDominant): a few sweeps reduce its error enough
-        amg.large_sweeps = active == 0 ? kDominantSweeps : kLargeCoarsestSweeps;
-        if (active <= kCoarsest || nco >= active * kStall || nco < 1) break;  // Fr is the coarsest level
-        if (ovf) break;  // a coarse row would be too wide: stop at the finer level
-        C.n = nco;
-        C.nnz = cnnz;
-        if (!ensure(m, C.col, sizeof(int32_t) * (cnnz > 0 ? cnnz : 1)) ||
-            !ensure(m, C.val, sizeof(double) * (cnnz > 0 ? cnnz : 1)))
-            return false;
-        coarse_fill(m, Fr, C, nco, fexc);
-        ++amg.nlev;
+void amg_build(bchar_mesh_t m) {
+    Amg &A = m->amg;
+    BuildArgs a{};
+    a.v = hier_view(m);
+    a.n0 = static_cast<int>(A.n0);
+    a.e0 = A.e0;
+    a.schur = A.schur ? 1 : 0;
+    a.nc = m->nc;
+    a.col_ptr = ptr<int64_t>(m->col_ptr);
+    a.csc_row = ptr<int32_t>(m->csc_row);
+    a.a2 = ptr<double>(m->a2);
+    a.a2c = ptr<double>(m->a2c);
+    a.diag = ptr<double>(m->diag);
+    a.exc = ptr<double>(m->qexc);
+    a.g = ptr<double>(A.g);
+    a.t = ptr<double>(A.t);
+    a.cs = ptr<uint32_t>(A.cs);
+    a.pair = ptr<int2>(A.pair);
+    int32_t *s = ptr<int32_t>(A.scratch);
+    int32_t **dst[] = {&a.best0, &a.best1, &a.partner, &a.att, &a.lead, &a.pos, &a.agg, &a.cnt, &a.cap};
+    for (int32_t **d : dst) {
+        *d = s;
+        s += A.n0;
     }
-    return amg_scaled_copies(m, amg);
-}
-
-// The FP64 copy of every level's operator divided by a fixed scale (the
-// square of the largest |K|_phi), and the smoother weights.
-static bool amg_scaled_copies(bchar_mesh_t m, Amg &amg) {
-    cudaStream_t s = m->stream;
-    amg.scale = m->max_volphi * m->max_volphi;
-    const double inv = 1.0 / amg.scale;
-    for (int l = 0; l < amg.nlev; ++l) {
-        AmgLevel &L = amg.levels[l];
-        const int64_t nnzl = L.nnz > 0 ? L.nnz : 1;
-        if (!ensure(m, L.dval, sizeof(double) * nnzl) || !ensure(m, L.ddiag, sizeof(double) * L.n) ||
-            !ensure(m, L.ddinv, sizeof(double) * L.n))
-            return false;
-        const double *dg = L.diag_ext ? L.diag_ext : ptr<double>(L.diag);
-        if (L.nnz > 0) {
-            launch_dep(k_scaled_copy<double>, blocks_for(L.nnz), kThreads, s, L.nnz, ptr<double>(L.val),
-                       ptr<double>(L.dval), inv);
-            ++m->launches;
-        }
-        launch_dep(k_scaled_copy<double>, blocks_for(L.n), kThreads, s, L.n, dg, ptr<double>(L.ddiag), inv);
-        launch_dep(k_scaled_inv<double>, blocks_for(L.n), kThreads, s, L.n, ptr<int64_t>(L.ptr), dg,
-                   ptr<double>(L.ddinv), inv);
-        m->launches += 2;
+    cudaMemsetAsync(A.hier.p, 0, offsetof(Hier, L), m->stream);
+    static bool attrs = false;  // the shared-memory opt-in (harmless to repeat)
+    if (!attrs) {
+        cudaFuncSetAttribute(k_amg_build<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBuildSmem));
+        cudaFuncSetAttribute(k_amg_build<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBuildSmem));
+        attrs = true;
     }
-    return small_descriptors(m, amg);
-}
-
-// Buffers of one level in the V-cycle's precision.
-template <class T> struct LevelBufs;
-template <> struct LevelBufs<double> {
-    static double *val(AmgLevel &L) { return ptr<double>(L.dval); }
-    static double *diag(AmgLevel &L) { return ptr<double>(L.ddiag); }
-    static double *dinv(AmgLevel &L) { return ptr<double>(L.ddinv); }
-    static double *x(AmgLevel &L) { return ptr<double>(L.x); }
-    static double *x2(AmgLevel &L) { return ptr<double>(L.x2); }
-    static double *b(AmgLevel &L) { return ptr<double>(L.b); }
-    static double *r(AmgLevel &L) { return ptr<double>(L.r); }
-    static void *small(Amg &a) { return a.small_d.p; }
-};
-
-// z = S V(S res) / scale: one V-cycle of the sign-flipped operator in precision T.
-template <class T>
-static void vcycle(bchar_mesh_t m, Amg &amg, const double *res, double *z, const CgState *st, bool b_ready,
-                   const double *rp, double *pa, double *pb) {
-    using B = LevelBufs<T>;
-    cudaStream_t s = m->stream;
-    const int64_t nc = m->nc;
-    AmgLevel &L0 = amg.levels[0];
-    if (!b_ready) {
-        launch_dep(k_flip_in<T>, blocks_for(L0.n), kThreads, s, nc, res, B::b(L0), st);
-        ++m->launches;
-    }
-    const int big = amg.small_from < amg.nlev ? amg.small_from : amg.nlev - 1;  // levels cycled kernel by kernel
-    for (int l = 0; l < big; ++l) {  // down: pre-smooth from zero, residual, restrict
-        AmgLevel &L = amg.levels[l];
-        AmgLevel &C = amg.levels[l + 1];
-        const int bl = blocks_for(L.n);
-        launch_dep(k_presmooth_residual<T>, bl, kThreads, s, L.n, ptr<int64_t>(L.ptr), ptr<int32_t>(L.col), B::val(L),
-                                                        B::diag(L), B::dinv(L), B::b(L), B::x(L), B::r(L), st);
-        launch_dep(k_restrict<T>, blocks_for(C.n), kThreads, s, C.n, ptr<int64_t>(C.mptr), ptr<int32_t>(C.mlist), B::r(L),
-                                                           B::b(C), st);
-        m->launches += 2;
-    }
-    if (amg.small_from < amg.nlev) {  // the one-block levels down to the coarsest and back, one launch
-        launch_dep(k_small_cycle<T>, 1, 1024, s, static_cast<const SmallLevel<T> *>(B::small(amg)),
-                                             amg.nlev - amg.small_from, st);
-        ++m->launches;
-    } else {  // a coarsest level too large for one block: Jacobi sweeps from zero (even count: the result is in x)
-        AmgLevel &L = amg.levels[amg.nlev - 1];
-        const int bl = blocks_for(L.n);
-        launch_dep(k_jacobi0<T>, bl, kThreads, s, L.n, B::dinv(L), B::b(L), B::x(L), st);
-        for (int k = 0; k < amg.large_sweeps; ++k)
-            launch_dep(k_jacobi<T>, bl, kThreads, s, L.n, ptr<int64_t>(L.ptr), ptr<int32_t>(L.col), B::val(L),
-                                                B::diag(L), B::dinv(L), k & 1 ? B::x2(L) : B::x(L), B::b(L),
-                                                k & 1 ? B::x(L) : B::x2(L), st);
-        m->launches += 1 + amg.large_sweeps;
-    }
-    // up: prolong into x, post-smooth into x2 (the next finer level reads x2; the
-    // coarsest level, and a one-block cycle of a single level, leave theirs in x)
-    for (int l = big - 1; l >= 0; --l) {
-        AmgLevel &L = amg.levels[l];
-        AmgLevel &C = amg.levels[l + 1];
-        const T *xc = l + 1 == amg.nlev - 1 ? B::x(C) : B::x2(C);
-        if (L.n < kFuseBelow) {  // launch-bound levels: one kernel
-            launch_dep(k_prolong_smooth<T>, blocks_for(L.n), kThreads, s, L.n, ptr<int64_t>(L.ptr), ptr<int32_t>(L.col),
-                                                                     B::val(L), B::diag(L), B::dinv(L), ptr<int32_t>(L.agg), xc,
-                                                                     B::x(L), B::b(L), B::x2(L), st);
-            ++m->launches;
-        } else {  // large levels: the sweep's neighbours read one array instead of three
-            launch_dep(k_prolong<T>, blocks_for(L.n), kThreads, s, L.n, ptr<int32_t>(L.agg), xc, B::x(L), st);
-            launch_dep(k_jacobi<T>, blocks_for(L.n), kThreads, s, L.n, ptr<int64_t>(L.ptr), ptr<int32_t>(L.col), B::val(L),
-                                                             B::diag(L), B::dinv(L), B::x(L), B::b(L), B::x2(L), st);
-            m->launches += 2;
-        }
-    }
-    const T *x0 = amg.nlev > 1 ? B::x2(L0) : B::x(L0);
-    if (pa)
-        launch_dep(k_flip_out_dots<T>, kRedBlocks, kThreads, s, nc, x0, 1.0 / amg.scale, z, res, rp, pa, pb, st);
+    const int grid = solve_grid(A.e0);
+    if (A.e0 <= 10 * A.n0)
+        launch_cooperative(k_amg_build<4>, grid, kBuildThreads, kBuildSmem, m->stream, a);
     else
-        launch_dep(k_flip_out<T>, blocks_for(L0.n), kThreads, s, nc, x0, 1.0 / amg.scale, z, st);
+        launch_cooperative(k_amg_build<16>, grid, kBuildThreads, kBuildSmem, m->stream, a);
     ++m->launches;
 }
 
-// One damped-Jacobi sweep on the finest level (for timing; on a large finest
-// level this is the V-cycle's post-smoothing kernel).
-void amg_smooth_once(bchar_mesh_t m, Amg &amg) {
-    AmgLevel &L = amg.levels[0];
-    k_jacobi<double><<<blocks_for(L.n), kThreads, 0, m->stream>>>(L.n, ptr<int64_t>(L.ptr), ptr<int32_t>(L.col),
-                                                                   ptr<double>(L.dval), ptr<double>(L.ddiag),
-                                                                   ptr<double>(L.ddinv), ptr<double>(L.x),
-                                                                   ptr<double>(L.b), ptr<double>(L.x2), nullptr);
+void amg_release(Amg &A) {
+    Buf *all[] = {&A.hier, &A.seg, &A.rs, &A.rl, &A.dg, &A.ex, &A.om, &A.x, &A.b, &A.own, &A.gs, &A.gc, &A.ecol, &A.ew,
+                  &A.g, &A.t, &A.cs, &A.pair, &A.scratch, &A.raw_cnt, &A.raw_off, &A.raw_key, &A.vec, &A.stat};
+    for (Buf *b : all) release(*b);
 }
-
-void amg_apply(bchar_mesh_t m, Amg &amg, const double *res, double *z, const CgState *st, bool b_ready,
-               const double *rp, double *pa, double *pb) {
-    vcycle<double>(m, amg, res, z, st, b_ready, rp, pa, pb);
-}
-
-double *amg_finest_rhs(Amg &amg) { return ptr<double>(amg.levels[0].b); }
 
 }  // namespace bchar

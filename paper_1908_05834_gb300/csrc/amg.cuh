@@ -1,22 +1,100 @@
-// Declarations of the aggregation multigrid preconditioner (amg.cu).
+// Declarations of the linear solver of the minimisation: the column pattern of
+// the row-eliminated normal equations (schur.cu), the aggregation-multigrid
+// hierarchy (amg.cu) and the preconditioned conjugate gradients (pcg.cu).
 #pragma once
 
 #include "internal.cuh"
 
 namespace bchar {
 
-// Builds the hierarchy for the current matrix (the minimisation's weights
-// change by orders of magnitude between iterations, so it is built anew each time).
-bool amg_build(bchar_mesh_t m, Amg &amg);
-// z = M^-1 res (one V-cycle).  With b_ready the caller has already written
-// the sign-flipped res into the finest level's right-hand side.  With rp, pa,
-// pb the last kernel also writes per-block partial sums of z.res into pa and
-// of z.rp into pb (kRedBlocks blocks).
-void amg_apply(bchar_mesh_t m, Amg &amg, const double *res, double *z, const CgState *st, bool b_ready = false,
-               const double *rp = nullptr, double *pa = nullptr, double *pb = nullptr);
-// The finest level's right-hand side.
-double *amg_finest_rhs(Amg &amg);
+constexpr int kMaxLevels = 40;
+constexpr int kMaxCtas = 256;        // blocks of the cooperative kernels at most
+constexpr int kSolveThreads = 512;   // threads per block of the conjugate gradients
+constexpr int kBuildThreads = 1024;  // threads per block of the hierarchy build
+constexpr int kDense = 32;           // a coarsest level of at most this many nodes is solved by its inverse
+
+// Levels of at most this many off-diagonal entries and nodes are built and
+// cycled by block 0 alone, between block barriers, from shared memory.
+constexpr int kBlockEntries = 4000;
+constexpr int kBlockNodes = 1500;
+constexpr int kBlockTotalNodes = 2600;  // nodes of all such levels (their vectors must fit shared memory)
+
+// Where one block's share of a level is: its rows (the members of its
+// aggregates, in aggregate order, then its nodes without a coarse counterpart)
+// in the level's order array, and its aggregates.
+struct Seg {
+    int m0, mlen, l0, llen, g0, glen;
+};
+
+struct LevelInfo {
+    int64_t noff;   // first node of the level in the node arrays
+    int64_t nnz;    // off-diagonal entries
+    int n;          // nodes
+    int nmem;       // nodes that have a coarse counterpart
+    int grid;       // 1: shared by all blocks, 0: block 0 alone
+};
+
+// Control block of the hierarchy and the solves, zeroed before every build.
+struct Hier {
+    unsigned bar[4];          // barrier counters: build, predictor solve, corrector solve, stage timing
+    int err;                  // a barrier's wait ran out
+    int overflow;             // the entry arrays are full: coarsening stops
+    unsigned long long ecur;  // entries in use
+    unsigned mcur[kMaxLevels];
+    unsigned long long nnzacc[kMaxLevels];
+    int nlev;
+    int dense;   // the coarsest level is solved by its inverse
+    int sweeps;  // else by this many Jacobi sweeps (even)
+    LevelInfo L[kMaxLevels];
+    int ctasum[2][kMaxCtas];
+    double part[4][kMaxCtas];
+    double inv[kDense * kDense];
+};
+
+// The conjugate gradients' results (and the step's running iteration count).
+struct SolveStat {
+    double rz, res_max;
+    int iters, converged;
+    int total;  // all solves of the step
+    int err;
+};
+
+// The level arrays (device pointers), passed by value to the kernels.
+struct HierView {
+    Hier *H;
+    Seg *seg;  // kMaxLevels x kMaxCtas
+    int64_t capn, cape;
+    int64_t *rs;                    // first entry of each row
+    int32_t *rl;                    // entries of each row
+    double *dg, *ex, *om, *x, *b;   // diagonal, excess, smoother weight, V-cycle vectors
+    int32_t *own;                   // a level's nodes grouped by aggregate, then those without a coarse counterpart
+    int32_t *gs, *gc;               // per coarse node: first member in the finer level's own, members
+    int32_t *ecol;
+    double *ew;                     // weights w > 0: the operator is diag - W
+};
+
+// Grid of the cooperative kernels for a finest level of e0 entries.
+int solve_grid(int64_t e0);
+
+// Once per step: the finest level's pattern (false: out of memory).
+bool schur_pattern(bchar_mesh_t m);
+// The hierarchy for the current weights (rebuilt every interior-point
+// iteration: they change by orders of magnitude).
+void amg_build(bchar_mesh_t m);
+// One solve of the normal equations for m->rhs into m->cg_d; which = 0: from
+// zero, 1: from the finest level's solution left by solve 0.  The tolerances
+// are read on the device: z.res <= rz_rel mu, max |res_l| / b_l <=
+// max(res_rel rp_max, res_floor), with mu and rp_max at scal[0], scal[1].
+struct SolveTol {
+    double rz_rel, res_rel, res_floor;
+    int max_iter;   // of this solve
+    int max_total;  // of the step
+};
+void pcg_launch(bchar_mesh_t m, int which, const double *scal, const SolveTol &tol);
 void amg_release(Amg &amg);
-void amg_smooth_once(bchar_mesh_t m, Amg &amg);
+HierView hier_view(bchar_mesh_t m);
+// Timing aids: one damped-Jacobi sweep of the finest level; one V-cycle.
+void amg_smooth_once(bchar_mesh_t m);
+void amg_vcycle_once(bchar_mesh_t m);
 
 }  // namespace bchar

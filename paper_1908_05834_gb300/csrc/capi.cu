@@ -455,7 +455,7 @@ bchar_status bchar_step(bchar_mesh_t m, double dt, const void *c_in, void *c_out
     launch_scaling(m);
     cudaEventRecord(ev[4], m->stream);
     int cg_iters = 0, ip_iters = 0;
-    if (!launch_minimise(m, &cg_iters, &ip_iters)) return BCHAR_ERR_OUT_OF_MEMORY;
+    if ((st = launch_minimise(m, &cg_iters, &ip_iters)) != BCHAR_OK) return st;
     cudaEventRecord(ev[5], m->stream);
     launch_finalise(m);
     cudaEventRecord(ev[6], m->stream);
@@ -616,10 +616,8 @@ bchar_status bchar_time_stage(bchar_mesh_t m, int stage, int reps, float *mean_m
         case BCHAR_STAGE_CG_MATVEC: launch_cg_matvec_once(m, ptr<CgState>(st)); break;
         case BCHAR_STAGE_UPDATE: launch_update(m, cin.p, cout.p, BCHAR_C_F64); break;
         case BCHAR_STAGE_ASSEMBLE: launch_assemble(m); break;
-        case BCHAR_STAGE_SMOOTH: amg_smooth_once(m, m->amg); break;
-        case BCHAR_STAGE_VCYCLE:  // on the finest right-hand side left by the last solve; z is scratch after the step
-            amg_apply(m, m->amg, nullptr, ptr<double>(m->cg_z), nullptr, true);
-            break;
+        case BCHAR_STAGE_SMOOTH: amg_smooth_once(m); break;
+        case BCHAR_STAGE_VCYCLE: amg_vcycle_once(m); break;  // on the residual left by the last solve
         case BCHAR_STAGE_SCALING: launch_scaling_once(m); break;
         default: launch_track(m, m->dt, m->substeps); break;
         }
@@ -630,7 +628,7 @@ bchar_status bchar_time_stage(bchar_mesh_t m, int stage, int reps, float *mean_m
     // graph is captured on a private stream and launched on the handle's.
     cudaGraphExec_t exec = nullptr;
     if (stage == BCHAR_STAGE_CG_MATVEC || stage == BCHAR_STAGE_UPDATE || stage == BCHAR_STAGE_SMOOTH ||
-        stage == BCHAR_STAGE_SCALING || stage == BCHAR_STAGE_VCYCLE) {
+        stage == BCHAR_STAGE_SCALING) {
         cudaStream_t user = m->stream, cap = nullptr;
         cudaGraph_t graph = nullptr;
         bool ok = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) == cudaSuccess;

@@ -98,27 +98,16 @@ struct Buf {
     int64_t *acct = nullptr;  // the owning handle's byte counter
 };
 
-// One level of the multigrid hierarchy: a symmetric CSR operator (off-diagonal
-// entries only) with its diagonal and excess, the map to the next coarser
-// level, the members of each of its own nodes' aggregates (coarse levels),
-// plus work vectors.
-struct AmgLevel {
-    int64_t n = 0, nnz = 0;
-    Buf ptr, col, val, diag, exc, agg, mptr, mlist, x, x2, b, r;  // mptr/mlist: members of each aggregate
-    Buf dval, ddiag;                   // the operator divided by the scale (work vectors: x, x2, b, r)
-    Buf ddinv;                         // smoother weights omega_i / diag_i of the scaled copy
-    const double *diag_ext = nullptr;  // level 0 shares the minimisation's diagonal
-    const double *exc_ext = nullptr;   // and its excess (the penalty shift)
-};
-
+// The multigrid hierarchy and the conjugate gradients on it (amg.cuh): all
+// levels in shared arrays, the finest first.
 struct Amg {
-    std::vector<AmgLevel> levels;
-    int nlev = 0;
-    Buf tmp;
-    double scale = 1.0;  // the V-cycle's levels hold operator / scale
-    int small_from = 0;        // levels small_from..nlev-1 are cycled by one block (nlev: none)
-    int large_sweeps = 0;      // Jacobi sweeps of a coarsest level too large for one block
-    Buf small_d;               // device descriptors of the small levels
+    Buf hier, seg, stat;                                  // control block, blocks' shares, results
+    Buf rs, rl, dg, ex, om, x, b, own, gs, gc, ecol, ew;  // level arrays
+    Buf g, t, cs, pair, raw_cnt, raw_off, raw_key;        // the finest level's values from A's entries
+    Buf scratch, vec;                                     // matching scratch; vectors of the conjugate gradients
+    int64_t n0 = 0, e0 = 0;      // nodes and entries of the finest level
+    int64_t capn = 0, cape = 0;  // room in the level arrays
+    bool schur = false;          // finest level: the columns, rows eliminated (else rows and columns)
 };
 
 }  // namespace bchar
@@ -267,7 +256,7 @@ bool launch_tiles(bchar_mesh_t m);  // tile boundaries of both views (false: out
 bool launch_balance(bchar_mesh_t m);  // components.cu
 void launch_scaling(bchar_mesh_t m);
 void launch_scaling_once(bchar_mesh_t m);  // one column and one row scaling (timing aid)
-bool launch_minimise(bchar_mesh_t m, int *cg_iters, int *ip_iters);  // false: out of memory
+bchar_status launch_minimise(bchar_mesh_t m, int *cg_iters, int *ip_iters);
 void launch_finalise(bchar_mesh_t m);
 void launch_update(bchar_mesh_t m, const void *c_in, void *c_out, int c_dtype);
 void launch_cg_matvec_once(bchar_mesh_t m, CgState *st);  // q = J p with the current p, for timing

@@ -533,29 +533,6 @@ __global__ void k_cg_update(int64_t n2, const double *p, const double *q, double
     if (threadIdx.x == 0) partials[blockIdx.x] = mx;
 }
 
-// The same, also writing the next V-cycle's right-hand side b = S res in its
-// precision T (S: +1 rows, -1 columns), so that the V-cycle needs no pass of
-// its own over res.
-template <class T>
-__global__ void k_cg_update_b(int64_t nc, const double *p, const double *q, double *d, double *res, double *rp,
-                              const double *b_row, const double *volphi, double *partials, T *b, const CgState *st) {
-    dep_enter();
-    if (st->converged) return;
-    const double alpha = st->alpha;
-    double mx = 0.0;
-    GRID_STRIDE(l, 2 * nc) {
-        d[l] += alpha * p[l];
-        const double r0 = res[l];
-        rp[l] = r0;
-        const double r = r0 - alpha * q[l];
-        res[l] = r;
-        b[l] = static_cast<T>(l < nc ? r : -r);
-        mx = fmax(mx, fabs(r) / ip_target(nc, l, b_row, volphi));
-    }
-    mx = block_max(mx);
-    if (threadIdx.x == 0) partials[blockIdx.x] = mx;
-}
-
 // partial sums of z.res and z.rp (flexible, Polak-Ribiere form of beta: the
 // preconditioner may differ slightly between applications)
 __global__ void k_dot2(int64_t n, const double *z, const double *res, const double *rp, double *pa, double *pb,
@@ -607,6 +584,7 @@ __global__ void k_cg_pupdate(int64_t n2, const double *z, double *p, const CgSta
 // Scalars of one interior-point iteration, reduced over blocks (kRedBlocks
 // partial slots each) and read back once.
 struct IpScalars {
+    double mu;          // mean complementarity (the solves read it and rp_max, in this order)
     double rp_max;      // max_l |rp_l| / b_l (the scaled constraint residual)
     double rd_max;      // max_e |rd_e|
     double rpq_max;     // max_l of the stationarity residuals of p and n
@@ -615,6 +593,8 @@ struct IpScalars {
     double rp_l1;       // sum_l |rp_l| (unscaled)
     double ap, ad;      // largest primal / dual step to the boundary (<= 1)
     double comp_aff;    // the same sum after the predictor's steps
+    double sigma_mu;    // the corrector's complementarity target
+    int err;            // a solver kernel's barrier failed
 };
 
 constexpr int kIpSlots = 8;  // partial-sum slots per block in the reduction scratch
@@ -697,7 +677,7 @@ __global__ void k_ip_nodes(int64_t nc, const int64_t *row_ptr, const int64_t *co
     }
 }
 
-__global__ void k_ip_reduce_resid(const double *part, int nparts, IpScalars *st) {
+__global__ void k_ip_reduce_resid(const double *part, int nparts, double pairs, const int *solver_err, IpScalars *st) {
     double rd = 0.0, rp = 0.0, rpq = 0.0, dm = 0.0, comp = 0.0, l1 = 0.0;
     for (int k = threadIdx.x; k < nparts; k += blockDim.x) {
         const double *pb = part + kIpSlots * k;
@@ -721,16 +701,20 @@ __global__ void k_ip_reduce_resid(const double *part, int nparts, IpScalars *st)
         st->rpq_max = rpq;
         st->dual_max = dm;
         st->comp = comp;
+        st->mu = comp / pairs;
+        st->err = solver_err ? *solver_err : 0;
     }
 }
 
 // Normal-equation weights: D_e, a2_e = a_e^2 D_e, and per node
-// exc_l = b_l^2 (eps^2 + p_l / zp_l + n_l / zn_l) and diag_l = sum a^2 D + exc_l.
+// exc_l = b_l^2 (eps^2 + p_l / zp_l + n_l / zn_l) and diag_l = sum a^2 D + exc_l;
+// with g, t also the factors of the system with the rows eliminated,
+// g_e = a2_e / sqrt(diag_row) and t_row = exc_row / diag_row.
 __global__ void k_ip_weights(int64_t nc, const int64_t *row_ptr, const int64_t *col_ptr, const int32_t *csc_src,
                              const double *a, const double *b_row, const double *volphi, double eps2,
                              const double *f, const double *u, const double *zl, const double *zh, const double *p,
                              const double *n, const double *zp, const double *zn, double *D, double *a2, double *diag,
-                             double *exc) {
+                             double *exc, double *g, double *t) {
     dep_enter();
     GRID_STRIDE(l, 2 * nc) {
         double d = 0.0;
@@ -751,18 +735,24 @@ __global__ void k_ip_weights(int64_t nc, const int64_t *row_ptr, const int64_t *
         const double x = bl * bl * (eps2 + p[l] / zp[l] + n[l] / zn[l]);
         diag[l] = d + x;
         exc[l] = x;
+        if (g && l < nc) {
+            const double w = 1.0 / sqrt(d + x);
+            for (int64_t e = row_ptr[l]; e < row_ptr[l + 1]; ++e) g[e] = a2[e] * w;
+            t[l] = x / (d + x);
+        }
     }
 }
 
 // Reduced right-hand side per entry for the predictor (corrector = 0) or the
-// corrector (sigma_mu = sigma * mu, with the predictor's direction in df..dzh):
+// corrector (st->sigma_mu = sigma * mu, with the predictor's direction in df..dzh):
 //   cl = target of f zl, ch = target of u zh,
 //   q = -rd + cl / f - ch / u + (zh / u) ru.
 __global__ void k_ip_q(int64_t nc, const int64_t *row_ptr, const int32_t *col, const double *a, const double *y,
                        const double *f, const double *u, const double *zl, const double *zh, int corrector,
-                       double sigma_mu, const double *df, const double *du, const double *dzl, const double *dzh,
+                       const IpScalars *st, const double *df, const double *du, const double *dzl, const double *dzh,
                        double *cl, double *ch, double *q) {
     dep_enter();
+    const double sigma_mu = corrector ? st->sigma_mu : 0.0;
     GRID_STRIDE(i, nc) {
         const double yi = y[i];
         for (int64_t e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
@@ -787,9 +777,10 @@ __global__ void k_ip_q(int64_t nc, const int64_t *row_ptr, const int32_t *col, c
 __global__ void k_ip_rhs(int64_t nc, const int64_t *row_ptr, const int64_t *col_ptr, const int32_t *csc_src,
                          const double *a, const double *D, const double *q, const double *rp, const double *b_row,
                          const double *volphi, double gamma, const double *y, const double *p, const double *n,
-                         const double *zp, const double *zn, int corrector, double sigma_mu, const double *dp,
+                         const double *zp, const double *zn, int corrector, const IpScalars *st, const double *dp,
                          const double *dn, const double *dzp, const double *dzn, double *cp, double *cn, double *rhs) {
     dep_enter();
+    const double sigma_mu = corrector ? st->sigma_mu : 0.0;
     GRID_STRIDE(l, 2 * nc) {
         double s = 0.0;
         if (l < nc) {
@@ -920,11 +911,16 @@ __global__ void k_ip_comp_aff(int64_t nnz, int64_t n2, const double *f, const do
     }
 }
 
-__global__ void k_ip_reduce_comp_aff(const double *part, int nparts, IpScalars *st) {
+// Mehrotra's centring target (comp_aff / comp)^3 mu, not below the floor.
+__global__ void k_ip_reduce_comp_aff(const double *part, int nparts, double mu_floor, IpScalars *st) {
     double s = 0.0;
     for (int k = threadIdx.x; k < nparts; k += blockDim.x) s += part[kIpSlots * k + 4] + part[kIpSlots * k + 5];
     s = block_sum(s);
-    if (threadIdx.x == 0) st->comp_aff = s;
+    if (threadIdx.x == 0) {
+        const double r = s / st->comp;
+        st->comp_aff = s;
+        st->sigma_mu = fmax(fmin(1.0, r * r * r) * st->mu, mu_floor);
+    }
 }
 
 // Step with fraction 0.99 of the way to the boundary.
@@ -982,22 +978,13 @@ __global__ void k_ip_finish(int64_t nnz, const double *f, double *qx, DevInfo *i
     if (at) atomicAdd(&info->n_at_bounds, at);
 }
 
-static void precondition(bchar_mesh_t m, bool amg, const double *res, double *z, const CgState *st,
-                         bool b_ready = false, const double *rp = nullptr, double *pa = nullptr,
-                         double *pb = nullptr) {
-    if (amg) {
-        amg_apply(m, m->amg, res, z, st, b_ready, rp, pa, pb);
-    } else {
-        k_jacobi_precond<<<blocks_for(2 * m->nc), kThreads, 0, m->stream>>>(2 * m->nc, ptr<double>(m->diag), res, z, st);
-        ++m->launches;
-    }
-}
-
 // A solve of the conjugate gradients stops when its residual has not dropped
 // by 1 % for kStallIters iterations (it cannot improve further in FP64).
 constexpr int kStallIters = 400;
 
-// The conjugate gradients on (A-hat D A-hat^T + diag(exc)) d = rhs, from
+// The conjugate gradients with the Jacobi preconditioner (qp_precond = 0; with
+// the multigrid the whole solve is one kernel, pcg.cu)
+// on (A-hat D A-hat^T + diag(exc)) d = rhs, from
 // d = 0 (or, with warm, from the d already in place), until z.res <= target_rz
 // (z the preconditioned residual: about the squared error of d in the norm of
 // the matrix, which bounds the error of A-hat^T d where the interior-point
@@ -1008,7 +995,7 @@ constexpr int kStallIters = 400;
 // into a CUDA graph per preconditioner build (*exec; destroyed by the caller)
 // and replayed until the solve has converged (its kernels do nothing then);
 // the host polls once per batch.  Returns the iterations done.
-static int pcg_solve(bchar_mesh_t m, const double *rhs, double target_rz, double target_res, bool amg, bool warm,
+static int pcg_solve(bchar_mesh_t m, const double *rhs, double target_rz, double target_res, bool warm,
                      int max_iter, cudaGraphExec_t *exec, int *graph_launches) {
     const int64_t nc = m->nc, n2 = 2 * nc;
     const int bl = blocks_for(n2);
@@ -1034,30 +1021,23 @@ static int pcg_solve(bchar_mesh_t m, const double *rhs, double target_rz, double
         k_copy<<<bl, kThreads, 0, s>>>(n2, rhs, res, nullptr);
         ++m->launches;
     }
-    precondition(m, amg, res, z, nullptr);
+    k_jacobi_precond<<<bl, kThreads, 0, s>>>(n2, diag, res, z, nullptr);
     k_dot<<<kRedBlocks, kThreads, 0, s>>>(n2, res, z, part_rz, nullptr);
     // the right-hand side's residual norm is not formed: the first iteration checks it
     k_cg_start<<<1, 1024, 0, s>>>(part_rz, kRedBlocks, target_rz, target_res, INFINITY, st);
     k_copy<<<bl, kThreads, 0, s>>>(n2, z, p, nullptr);
-    m->launches += 3;
-    const int batch = amg ? 8 : 32;
+    m->launches += 4;
+    const int batch = 32;
     const int mv_grid = tile_grid(2 * m->ntile);  // <= kRedBlocks partial sums of p.q
     auto enqueue_batch = [&]() {
         for (int k = 0; k < batch; ++k) {
             launch_dep_smem(k_cg_matvec, mv_grid, kTileThreads, kTileSmem, s, row_view(m, a2), col_view(m, a2c), diag, p,
                             q, part, st);
             launch_dep(k_cg_alpha, 1, 1024, s, part, mv_grid, st);
-            if (amg) {
-                launch_dep(k_cg_update_b<double>, kRedBlocks, kThreads, s, nc, p, q, d, res, rp, brow, volphi, part_res,
-                           amg_finest_rhs(m->amg), st);
-                precondition(m, amg, res, z, st, true, rp, part_rz, part_zp);
-                m->launches += 3;
-            } else {
-                launch_dep(k_cg_update, kRedBlocks, kThreads, s, n2, p, q, d, res, rp, brow, volphi, part_res, st);
-                precondition(m, amg, res, z, st);
-                launch_dep(k_dot2, kRedBlocks, kThreads, s, n2, z, res, rp, part_rz, part_zp, st);
-                m->launches += 4;
-            }
+            launch_dep(k_cg_update, kRedBlocks, kThreads, s, n2, p, q, d, res, rp, brow, volphi, part_res, st);
+            launch_dep(k_jacobi_precond, bl, kThreads, s, n2, diag, res, z, st);
+            launch_dep(k_dot2, kRedBlocks, kThreads, s, n2, z, res, rp, part_rz, part_zp, st);
+            m->launches += 5;
             launch_dep(k_cg_beta, 1, 1024, s, part_rz, part_zp, part_res, kRedBlocks, st);
             launch_dep(k_cg_pupdate, bl, kThreads, s, n2, z, p, st);
             m->launches += 2;
@@ -1139,7 +1119,7 @@ constexpr double kIpStep = 0.99;
 // take up to twice the iterations on the 1024^2 workload.
 constexpr double kIpStartViol = 0.1;
 
-bool launch_minimise(bchar_mesh_t m, int *cg_iters, int *ip_iters) {
+bchar_status launch_minimise(bchar_mesh_t m, int *cg_iters, int *ip_iters) {
     const bool trace = getenv("BCHAR_TRACE") != nullptr;  // diagnostic: per-iteration scalars on stderr
     double t_start = 0.0;
     if (trace) {
@@ -1151,11 +1131,11 @@ bool launch_minimise(bchar_mesh_t m, int *cg_iters, int *ip_iters) {
     Buf *ent[] = {&m->ip_f, &m->ip_u, &m->ip_zl, &m->ip_zh, &m->ip_D, &m->ip_q, &m->ip_cl, &m->ip_ch,
                   &m->ip_df, &m->ip_du, &m->ip_dzl, &m->ip_dzh};
     for (Buf *b : ent)
-        if (!ensure(m, *b, zb)) return false;
+        if (!ensure(m, *b, zb)) return BCHAR_ERR_OUT_OF_MEMORY;
     Buf *nod[] = {&m->ip_p, &m->ip_n, &m->ip_zp, &m->ip_zn, &m->ip_cp, &m->ip_cn, &m->ip_dp, &m->ip_dn,
                   &m->ip_dzp, &m->ip_dzn};
     for (Buf *b : nod)
-        if (!ensure(m, *b, nb)) return false;
+        if (!ensure(m, *b, nb)) return BCHAR_ERR_OUT_OF_MEMORY;
     static_assert(kIpSlots * kRedBlocks <= 152 * 64, "interior-point partials fit the first scratch section");
     cudaStream_t s = m->stream;
     const double eps2 = m->opt.penalty * m->opt.penalty;
@@ -1181,6 +1161,9 @@ bool launch_minimise(bchar_mesh_t m, int *cg_iters, int *ip_iters) {
     const int blm = blocks_for(nnz > n2 ? nnz : n2);
     const double pairs = 2.0 * static_cast<double>(nnz) + 2.0 * static_cast<double>(n2);
     const bool use_amg = m->opt.qp_precond == 1;
+    bool have_pattern = false;  // the finest level's pattern of this step
+    SolveStat *stat = nullptr, solve{};
+    const int *solver_err = nullptr;
 
     k_ip_init<<<blm, kThreads, 0, s>>>(nnz, n2, kIpStartViol * gamma, kIpStartViol, gamma, f, u, zl, zh, y, p, n, zp,
                                        zn);
@@ -1191,11 +1174,18 @@ bool launch_minimise(bchar_mesh_t m, int *cg_iters, int *ip_iters) {
         launch_dep(k_ip_entries, blr, kThreads, s, nc, row_ptr, col, a, y, f, u, zl, zh, part);
         launch_dep(k_ip_nodes, blr, kThreads, s, nc, row_ptr, col_ptr, csc_src, a, brow, volphi, eps2, gamma, y, f, p,
                    n, zp, zn, rp, part);
-        k_ip_reduce_resid<<<1, 1024, 0, s>>>(part, blr, st);
+        k_ip_reduce_resid<<<1, 1024, 0, s>>>(part, blr, pairs, have_pattern ? solver_err : nullptr, st);
         m->launches += 3;
         cudaMemcpyAsync(&hs, st, sizeof hs, cudaMemcpyDeviceToHost, s);
+        if (have_pattern) cudaMemcpyAsync(&solve, stat, sizeof solve, cudaMemcpyDeviceToHost, s);
         if (cudaStreamSynchronize(s) != cudaSuccess) break;  // the caller reads the error
-        const double mu = hs.comp / pairs;
+        if (cudaPeekAtLastError() != cudaSuccess) break;     // a launch failed: likewise
+        if (have_pattern) total_cg = solve.total;
+        if (hs.err) {
+            m->err = "a solver kernel's grid barrier timed out";
+            return BCHAR_ERR_CUDA;
+        }
+        const double mu = hs.mu;
         if (trace)
             fprintf(stderr, "[bchar] ip %d rp %.3e rd %.3e rpq %.3e mu %.3e dual %.3e ap %.3e ad %.3e cg %d (%.1f ms)\n",
                     it, hs.rp_max, hs.rd_max, hs.rpq_max, mu, hs.dual_max, hs.ap, hs.ad, total_cg,
@@ -1206,40 +1196,46 @@ bool launch_minimise(bchar_mesh_t m, int *cg_iters, int *ip_iters) {
             break;
         }
         if (it == m->opt.qp_max_refine || total_cg >= m->opt.qp_max_iter) break;
+        if (use_amg && !have_pattern) {
+            if (!schur_pattern(m)) return BCHAR_ERR_OUT_OF_MEMORY;
+            have_pattern = true;
+            stat = ptr<SolveStat>(m->amg.stat);
+            solver_err = &ptr<Hier>(m->amg.hier)->err;
+            cudaMemsetAsync(stat, 0, sizeof(SolveStat), s);
+        }
         // normal-equation matrix and its preconditioner; the weights change by orders of
         // magnitude between iterations, so the aggregates are built anew every time
+        const bool schur = use_amg && m->amg.schur;
         launch_dep(k_ip_weights, bl2, kThreads, s, nc, row_ptr, col_ptr, csc_src, a, brow, volphi, eps2, f, u, zl, zh, p,
-                   n, zp, zn, D, ptr<double>(m->a2), ptr<double>(m->diag), ptr<double>(m->qexc));
+                   n, zp, zn, D, ptr<double>(m->a2), ptr<double>(m->diag), ptr<double>(m->qexc),
+                   schur ? ptr<double>(m->amg.g) : nullptr, schur ? ptr<double>(m->amg.t) : nullptr);
         k_qp_gather_cols<<<blocks_for(nnz), kThreads, 0, s>>>(nnz, csc_src, ptr<double>(m->a2), ptr<double>(m->a2c));
         m->launches += 2;
-        const bool amg = use_amg && amg_build(m, m->amg);
+        if (use_amg) amg_build(m);
         // each direction solved until its squared energy-norm error is about <= 1e-2 mu (then
         // every entry's step error stays about <= 0.1 of its distance to the bound) and the
         // constraint residual it leaves is, relative to each target, <= 0.1 of the current
         // one (which the step then reduces), but not below half the stopping tolerance
-        const double target_rz = 1e-2 * mu;
-        const double target_res = fmax(0.1 * hs.rp_max, 0.5 * m->opt.qp_tol);
+        const SolveTol tol{1e-2, 0.1, 0.5 * m->opt.qp_tol, kIpCgPerSolve, m->opt.qp_max_iter};
         cudaGraphExec_t exec = nullptr;
         int graph_launches = 0;
         for (int corr = 0; corr < 2; ++corr) {
-            const double sigma_mu = corr ? fmax(fmin(1.0, pow(hs.comp_aff / hs.comp, 3.0)) * mu, kIpMuFloor) : 0.0;
-            launch_dep(k_ip_q, blr, kThreads, s, nc, row_ptr, col, a, y, f, u, zl, zh, corr, sigma_mu, df, du, dzl,
-                       dzh, cl, ch, q);
+            launch_dep(k_ip_q, blr, kThreads, s, nc, row_ptr, col, a, y, f, u, zl, zh, corr, st, df, du, dzl, dzh, cl,
+                       ch, q);
             launch_dep(k_ip_rhs, bl2, kThreads, s, nc, row_ptr, col_ptr, csc_src, a, D, q, rp, brow, volphi, gamma, y,
-                       p, n, zp, zn, corr, sigma_mu, dp, dn, dzp, dzn, cp, cn, rhs);
+                       p, n, zp, zn, corr, st, dp, dn, dzp, dzn, cp, cn, rhs);
             m->launches += 2;
-            const int left = m->opt.qp_max_iter - total_cg;
-            const int cap = left < kIpCgPerSolve ? left : kIpCgPerSolve;
-            // the right-hand side's L1 norm: the node pass's |rp|_1 bounds it well enough for the start
             // the corrector's system differs from the predictor's only in its right-hand
             // side (the centring and second-order terms): its solve starts from the
             // predictor's direction
-            const int done = pcg_solve(m, rhs, target_rz, target_res, amg, corr == 1, cap > 0 ? cap : 1,
-                                       &exec, &graph_launches);
-            total_cg += done;
-            if (trace)
-                fprintf(stderr, "[bchar]   solve %d: %d CG iterations, levels %d, coarsest %lld\n", corr, done,
-                        amg ? m->amg.nlev : 0, amg ? static_cast<long long>(m->amg.levels[m->amg.nlev - 1].n) : 0LL);
+            if (use_amg) {
+                pcg_launch(m, corr, &st->mu, tol);
+            } else {
+                const int left = m->opt.qp_max_iter - total_cg;
+                const int cap = left < kIpCgPerSolve ? left : kIpCgPerSolve;
+                total_cg += pcg_solve(m, rhs, tol.rz_rel * mu, fmax(tol.res_rel * hs.rp_max, tol.res_floor), corr == 1,
+                                      cap > 0 ? cap : 1, &exec, &graph_launches);
+            }
             launch_dep(k_ip_dir, blr, kThreads, s, nc, row_ptr, col, a, dy, f, u, zl, zh, D, q, cl, ch, df, du, dzl,
                        dzh, part);
             launch_dep(k_ip_dir_nodes, blr, kThreads, s, nc, brow, volphi, gamma, y, dy, p, n, zp, zn, cp, cn, dp, dn,
@@ -1249,10 +1245,8 @@ bool launch_minimise(bchar_mesh_t m, int *cg_iters, int *ip_iters) {
             if (!corr) {
                 launch_dep(k_ip_comp_aff, blr, kThreads, s, nnz, n2, f, u, zl, zh, df, du, dzl, dzh, p, n, zp, zn, dp,
                            dn, dzp, dzn, st, part);
-                k_ip_reduce_comp_aff<<<1, 1024, 0, s>>>(part, blr, st);
+                k_ip_reduce_comp_aff<<<1, 1024, 0, s>>>(part, blr, kIpMuFloor, st);
                 m->launches += 2;
-                cudaMemcpyAsync(&hs, st, sizeof hs, cudaMemcpyDeviceToHost, s);
-                cudaStreamSynchronize(s);
             }
         }
         if (exec) cudaGraphExecDestroy(exec);
@@ -1273,9 +1267,20 @@ bool launch_minimise(bchar_mesh_t m, int *cg_iters, int *ip_iters) {
     m->ip_converged = converged;
     *cg_iters = total_cg;
     *ip_iters = it;
-    m->amg_levels = use_amg ? m->amg.nlev : 0;
-    m->amg_coarsest = use_amg && m->amg.nlev > 0 ? m->amg.levels[m->amg.nlev - 1].n : 0;
-    return true;
+    m->amg_levels = 0;
+    m->amg_coarsest = 0;
+    if (have_pattern) {
+        Hier *H = ptr<Hier>(m->amg.hier);
+        LevelInfo L[kMaxLevels];
+        int nlev = 0;
+        cudaMemcpyAsync(&nlev, &H->nlev, sizeof nlev, cudaMemcpyDeviceToHost, s);
+        cudaMemcpyAsync(L, H->L, sizeof L, cudaMemcpyDeviceToHost, s);
+        if (cudaStreamSynchronize(s) == cudaSuccess && nlev > 0 && nlev <= kMaxLevels) {
+            m->amg_levels = nlev;
+            m->amg_coarsest = L[nlev - 1].n;
+        }
+    }
+    return BCHAR_OK;
 }
 
 void launch_cg_matvec_once(bchar_mesh_t m, CgState *st) {
