@@ -80,7 +80,8 @@ struct BuildArgs {
     const double *g, *t;                  // a2 / sqrt(diag_row) per entry; exc / diag per row
     const uint32_t *cs;                   // first contribution of each entry of the finest level
     const int2 *pair;                     // contributions: two entries of one row of A
-    int32_t *best0, *best1, *partner, *att, *lead, *pos, *agg, *cnt, *cap;  // n0 each
+    int same;                             // 1: the aggregates of the build before
+    int32_t *best0, *best1, *partner, *att, *lead, *pos, *cnt, *cap;  // n0 each
 };
 
 __device__ __forceinline__ uint32_t edge_hash(int64_t i, int64_t j) {
@@ -95,10 +96,18 @@ __device__ __forceinline__ uint32_t edge_hash(int64_t i, int64_t j) {
 }
 
 // Rank of an edge: exponent field of the weight, then the hash.
-__device__ __forceinline__ unsigned long long edge_rank(int i, int j, double w) {
-    const unsigned long long cls = (static_cast<unsigned long long>(__double_as_longlong(w)) >> 52) & 0x7ffull;
-    return (cls << 32) | edge_hash(i, j);
+__device__ __forceinline__ unsigned long long edge_rank(int i, int j, int hi) {
+    return (static_cast<unsigned long long>(hi >> 20) << 32) | edge_hash(i, j);
 }
+
+// The high word of a positive double is monotone in it, and as an integer a
+// piecewise linear log2 in units of 2^-20 (off by at most 0.086): the tests of
+// the matching compare those, because a warp instruction of the FP64 pipe costs
+// 19 clocks of the SM and an integer one a quarter of a clock.
+__device__ __forceinline__ int high_word(double w) { return __double2hiint(w); }
+constexpr int kStrengthHi = 3483294;  // -log2(kStrength) = 3.3219, in those units
+constexpr int kAttachHi = 2 << 20;    // -log2(kAttach)
+static_assert(kStrength == 0.1 && kAttach == 0.25, "the constants above follow them");
 
 // The higher-ranked of (key, j) and (k2, j2); j < 0 is none; ties go to the smaller node.
 __device__ __forceinline__ void take_higher(unsigned long long &key, int &j, unsigned long long k2, int j2) {
@@ -106,10 +115,6 @@ __device__ __forceinline__ void take_higher(unsigned long long &key, int &j, uns
         key = k2;
         j = j2;
     }
-}
-
-__device__ __forceinline__ bool leaves(const HierView &v, int64_t k) {
-    return v.rl[k] == 0 || v.ex[k] >= (1.0 - kDominant) * v.dg[k];
 }
 
 // Exclusive scan of one int per thread over the block (kBuildThreads); tmp: 33 ints of shared memory.
@@ -142,55 +147,63 @@ __device__ __forceinline__ double warp_sum(double s) {
     return s;
 }
 
-// ---- the finest level's values: LPR lanes per row
+// ---- a level's diagonals, one thread per row: the entries' weights are summed
+// to the diagonal on top of the excess (base: what the row has of it so far), and
+// the node is marked when it leaves the hierarchy (partner: -3, else -1).
+
+__device__ __forceinline__ void finish_row(const HierView &v, int64_t k, double ex, int32_t *partner) {
+    const int64_t e0 = v.rs[k];
+    const int len = v.rl[k];
+    double s = 0.0;
+    for (int e = 0; e < len; ++e) s += v.ew[e0 + e];
+    const double d = ex + s;
+    v.ex[k] = ex;
+    v.dg[k] = d;
+    v.om[k] = (len == 0 ? 1.0 : kOmega) / d;
+    *partner = len == 0 || ex >= (1.0 - kDominant) * d ? -3 : -1;
+}
+
+// ---- the finest level's weights (LPR lanes per row), then its diagonals
 
 template <int LPR> __device__ void level0_values(const BuildArgs &a, int i0, int i1) {
     const int lane = threadIdx.x & 31, sub = lane % LPR;
     const HierView &v = a.v;
-    for (int r0 = i0 + static_cast<int>(threadIdx.x >> 5) * (32 / LPR); r0 < i1; r0 += blockDim.x / LPR) {
-        const int i = r0 + lane / LPR;
-        const bool ok = i < i1;
-        double s = 0.0, x = 0.0;
-        int len = 0;
-        if (ok) {
-            const int64_t e0 = v.rs[i];
-            len = v.rl[i];
-            if (a.schur) {
-                for (int e = sub; e < len; e += LPR) {
-                    double w = 0.0;
-                    const uint32_t k1 = a.cs[e0 + e + 1];
-                    for (uint32_t k = a.cs[e0 + e]; k < k1; ++k) {
-                        const int2 p = a.pair[k];
-                        w += a.g[p.x] * a.g[p.y];
-                    }
-                    v.ew[e0 + e] = w;
-                    s += w;
+    for (int i = i0 + static_cast<int>(threadIdx.x) / LPR; i < i1; i += blockDim.x / LPR) {
+        const int64_t e0 = v.rs[i];
+        const int len = v.rl[i];
+        if (a.schur) {
+            for (int e = sub; e < len; e += LPR) {
+                double w = 0.0;
+                const uint32_t k1 = a.cs[e0 + e + 1];
+                for (uint32_t k = a.cs[e0 + e]; k < k1; ++k) {
+                    const int2 p = a.pair[k];
+                    w += a.g[p.x] * a.g[p.y];
                 }
-                for (int64_t p = a.col_ptr[i] + sub; p < a.col_ptr[i + 1]; p += LPR) x += a.a2c[p] * a.t[a.csc_row[p]];
-            } else {
-                const bool row = i < a.nc;
-                const int64_t src = row ? e0 : a.col_ptr[i - a.nc];  // the row entries come first, in CSR order
-                for (int e = sub; e < len; e += LPR) v.ew[e0 + e] = row ? a.a2[src + e] : a.a2c[src + e];
+                v.ew[e0 + e] = w;
             }
+        } else {
+            const bool row = i < a.nc;
+            const int64_t src = row ? e0 : a.col_ptr[i - a.nc];  // the row entries come first, in CSR order
+            for (int e = sub; e < len; e += LPR) v.ew[e0 + e] = row ? a.a2[src + e] : a.a2c[src + e];
         }
-        for (int o = LPR / 2; o > 0; o >>= 1) {
-            s += __shfl_xor_sync(0xffffffffu, s, o);
-            x += __shfl_xor_sync(0xffffffffu, x, o);
+    }
+    __syncthreads();
+    for (int i = i0 + static_cast<int>(threadIdx.x); i < i1; i += blockDim.x) {
+        double ex;
+        if (a.schur) {
+            ex = a.exc[a.nc + i];
+            for (int64_t p = a.col_ptr[i]; p < a.col_ptr[i + 1]; ++p) ex += a.a2c[p] * a.t[a.csc_row[p]];
+        } else {
+            ex = a.exc[i];
         }
-        if (ok && sub == 0) {
-            const double ex = a.schur ? a.exc[a.nc + i] + x : a.exc[i];
-            const double d = a.schur ? ex + s : a.diag[i];
-            v.ex[i] = ex;
-            v.dg[i] = d;
-            v.om[i] = (len == 0 ? 1.0 : kOmega) / d;
-        }
+        finish_row(v, i, ex, &a.partner[i]);
     }
 }
 
 // ---- one matching round (LPR lanes per node of the level at node offset noff)
 
 template <int LPR>
-__device__ void rank_round(const BuildArgs &a, int64_t noff, int n, int i0, int i1, int round, const int32_t *bprev,
+__device__ void rank_round(const BuildArgs &a, int64_t noff, int i0, int i1, int round, const int32_t *bprev,
                            int32_t *bcur) {
     const HierView &v = a.v;
     const int lane = threadIdx.x & 31, sub = lane % LPR;
@@ -199,41 +212,33 @@ __device__ void rank_round(const BuildArgs &a, int64_t noff, int n, int i0, int 
         const int i = r0 + lane / LPR;
         const bool ok = i < i1;
         unsigned long long key = 0, akey = 0;
-        int bj = -1, aj = -1, mate = -3;
-        double wmax = 0.0, di = 0.0;
+        int bj = -1, aj = -1, mate = -3, wmax = 0, di = 0;
         if (ok) {
-            di = v.dg[noff + i];
-            if (round == 0) {
-                mate = leaves(v, noff + i) ? -3 : -1;
-            } else {
-                mate = partner[i];
-                if (mate == -1) {  // did the previous round's choices meet?
-                    const int b = bprev[i];
-                    if (b >= 0 && bprev[b] == i) mate = b;
-                }
+            di = high_word(v.dg[noff + i]);
+            mate = partner[i];
+            if (round > 0 && mate == -1) {  // did the previous round's choices meet?
+                const int b = bprev[i];
+                if (b >= 0 && bprev[b] == i) mate = b;
             }
-            const bool open = mate == -1;
-            if (open) {
+            if (mate == -1) {
                 const int64_t e0 = v.rs[noff + i];
                 const int len = v.rl[noff + i];
                 for (int e = sub; e < len; e += LPR) {
                     const int j = v.ecol[e0 + e];
-                    const double w = v.ew[e0 + e];
-                    if (!(w > 0.0)) continue;
-                    if (round == 0) {
-                        if (leaves(v, noff + j)) continue;
-                    } else {
-                        if (partner[j] != -1) continue;
+                    const int w = high_word(v.ew[e0 + e]);
+                    if (w <= 0) continue;
+                    if (partner[j] != -1) continue;
+                    if (round > 0) {
                         const int b = bprev[j];
                         if (b >= 0 && bprev[b] == j) continue;
                     }
                     const unsigned long long k = edge_rank(i, j, w);
                     if (round == 0) {
-                        wmax = fmax(wmax, w);
+                        wmax = max(wmax, w);
                         take_higher(akey, aj, k, j);
                     }
-                    // strong: w >= kStrength sqrt(d_i d_j), compared squared
-                    if (w * w >= (kStrength * kStrength) * (di * v.dg[noff + j])) take_higher(key, bj, k, j);
+                    // strong: w >= kStrength sqrt(d_i d_j)
+                    if (2 * (w + kStrengthHi) >= di + high_word(v.dg[noff + j])) take_higher(key, bj, k, j);
                 }
             }
         }
@@ -241,16 +246,17 @@ __device__ void rank_round(const BuildArgs &a, int64_t noff, int n, int i0, int 
             take_higher(key, bj, __shfl_xor_sync(0xffffffffu, key, o), __shfl_xor_sync(0xffffffffu, bj, o));
             if (round == 0) {
                 take_higher(akey, aj, __shfl_xor_sync(0xffffffffu, akey, o), __shfl_xor_sync(0xffffffffu, aj, o));
-                wmax = fmax(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
+                wmax = max(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
             }
         }
         if (ok && sub == 0) {
             bcur[i] = bj;
-            partner[i] = mate;
-            if (round == 0) {
+            if (round > 0) {
+                partner[i] = mate;
+            } else {
                 // one-sided on purpose: a leaf hanging off a hub by an edge that is most of
                 // its own diagonal but little of the hub's should follow the hub
-                a.att[i] = (aj >= 0 && wmax >= kAttach * di) ? aj : -1;
+                a.att[i] = (aj >= 0 && wmax + kAttachHi >= di) ? aj : -1;
                 a.cnt[i] = 0;
                 a.cap[i] = 0;
             }
@@ -326,11 +332,10 @@ template <class Sync> __device__ void bitonic(unsigned long long *keys, int P, i
 // Merges the sorted entries (key: coarse node << 32 | arrival; all ones: none)
 // into the coarse row I, summing equal nodes in arrival order; one warp.
 __device__ void merge_row(const HierView &v, int64_t noff2, int I, const unsigned long long *keys, const double *vals,
-                          int n, double ex, int &len) {
+                          int n, int &len) {
     const int lane = threadIdx.x & 31;
     const int64_t dst = v.rs[noff2 + I];
     int runs = 0;
-    double d = 0.0;
     for (int base = 0; base < n; base += 32) {
         const int i = base + lane;
         const unsigned long long k = i < n ? keys[i] : ~0ull;
@@ -344,17 +349,10 @@ __device__ void merge_row(const HierView &v, int64_t noff2, int I, const unsigne
             const int64_t at = dst + runs + __popc(mask & ((1u << lane) - 1u));
             v.ecol[at] = J;
             v.ew[at] = s;
-            d += s;
         }
         runs += __popc(mask);
     }
-    d = warp_sum(d) + ex;
-    if (lane == 0) {
-        v.rl[noff2 + I] = runs;
-        v.dg[noff2 + I] = d;
-        v.ex[noff2 + I] = ex;
-        v.om[noff2 + I] = (runs == 0 ? 1.0 : kOmega) / d;
-    }
+    if (lane == 0) v.rl[noff2 + I] = runs;
     len = runs;
 }
 
@@ -386,13 +384,12 @@ __device__ int coarse_row_warp(const BuildArgs &a, int64_t noff, int64_t noff2, 
     const int cnt = v.gc[noff2 + I];
     int32_t *own = v.own + noff + v.gs[noff2 + I];
     sort_members(own, cnt);
-    double ex = 0.0;
-    int done = 0;  // entries of the members before this batch of 32
+    double shift = 0.0;  // edges to nodes without coarse counterpart join the coarse excess
+    int done = 0;        // entries of the members before this batch of 32
     for (int m0 = 0; m0 < cnt; m0 += 32) {
         const int m = m0 + lane < cnt ? own[m0 + lane] : -1;
         const int len = m >= 0 ? v.rl[noff + m] : 0;
         const int64_t e0 = m >= 0 ? v.rs[noff + m] : 0;
-        if (m >= 0) ex += v.ex[noff + m];
         int incl = len;
         for (int o = 1; o < 32; o <<= 1) {
             const int t = __shfl_up_sync(0xffffffffu, incl, o);
@@ -407,9 +404,9 @@ __device__ int coarse_row_warp(const BuildArgs &a, int64_t noff, int64_t noff2, 
             const int before = __shfl_sync(0xffffffffu, incl - len, k);
             const int64_t e = __shfl_sync(0xffffffffu, e0, k) + (t - before);
             if (t < tot) {
-                const int J = a.agg[v.ecol[e]];
+                const int J = v.agg[noff + v.ecol[e]];
                 const double w = v.ew[e];
-                if (J < 0) ex += w;  // an edge to a node without coarse counterpart joins the shift
+                if (J < 0) shift += w;
                 keys[done + t] = (J < 0 || J == I) ? ~0ull
                                                    : (static_cast<unsigned long long>(static_cast<unsigned>(J)) << 32) |
                                                          static_cast<unsigned>(done + t);
@@ -418,20 +415,21 @@ __device__ int coarse_row_warp(const BuildArgs &a, int64_t noff, int64_t noff2, 
         }
         done += tot;
     }
-    ex = warp_sum(ex);
+    if (__any_sync(0xffffffffu, shift != 0.0)) shift = warp_sum(shift);
+    if (lane == 0) v.ex[noff2 + I] = shift;
     const int P = pow2_at_least(raw);
     for (int i = raw + lane; i < P; i += 32) keys[i] = ~0ull;
     __syncwarp();
     bitonic(keys, P, lane, 32, [] { __syncwarp(); });
     int len;
-    merge_row(v, noff2, I, keys, vals, raw, ex, len);
+    merge_row(v, noff2, I, keys, vals, raw, len);
     __syncwarp();
     return len;
 }
 
 // A wider coarse row (raw <= kBlockRaw), by the whole block.
 __device__ int coarse_row_block(const BuildArgs &a, int64_t noff, int64_t noff2, int I, int raw,
-                                unsigned long long *keys, double *vals, double *ex_sm) {
+                                unsigned long long *keys, double *vals) {
     const HierView &v = a.v;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     __syncthreads();
@@ -439,17 +437,16 @@ __device__ int coarse_row_block(const BuildArgs &a, int64_t noff, int64_t noff2,
         const int cnt = v.gc[noff2 + I];
         int32_t *own = v.own + noff + v.gs[noff2 + I];
         sort_members(own, cnt);
-        double ex = 0.0;
+        double shift = 0.0;
         int done = 0;
         for (int k = 0; k < cnt; ++k) {
             const int m = own[k];
             const int len = v.rl[noff + m];
             const int64_t e0 = v.rs[noff + m];
-            if (lane == 0) ex += v.ex[noff + m];
             for (int e = lane; e < len; e += 32) {
-                const int J = a.agg[v.ecol[e0 + e]];
+                const int J = v.agg[noff + v.ecol[e0 + e]];
                 const double w = v.ew[e0 + e];
-                if (J < 0) ex += w;
+                if (J < 0) shift += w;
                 keys[done + e] = (J < 0 || J == I) ? ~0ull
                                                    : (static_cast<unsigned long long>(static_cast<unsigned>(J)) << 32) |
                                                          static_cast<unsigned>(done + e);
@@ -457,33 +454,80 @@ __device__ int coarse_row_block(const BuildArgs &a, int64_t noff, int64_t noff2,
             }
             done += len;
         }
-        ex = warp_sum(ex);
-        if (lane == 0) *ex_sm = ex;
+        shift = warp_sum(shift);
+        if (lane == 0) v.ex[noff2 + I] = shift;
     }
     const int P = pow2_at_least(raw);
     for (int i = raw + threadIdx.x; i < P; i += blockDim.x) keys[i] = ~0ull;
     __syncthreads();
     bitonic(keys, P, threadIdx.x, blockDim.x, [] { __syncthreads(); });
     int len = 0;
-    if (wid == 0) merge_row(v, noff2, I, keys, vals, raw, *ex_sm, len);
+    if (wid == 0) merge_row(v, noff2, I, keys, vals, raw, len);
     __syncthreads();
     return len;  // valid in warp 0
+}
+
+// The coarse rows g0 .. g1 - 1, one warp each, the wide ones by the whole block;
+// then their diagonals.  Returns each warp's entries.
+__device__ int coarse_rows(const BuildArgs &a, int64_t noff, int64_t noff2, int g0, int g1, unsigned long long *keys,
+                           double *vals, int *s_count, int *s_wide) {
+    const HierView &v = a.v;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    int got = 0;
+    for (int base = g0; base < g1; base += kBuildThreads) {
+        const int cnt_here = min(kBuildThreads, g1 - base);
+        __syncthreads();
+        if (tid == 0) *s_count = 0;
+        __syncthreads();
+        for (int q = wid; q < cnt_here; q += kBuildThreads / 32) {
+            const int I = base + q;
+            const int raw = v.raw[noff2 + I];
+            if (raw <= kWarpRaw)
+                got += coarse_row_warp(a, noff, noff2, I, raw, keys + wid * kWarpRaw, vals + wid * kWarpRaw);
+            else if (lane == 0)
+                s_wide[atomicAdd(s_count, 1)] = I;
+        }
+        __syncthreads();
+        const int nwide = *s_count;
+        for (int q = 0; q < nwide; ++q) {
+            const int I = s_wide[q];
+            const int raw = v.raw[noff2 + I];
+            if (raw > kBlockRaw) {  // block-uniform
+                if (tid == 0) {
+                    v.rl[noff2 + I] = 0;
+                    v.ex[noff2 + I] = 1.0;
+                    atomicExch(&v.H->overflow, 1);
+                }
+                continue;
+            }
+            const int len = coarse_row_block(a, noff, noff2, I, raw, keys, vals);
+            if (wid == 0) got += len;
+        }
+    }
+    __syncthreads();
+    for (int I = g0 + tid; I < g1; I += kBuildThreads) {
+        double ex = v.ex[noff2 + I];
+        const int64_t o = noff + v.gs[noff2 + I];
+        for (int q = 0; q < v.gc[noff2 + I]; ++q) ex += v.ex[noff + v.own[o + q]];
+        finish_row(v, noff2 + I, ex, &a.partner[I]);
+    }
+    return got;
 }
 
 // ---- the coarsest level's inverse
 //
 // Elimination without subtractions: with weights w and excess ex the pivot is
-// ex_k + sum_{j > k} w_kj, and eliminating k adds w_ik w_kj / d_k to w_ij and
-// w_ik ex_k / d_k to ex_i -- sums of positive terms, so a shift of 1e-14 of the
-// weights keeps its relative precision.  L = (I - F) with F >= 0 gives
-// inv = sum_k M_k M_k^T / d_k, M = (I - F)^{-1}, again sums of positive terms.
+// d_k = ex_k + sum_{j > k} w_kj, and eliminating k adds f w_kj to w_ij and f ex_k
+// to ex_i, f = w_ik / d_k -- sums of positive terms, so a shift of 1e-14 of the
+// weights keeps its relative precision.  The same steps applied to the unit
+// matrix give M, and inv = sum_k M_k M_k^T / d_k, again sums of positive terms.
+// Row i holds w_ij for j above the pivot and M_ij below it, one warp per row and
+// one lane per column: only the rows below the pivot issue FP64 instructions.
 __device__ void dense_inverse(const HierView &v, int64_t noff, int n, double *sm) {
     double(*w)[kDense + 1] = reinterpret_cast<double(*)[kDense + 1]>(sm);
-    double(*M)[kDense + 1] = w + kDense;
-    double *ex = &M[kDense][0], *d = ex + kDense;
+    double *ex = &w[kDense][0], *dinv = ex + kDense;
     const int i = threadIdx.x >> 5, j = threadIdx.x & 31;  // kBuildThreads = kDense^2
     w[i][j] = 0.0;
-    M[i][j] = 0.0;
     __syncthreads();
     if (i < n) {
         const int64_t e0 = v.rs[noff + i];
@@ -493,34 +537,29 @@ __device__ void dense_inverse(const HierView &v, int64_t noff, int n, double *sm
     }
     __syncthreads();
     for (int k = 0; k < n; ++k) {
-        if (i == 0) {
-            double s = j > k && j < n ? w[k][j] : 0.0;
-            s = warp_sum(s);
-            if (j == 0) d[k] = ex[k] + s;
+        if (i == k) {
+            const double s = warp_sum(j > k && j < n ? w[k][j] : 0.0);
+            if (j == 0) dinv[k] = 1.0 / (ex[k] + s);
         }
         __syncthreads();
-        const double dk = d[k], wik = w[i][k], wkj = w[k][j], exk = ex[k];
-        __syncthreads();
-        if (i > k && i < n) {
-            const double f = wik / dk;
-            if (j > k && j < n && j != i) w[i][j] += f * wkj;
-            if (j == k) {
-                ex[i] += f * exk;
-                w[i][k] = f;  // F below the diagonal
-            }
+        if (i > k && i < n) {  // warp-uniform
+            const double f = w[i][k] * dinv[k];
+            __syncwarp();
+            if (j == k)
+                w[i][k] = f;
+            else if (j < n && j != i)
+                w[i][j] += f * w[k][j];
+            else if (j == i)
+                ex[i] += f * ex[k];
         }
         __syncthreads();
     }
-    if (i == 0)  // column j of M, by lane j
-        for (int r = 0; r < n; ++r) {
-            double s = r == j ? 1.0 : 0.0;
-            for (int k = j; k < r; ++k) s += w[r][k] * M[k][j];
-            if (j < n) M[r][j] = r >= j ? s : 0.0;
-        }
-    __syncthreads();
-    if (i < n && j < n) {
+    if (i < n && j < n) {  // M_ki for k > i, M_ii = 1
         double s = 0.0;
-        for (int k = max(i, j); k < n; ++k) s += M[k][i] * M[k][j] / d[k];
+        for (int k = max(i, j); k < n; ++k) {
+            const double mi = k == i ? 1.0 : w[k][i], mj = k == j ? 1.0 : w[k][j];
+            s += mi * mj * dinv[k];
+        }
         v.H->inv[i * kDense + j] = s;
     }
 }
@@ -535,7 +574,6 @@ template <int LPR> __global__ void __launch_bounds__(kBuildThreads, 1) k_amg_bui
     __shared__ int tmp[33];
     __shared__ int s_base[2];
     __shared__ unsigned long long s_ebase;
-    __shared__ double s_ex;
     __shared__ int s_wide[kBuildThreads];
     const HierView &v = a.v;
     Hier *H = v.H;
@@ -549,9 +587,27 @@ template <int LPR> __global__ void __launch_bounds__(kBuildThreads, 1) k_amg_bui
     {
         const int ch = (n + nb - 1) / nb;
         level0_values<LPR>(a, min(n, b * ch), min(n, (b + 1) * ch));
-        if (b == 0 && tid == 0) H->ecur = static_cast<unsigned long long>(a.e0);
+        if (b == 0 && tid == 0 && !a.same) H->ecur = static_cast<unsigned long long>(a.e0);
     }
     if (!bar.sync()) return;
+    if (a.same) {  // values alone, one pass per level
+        const int nlev = H->nlev;
+        for (int l = 0; l + 1 < nlev; ++l) {
+            const LevelInfo F = H->L[l], C = H->L[l + 1];
+            if (nb > 1 && !F.grid) {
+                if (b != 0) return;
+                nb = 1;
+                bar.nb = 1;
+            }
+            const int ch = (C.n + nb - 1) / nb;
+            const int g0 = min(C.n, b * ch), g1 = min(C.n, g0 + ch);
+            coarse_rows(a, F.noff, C.noff, g0, g1, keys, vals, &s_base[1], s_wide);
+            if (!bar.sync()) return;
+        }
+        const LevelInfo Z = H->L[nlev - 1];
+        if (b == 0 && H->dense) dense_inverse(v, Z.noff, Z.n, reinterpret_cast<double *>(smem));
+        return;
+    }
     int l = 0, sweeps = kLargeSweeps;
     for (;; ++l) {
         if (nb > 1 && nnz <= kBlockEntries && n <= kBlockNodes) {
@@ -565,17 +621,17 @@ template <int LPR> __global__ void __launch_bounds__(kBuildThreads, 1) k_amg_bui
             H->L[l].n = n;
             H->L[l].nmem = 0;
             H->L[l].nnz = nnz;
-            H->L[l].grid = l == 0 ? 1 : grid;
+            H->L[l].grid = grid;
         }
         if (!grid && l > 0) block_nodes += n;
         if (n <= kDense || l + 1 == kMaxLevels) break;
         const int ch = (n + nb - 1) / nb;
         const int i0 = min(n, b * ch), i1 = min(n, i0 + ch);
-        rank_round<LPR>(a, noff, n, i0, i1, 0, nullptr, a.best0);
+        rank_round<LPR>(a, noff, i0, i1, 0, nullptr, a.best0);
         if (!bar.sync()) return;
         int32_t *bp = a.best0, *bc = a.best1;
         for (int r = 1; r < kHandshakes; ++r) {
-            rank_round<LPR>(a, noff, n, i0, i1, r, bp, bc);
+            rank_round<LPR>(a, noff, i0, i1, r, bp, bc);
             if (!bar.sync()) return;
             int32_t *t = bp;
             bp = bc;
@@ -638,7 +694,7 @@ template <int LPR> __global__ void __launch_bounds__(kBuildThreads, 1) k_amg_bui
                 atomicAdd(&a.cnt[I], 1);
                 atomicAdd(&a.cap[I], v.rl[noff + i]);
             }
-            a.agg[i] = I;
+            v.agg[noff + i] = I;
         }
         if (!bar.sync()) return;
         // per block of coarse nodes: where their members and entries go
@@ -658,6 +714,7 @@ template <int LPR> __global__ void __launch_bounds__(kBuildThreads, 1) k_amg_bui
                 if (pass == 1 && I < g1) {
                     v.gs[noff2 + I] = s_base[0] + m + ca;
                     v.gc[noff2 + I] = c;
+                    v.raw[noff2 + I] = cp;
                     v.rs[noff2 + I] = static_cast<int64_t>(s_ebase) + e + ea;
                     a.cnt[I] = 0;  // from here on the members placed so far
                 }
@@ -687,42 +744,11 @@ template <int LPR> __global__ void __launch_bounds__(kBuildThreads, 1) k_amg_bui
         if (!bar.sync()) return;
         if (*reinterpret_cast<volatile int *>(&H->overflow)) break;  // the finer level stays the coarsest
         for (int i = i0 + tid; i < i1; i += kBuildThreads) {
-            const int I = a.agg[i];
+            const int I = v.agg[noff + i];
             if (I >= 0) v.own[noff + v.gs[noff2 + I] + atomicAdd(&a.cnt[I], 1)] = i;
         }
         if (!bar.sync()) return;
-        // coarse rows: one warp each, the wide ones by the whole block
-        int got = 0, nwide = 0;
-        for (int base = g0; base < g1; base += kBuildThreads) {
-            const int cnt_here = min(kBuildThreads, g1 - base);
-            __syncthreads();
-            if (tid == 0) s_base[1] = 0;
-            __syncthreads();
-            for (int q = wid; q < cnt_here; q += kBuildThreads / 32) {
-                const int I = base + q;
-                const int raw = a.cap[I];
-                if (raw <= kWarpRaw)
-                    got += coarse_row_warp(a, noff, noff2, I, raw, keys + wid * kWarpRaw, vals + wid * kWarpRaw);
-                else if (lane == 0)
-                    s_wide[atomicAdd(&s_base[1], 1)] = I;
-            }
-            __syncthreads();
-            nwide = s_base[1];
-            for (int q = 0; q < nwide; ++q) {
-                const int I = s_wide[q];
-                const int raw = a.cap[I];
-                if (raw > kBlockRaw) {  // block-uniform
-                    if (tid == 0) {
-                        v.rl[noff2 + I] = 0;
-                        v.dg[noff2 + I] = v.ex[noff2 + I] = v.om[noff2 + I] = 1.0;
-                        atomicExch(&H->overflow, 1);
-                    }
-                    continue;
-                }
-                const int len = coarse_row_block(a, noff, noff2, I, raw, keys, vals, &s_ex);
-                if (wid == 0) got += len;
-            }
-        }
+        const int got = coarse_rows(a, noff, noff2, g0, g1, keys, vals, &s_base[1], s_wide);
         if (lane == 0 && got) atomicAdd(&H->nnzacc[l + 1], static_cast<unsigned long long>(got));
         if (!bar.sync()) return;
         if (*reinterpret_cast<volatile int *>(&H->overflow)) break;
@@ -739,24 +765,29 @@ template <int LPR> __global__ void __launch_bounds__(kBuildThreads, 1) k_amg_bui
         H->nlev = l + 1;
         H->dense = dense;
         H->sweeps = sweeps;
-        if (l > 0 && nb > 1) H->L[l].grid = 1;
     }
 }
 
 // ---- host side
 
-int solve_grid(int64_t e0) {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (sms < 1) sms = 1;
-    if (sms > kMaxCtas) sms = kMaxCtas;
-    // one block per ~800 entries: the FP64 pipe takes about 1.7 products per
-    // clock and SM, so a pass then costs ~500 clocks against ~2 300 for the barrier
-    // after it; up to one block's worth of work needs no grid barrier at all
-    int64_t g = e0 / 800;
-    if (e0 <= 6000) g = 1;
-    return static_cast<int>(g < 1 ? 1 : (g > sms ? sms : g));
+// A finest level of at most this size is solved by one cluster: a pass of its
+// kSmallCluster blocks takes about 1 300 clocks plus 19 per FP64 warp instruction
+// (0.06 clocks per entry), one across the grid about 4 000.
+constexpr int64_t kSmallEntries = 40000;
+constexpr int64_t kSmallNodes = 4096;
+
+SolveShape solve_shape(bchar_mesh_t m) {
+    Amg &A = m->amg;
+    if (!A.resident) {
+        const int n = solve_blocks_resident();
+        A.resident = n > kMaxCtas ? kMaxCtas / kWideCluster * kWideCluster : n;
+    }
+    if (A.e0 <= kSmallEntries && A.n0 <= kSmallNodes) return {kSmallCluster, kSmallCluster, 1};
+    // one block per ~300 entries (two warps of rows), as many as the device holds
+    int64_t g = (A.e0 / 300 + kWideCluster - 1) / kWideCluster * kWideCluster;
+    if (g < 2 * kWideCluster) g = 2 * kWideCluster;
+    if (g > A.resident) g = A.resident;
+    return {static_cast<int>(g), kWideCluster, 0};
 }
 
 template <typename... P, typename... A>
@@ -791,12 +822,14 @@ HierView hier_view(bchar_mesh_t m) {
     v.own = ptr<int32_t>(A.own);
     v.gs = ptr<int32_t>(A.gs);
     v.gc = ptr<int32_t>(A.gc);
+    v.agg = ptr<int32_t>(A.agg);
+    v.raw = ptr<int32_t>(A.raw);
     v.ecol = ptr<int32_t>(A.ecol);
     v.ew = ptr<double>(A.ew);
     return v;
 }
 
-void amg_build(bchar_mesh_t m) {
+void amg_build(bchar_mesh_t m, bool same_aggregates) {
     Amg &A = m->amg;
     BuildArgs a{};
     a.v = hier_view(m);
@@ -815,19 +848,20 @@ void amg_build(bchar_mesh_t m) {
     a.cs = ptr<uint32_t>(A.cs);
     a.pair = ptr<int2>(A.pair);
     int32_t *s = ptr<int32_t>(A.scratch);
-    int32_t **dst[] = {&a.best0, &a.best1, &a.partner, &a.att, &a.lead, &a.pos, &a.agg, &a.cnt, &a.cap};
+    int32_t **dst[] = {&a.best0, &a.best1, &a.partner, &a.att, &a.lead, &a.pos, &a.cnt, &a.cap};
     for (int32_t **d : dst) {
         *d = s;
         s += A.n0;
     }
-    cudaMemsetAsync(A.hier.p, 0, offsetof(Hier, L), m->stream);
+    a.same = same_aggregates ? 1 : 0;
+    cudaMemsetAsync(A.hier.p, 0, same_aggregates ? offsetof(Hier, overflow) : offsetof(Hier, L), m->stream);
     static bool attrs = false;  // the shared-memory opt-in (harmless to repeat)
     if (!attrs) {
         cudaFuncSetAttribute(k_amg_build<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBuildSmem));
         cudaFuncSetAttribute(k_amg_build<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBuildSmem));
         attrs = true;
     }
-    const int grid = solve_grid(A.e0);
+    const int grid = solve_shape(m).grid;
     if (A.e0 <= 10 * A.n0)
         launch_cooperative(k_amg_build<4>, grid, kBuildThreads, kBuildSmem, m->stream, a);
     else
@@ -836,7 +870,7 @@ void amg_build(bchar_mesh_t m) {
 }
 
 void amg_release(Amg &A) {
-    Buf *all[] = {&A.hier, &A.seg, &A.rs, &A.rl, &A.dg, &A.ex, &A.om, &A.x, &A.b, &A.own, &A.gs, &A.gc, &A.ecol, &A.ew,
+    Buf *all[] = {&A.hier, &A.seg, &A.rs, &A.rl, &A.dg, &A.ex, &A.om, &A.x, &A.b, &A.own, &A.gs, &A.gc, &A.agg, &A.raw, &A.ecol, &A.ew,
                   &A.g, &A.t, &A.cs, &A.pair, &A.scratch, &A.raw_cnt, &A.raw_off, &A.raw_key, &A.vec, &A.stat};
     for (Buf *b : all) release(*b);
 }

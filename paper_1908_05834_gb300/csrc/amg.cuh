@@ -34,10 +34,13 @@ struct LevelInfo {
     int grid;       // 1: shared by all blocks, 0: block 0 alone
 };
 
-// Control block of the hierarchy and the solves, zeroed before every build.
+// Control block of the hierarchy and the solves.
 struct Hier {
+    // zeroed before every build
     unsigned bar[4];          // barrier counters: build, predictor solve, corrector solve, stage timing
     int err;                  // a barrier's wait ran out
+    int notier[3];            // per solve: the first cluster's levels do not fit its shared memory
+    // zeroed before a build with new aggregates
     int overflow;             // the entry arrays are full: coarsening stops
     unsigned long long ecur;  // entries in use
     unsigned mcur[kMaxLevels];
@@ -69,18 +72,25 @@ struct HierView {
     double *dg, *ex, *om, *x, *b;   // diagonal, excess, smoother weight, V-cycle vectors
     int32_t *own;                   // a level's nodes grouped by aggregate, then those without a coarse counterpart
     int32_t *gs, *gc;               // per coarse node: first member in the finer level's own, members
+    int32_t *agg, *raw;             // aggregate of each node (-1: none); entries of a coarse node's members
     int32_t *ecol;
     double *ew;                     // weights w > 0: the operator is diag - W
 };
 
-// Grid of the cooperative kernels for a finest level of e0 entries.
-int solve_grid(int64_t e0);
+// Shape of the cooperative kernels for the current finest level.
+struct SolveShape {
+    int grid, cluster, small;
+};
+constexpr int kWideCluster = 8;    // blocks per cluster of a solve across the grid
+constexpr int kSmallCluster = 16;  // of a solve by one cluster alone
+SolveShape solve_shape(bchar_mesh_t m);
+int solve_blocks_resident();  // pcg.cu
 
 // Once per step: the finest level's pattern (false: out of memory).
 bool schur_pattern(bchar_mesh_t m);
-// The hierarchy for the current weights (rebuilt every interior-point
-// iteration: they change by orders of magnitude).
-void amg_build(bchar_mesh_t m);
+// The hierarchy for the current weights; with same_aggregates the values alone,
+// on the aggregates of the build before.
+void amg_build(bchar_mesh_t m, bool same_aggregates);
 // One solve of the normal equations for m->rhs into m->cg_d; which = 0: from
 // zero, 1: from the finest level's solution left by solve 0.  The tolerances
 // are read on the device: z.res <= rz_rel mu, max |res_l| / b_l <=

@@ -102,11 +102,12 @@ struct Buf {
 // levels in shared arrays, the finest first.
 struct Amg {
     Buf hier, seg, stat;                                  // control block, blocks' shares, results
-    Buf rs, rl, dg, ex, om, x, b, own, gs, gc, ecol, ew;  // level arrays
+    Buf rs, rl, dg, ex, om, x, b, own, gs, gc, agg, raw, ecol, ew;  // level arrays
     Buf g, t, cs, pair, raw_cnt, raw_off, raw_key;        // the finest level's values from A's entries
     Buf scratch, vec;                                     // matching scratch; vectors of the conjugate gradients
     int64_t n0 = 0, e0 = 0;      // nodes and entries of the finest level
     int64_t capn = 0, cape = 0;  // room in the level arrays
+    int resident = 0;            // blocks of the solve kernel the device holds at once
     bool schur = false;          // finest level: the columns, rows eliminated (else rows and columns)
 };
 

@@ -239,11 +239,11 @@ bool schur_pattern(bchar_mesh_t m) {
     Buf *dbl[] = {&A.dg, &A.ex, &A.om, &A.x, &A.b};
     for (Buf *b : dbl)
         if (!ensure_more(m, *b, sizeof(double) * cn)) return false;
-    Buf *i32[] = {&A.rl, &A.own, &A.gs, &A.gc};
+    Buf *i32[] = {&A.rl, &A.own, &A.gs, &A.gc, &A.agg, &A.raw};
     for (Buf *b : i32)
         if (!ensure_more(m, *b, sizeof(int32_t) * cn)) return false;
-    if (!ensure_more(m, A.rs, sizeof(int64_t) * cn) || !ensure_more(m, A.scratch, sizeof(int32_t) * 9 * A.n0) ||
-        !ensure_more(m, A.vec, sizeof(double) * 6 * A.n0) || !ensure_more(m, A.g, sizeof(double) * (nnz > 0 ? nnz : 1)) ||
+    if (!ensure_more(m, A.rs, sizeof(int64_t) * cn) || !ensure_more(m, A.scratch, sizeof(int32_t) * 8 * A.n0) ||
+        !ensure_more(m, A.vec, sizeof(double) * 7 * A.n0) || !ensure_more(m, A.g, sizeof(double) * (nnz > 0 ? nnz : 1)) ||
         !ensure(m, A.t, sizeof(double) * nc))
         return false;
     if (A.schur) {

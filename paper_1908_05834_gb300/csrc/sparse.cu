@@ -1204,19 +1204,21 @@ bchar_status launch_minimise(bchar_mesh_t m, int *cg_iters, int *ip_iters) {
             cudaMemsetAsync(stat, 0, sizeof(SolveStat), s);
         }
         // normal-equation matrix and its preconditioner; the weights change by orders of
-        // magnitude between iterations, so the aggregates are built anew every time
+        // magnitude between iterations, so the aggregates are found anew
         const bool schur = use_amg && m->amg.schur;
         launch_dep(k_ip_weights, bl2, kThreads, s, nc, row_ptr, col_ptr, csc_src, a, brow, volphi, eps2, f, u, zl, zh, p,
                    n, zp, zn, D, ptr<double>(m->a2), ptr<double>(m->diag), ptr<double>(m->qexc),
                    schur ? ptr<double>(m->amg.g) : nullptr, schur ? ptr<double>(m->amg.t) : nullptr);
         k_qp_gather_cols<<<blocks_for(nnz), kThreads, 0, s>>>(nnz, csc_src, ptr<double>(m->a2), ptr<double>(m->a2c));
         m->launches += 2;
-        if (use_amg) amg_build(m);
+        if (use_amg) amg_build(m, false);
         // each direction solved until its squared energy-norm error is about <= 1e-2 mu (then
         // every entry's step error stays about <= 0.1 of its distance to the bound) and the
         // constraint residual it leaves is, relative to each target, <= 0.1 of the current
         // one (which the step then reduces), but not below half the stopping tolerance
-        const SolveTol tol{1e-2, 0.1, 0.5 * m->opt.qp_tol, kIpCgPerSolve, m->opt.qp_max_iter};
+        const double half = 0.5 * m->opt.qp_tol;
+        const SolveTol tols[2] = {{1e-2, 0.1, half, kIpCgPerSolve, m->opt.qp_max_iter},
+                                  {1e-2, 0.1, half, kIpCgPerSolve, m->opt.qp_max_iter}};
         cudaGraphExec_t exec = nullptr;
         int graph_launches = 0;
         for (int corr = 0; corr < 2; ++corr) {
@@ -1228,6 +1230,7 @@ bchar_status launch_minimise(bchar_mesh_t m, int *cg_iters, int *ip_iters) {
             // the corrector's system differs from the predictor's only in its right-hand
             // side (the centring and second-order terms): its solve starts from the
             // predictor's direction
+            const SolveTol &tol = tols[corr];
             if (use_amg) {
                 pcg_launch(m, corr, &st->mu, tol);
             } else {
