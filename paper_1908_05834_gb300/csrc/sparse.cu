@@ -1203,15 +1203,16 @@ bchar_status launch_minimise(bchar_mesh_t m, int *cg_iters, int *ip_iters) {
             solver_err = &ptr<Hier>(m->amg.hier)->err;
             cudaMemsetAsync(stat, 0, sizeof(SolveStat), s);
         }
-        // normal-equation matrix and its preconditioner; the weights change by orders of
-        // magnitude between iterations, so the aggregates are found anew
+        // normal-equation matrix and its preconditioner; the aggregates are found anew every
+        // other iteration (no effect on the CG iterations, where every third costs up to
+        // 30 % more of them: the weights change by orders of magnitude)
         const bool schur = use_amg && m->amg.schur;
         launch_dep(k_ip_weights, bl2, kThreads, s, nc, row_ptr, col_ptr, csc_src, a, brow, volphi, eps2, f, u, zl, zh, p,
                    n, zp, zn, D, ptr<double>(m->a2), ptr<double>(m->diag), ptr<double>(m->qexc),
                    schur ? ptr<double>(m->amg.g) : nullptr, schur ? ptr<double>(m->amg.t) : nullptr);
         k_qp_gather_cols<<<blocks_for(nnz), kThreads, 0, s>>>(nnz, csc_src, ptr<double>(m->a2), ptr<double>(m->a2c));
         m->launches += 2;
-        if (use_amg) amg_build(m, false);
+        if (use_amg) amg_build(m, it % 2 == 1);
         // the corrector's direction is solved until its squared energy-norm error is about
         // <= 1e-2 mu (then every entry's step error stays about <= 0.1 of its distance to the
         // bound) and the constraint residual it leaves is, relative to each target, <= half
