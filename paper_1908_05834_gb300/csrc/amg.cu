@@ -49,6 +49,7 @@
 #include "amg.cuh"
 #include "device.cuh"
 #include "gridbar.cuh"
+#include "ip.cuh"
 
 namespace bchar {
 
@@ -80,6 +81,7 @@ struct BuildArgs {
     const double *g, *t;                  // a2 / sqrt(diag_row) per entry; exc / diag per row
     const uint32_t *cs;                   // first contribution of each entry of the finest level
     const int2 *pair;                     // contributions: two entries of one row of A
+    IpArgs ip;
     int same;                             // 1: the aggregates of the build before
     int32_t *best0, *best1, *partner, *att, *lead, *pos, *cnt, *cap;  // n0 each
 };
@@ -566,7 +568,7 @@ __device__ void dense_inverse(const HierView &v, int64_t noff, int n, double *sm
 
 // ---- the build
 
-template <int LPR> __global__ void __launch_bounds__(kBuildThreads, 1) k_amg_build(BuildArgs a) {
+template <int LPR> __global__ void __launch_bounds__(kBuildThreads, 1) k_amg_build(const __grid_constant__ BuildArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned long long *keys = reinterpret_cast<unsigned long long *>(smem);
     double *vals = reinterpret_cast<double *>(smem + sizeof(unsigned long long) * kBlockRaw);
@@ -579,7 +581,26 @@ template <int LPR> __global__ void __launch_bounds__(kBuildThreads, 1) k_amg_bui
     Hier *H = v.H;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     int nb = gridDim.x, b = blockIdx.x;
-    GridBar bar(&H->bar[0], &H->err, gridDim.x);
+    GridBar bar(&H->bar[0], &a.ip.st->err, gridDim.x);
+    if (__syncthreads_or(a.ip.st->stop | a.ip.st->err)) return;
+    if (b == 0) {  // the control block's values, for this build (behind the weights' barrier) and the solves
+        if (!a.same && tid < kMaxLevels) {
+            H->mcur[tid] = 0;
+            H->nnzacc[tid] = 0;
+        }
+        if (tid == 0) {
+            if (!a.same) H->overflow = 0;
+            if (!a.same) H->ecur = static_cast<unsigned long long>(a.e0);
+            H->bar[1] = 0;
+            H->notier[0] = 0;
+        }
+    }
+    {
+        int64_t r0, r1;
+        ip_range(a.nc, b, nb, r0, r1);
+        if (!ip_weights(a.ip, bar, r0, r1)) return;
+    }
+    if (!bar.sync()) return;
 
     int n = a.n0;
     int64_t noff = 0, nnz = a.e0;
@@ -587,7 +608,6 @@ template <int LPR> __global__ void __launch_bounds__(kBuildThreads, 1) k_amg_bui
     {
         const int ch = (n + nb - 1) / nb;
         level0_values<LPR>(a, min(n, b * ch), min(n, (b + 1) * ch));
-        if (b == 0 && tid == 0 && !a.same) H->ecur = static_cast<unsigned long long>(a.e0);
     }
     if (!bar.sync()) return;
     if (a.same) {  // values alone, one pass per level
@@ -772,7 +792,10 @@ template <int LPR> __global__ void __launch_bounds__(kBuildThreads, 1) k_amg_bui
 
 // A finest level of at most this size is solved by one cluster: a pass of its
 // kSmallCluster blocks takes about 1 300 clocks plus 19 per FP64 warp instruction
-// (0.06 clocks per entry), one across the grid about 4 000.
+// (0.06 clocks per entry), one across the grid about 4 000.  Three more clusters
+// that share the passes over A's entries took 3 % off a 64^2 step alone, but a
+// batch of seven small meshes took 58 ms instead of 36: their launches no longer
+// fit side by side.
 constexpr int64_t kSmallEntries = 40000;
 constexpr int64_t kSmallNodes = 4096;
 
@@ -829,7 +852,7 @@ HierView hier_view(bchar_mesh_t m) {
     return v;
 }
 
-void amg_build(bchar_mesh_t m, bool same_aggregates) {
+void amg_build(bchar_mesh_t m, const IpArgs &ip, bool same_aggregates) {
     Amg &A = m->amg;
     BuildArgs a{};
     a.v = hier_view(m);
@@ -853,8 +876,8 @@ void amg_build(bchar_mesh_t m, bool same_aggregates) {
         *d = s;
         s += A.n0;
     }
+    a.ip = ip;
     a.same = same_aggregates ? 1 : 0;
-    cudaMemsetAsync(A.hier.p, 0, same_aggregates ? offsetof(Hier, overflow) : offsetof(Hier, L), m->stream);
     static bool attrs = false;  // the shared-memory opt-in (harmless to repeat)
     if (!attrs) {
         cudaFuncSetAttribute(k_amg_build<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBuildSmem));

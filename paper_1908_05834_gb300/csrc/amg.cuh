@@ -36,11 +36,9 @@ struct LevelInfo {
 
 // Control block of the hierarchy and the solves.
 struct Hier {
-    // zeroed before every build
-    unsigned bar[4];          // barrier counters: build, predictor solve, corrector solve, stage timing
-    int err;                  // a barrier's wait ran out
-    int notier[3];            // per solve: the first cluster's levels do not fit its shared memory
-    // zeroed before a build with new aggregates
+    unsigned bar[3];          // barrier counters: build (zeroed by the solves), solves (by the build), stage timing
+    int notier[2];            // (solves, stage timing) the first cluster's levels do not fit its shared memory
+    // set by a build with new aggregates
     int overflow;             // the entry arrays are full: coarsening stops
     unsigned long long ecur;  // entries in use
     unsigned mcur[kMaxLevels];
@@ -52,14 +50,6 @@ struct Hier {
     int ctasum[2][kMaxCtas];
     double part[4][kMaxCtas];
     double inv[kDense * kDense];
-};
-
-// The conjugate gradients' results (and the step's running iteration count).
-struct SolveStat {
-    double rz, res_max;
-    int iters, converged;
-    int total;  // all solves of the step
-    int err;
 };
 
 // The level arrays (device pointers), passed by value to the kernels.
@@ -81,6 +71,7 @@ struct HierView {
 struct SolveShape {
     int grid, cluster, small;
 };
+struct IpArgs;  // ip.cuh
 constexpr int kWideCluster = 8;    // blocks per cluster of a solve across the grid
 constexpr int kSmallCluster = 16;  // of a solve by one cluster alone
 SolveShape solve_shape(bchar_mesh_t m);
@@ -88,19 +79,18 @@ int solve_blocks_resident();  // pcg.cu
 
 // Once per step: the finest level's pattern (false: out of memory).
 bool schur_pattern(bchar_mesh_t m);
-// The hierarchy for the current weights; with same_aggregates the values alone,
-// on the aggregates of the build before.
-void amg_build(bchar_mesh_t m, bool same_aggregates);
-// One solve of the normal equations for m->rhs into m->cg_d; which = 0: from
-// zero, 1: from the finest level's solution left by solve 0.  The tolerances
-// are read on the device: z.res <= rz_rel mu, max |res_l| / b_l <=
-// max(res_rel rp_max, res_floor), with mu and rp_max at scal[0], scal[1].
+// An interior-point iteration: the weights of the normal equations and the
+// hierarchy for them; with same_aggregates the values alone, on the aggregates
+// of the build before.
+void amg_build(bchar_mesh_t m, const IpArgs &ip, bool same_aggregates);
+// Its predictor and corrector, the step and the residuals after it.  The
+// tolerances of the two solves: z.res <= rz_rel mu, max |res_l| / b_l <=
+// max(res_rel rp_max, res_floor).
 struct SolveTol {
     double rz_rel, res_rel, res_floor;
     int max_iter;   // of this solve
-    int max_total;  // of the step
 };
-void pcg_launch(bchar_mesh_t m, int which, const double *scal, const SolveTol &tol);
+void pcg_launch(bchar_mesh_t m, const IpArgs &ip, const SolveTol (&tol)[2]);
 void amg_release(Amg &amg);
 HierView hier_view(bchar_mesh_t m);
 // Timing aids: one damped-Jacobi sweep of the finest level; one V-cycle.

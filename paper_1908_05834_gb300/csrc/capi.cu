@@ -185,6 +185,8 @@ void bchar_destroy(bchar_mesh_t m) {
     release(m->rec);
     for (cudaEvent_t e : m->stage_ev)
         if (e) cudaEventDestroy(e);
+    for (cudaEvent_t e : m->ip_ev)
+        if (e) cudaEventDestroy(e);
     if (m->info_host.p) cudaFreeHost(m->info_host.p);
     amg_release(m->amg);
     delete m;
@@ -274,7 +276,7 @@ bchar_status bchar_create_mesh(int dim, const int64_t *n_cells, const double *co
          ensure(m, m->cg_z, sizeof(double) * 2 * nc) && ensure(m, m->cg_p, sizeof(double) * 2 * nc) &&
          ensure(m, m->cg_q, sizeof(double) * 2 * nc) && ensure(m, m->cg_rp, sizeof(double) * 2 * nc) && ensure(m, m->partials, sizeof(double) * 4 * 152 * 64) &&
          ensure(m, m->dinfo, sizeof(DevInfo)) && ensure(m, m->cg, sizeof(CgState));
-    if (ok && cudaMallocHost(&m->info_host.p, sizeof(DevInfo) + sizeof(CgState)) != cudaSuccess) {
+    if (ok && cudaMallocHost(&m->info_host.p, sizeof(DevInfo) + sizeof(CgState) + 2 * kIpScalarBytes) != cudaSuccess) {
         cudaGetLastError();
         m->info_host.p = nullptr;
         ok = false;

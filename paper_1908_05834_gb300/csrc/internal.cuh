@@ -91,6 +91,8 @@ struct CgState {
     int iters;
 };
 
+constexpr size_t kIpScalarBytes = 128;  // room of the interior point's scalars (ip.cuh)
+
 // A growable device buffer.
 struct Buf {
     void *p = nullptr;
@@ -163,7 +165,8 @@ struct bchar_mesh_s {
     // p - q, their multipliers, complementarity targets and a direction
     bchar::Buf ip_p, ip_n, ip_zp, ip_zn, ip_cp, ip_cn, ip_dp, ip_dn, ip_dzp, ip_dzn;
     bchar::Buf scan_tmp, partials, dinfo, cg, cg_rp; // scratch (cg_rp: previous residual of the flexible CG)
-    bchar::Buf info_host;                            // pinned DevInfo
+    bchar::Buf info_host;                            // pinned DevInfo, CgState, two IpScalars
+    cudaEvent_t ip_ev[2] = {};                       // the interior point's scalars have arrived (created on first use)
     bchar::Amg amg;                                  // preconditioner of the minimisation
     int64_t nnz = 0;
     int substeps = 1;

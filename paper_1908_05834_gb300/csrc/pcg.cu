@@ -34,6 +34,7 @@
 #include "amg.cuh"
 #include "device.cuh"
 #include "gridbar.cuh"
+#include "ip.cuh"
 
 namespace bchar {
 
@@ -65,11 +66,9 @@ struct PcgArgs {
     double *dy;                               // its solution
     double *d, *r, *p0, *p1, *q, *z, *ib;     // finest level; ib: 1 / target of each constraint
     const double *b_row, *volphi;
-    const double *scal;  // mu, rp_max
-    SolveTol tol;
-    int which;    // 0: from zero, 1: from d
-    int vcycle;   // 1: one V-cycle only (timing)
-    SolveStat *st;
+    IpArgs ip;
+    SolveTol tol[2];  // predictor (from zero), corrector (from the predictor's d)
+    int vcycle;       // 1: one V-cycle only (timing)
 };
 
 // ---------------------------------------------------------------- clusters
@@ -1056,7 +1055,8 @@ __device__ void tier_cycle(const Shared &sh, unsigned rank, unsigned nr) {
 
 // The right-hand side and the start's residual at row (id, its entries), in the
 // sign-flipped unknowns (+1 rows, -1 columns); LPR lanes share it.
-template <int LPR> __device__ double start_residual(const PcgArgs &a, const HierView &v, int id, int sub) {
+template <int LPR>
+__device__ double start_residual(const PcgArgs &a, const HierView &v, int which, int id, int sub) {
     double s = 0.0;
     if (a.schur) {
         for (int64_t q = a.col_ptr[id] + sub; q < a.col_ptr[id + 1]; q += LPR) {
@@ -1067,7 +1067,7 @@ template <int LPR> __device__ double start_residual(const PcgArgs &a, const Hier
     } else if (sub == 0) {
         s = id < a.nc ? a.rhs[id] : -a.rhs[id];
     }
-    if (a.which) {
+    if (which) {
         const int64_t e0 = v.rs[id];
         const int len = v.rl[id];
         for (int e = sub; e < len; e += LPR) s += v.ew[e0 + e] * a.d[v.ecol[e0 + e]];
@@ -1105,7 +1105,8 @@ __device__ __forceinline__ void invert_rz(Shared &sh) {
 
 // A system solved by one cluster: every level in its blocks' shared memory (the
 // finest one spread).  Returns the iterations.
-__device__ int solve_small(const PcgArgs &a, Shared &sh, unsigned rank, unsigned nr, double trz, double tres, int cap) {
+__device__ int solve_small(const PcgArgs &a, Shared &sh, unsigned rank, unsigned nr, int which, double trz, double tres,
+                           int cap) {
     const HierView &v = a.v;
     const View R = view(sh.lev[0]);
     const int tid = threadIdx.x;
@@ -1117,11 +1118,11 @@ __device__ int solve_small(const PcgArgs &a, Shared &sh, unsigned rank, unsigned
     const unsigned pstep = static_cast<unsigned>(cx) * 8u;
     for_items<8>(R.nrow, [&](bool ok, int sub, int k) {
         const int id = ok ? R.id[k] : 0;
-        const double s = start_residual<8>(a, v, id, sub);
+        const double s = start_residual<8>(a, v, which, id, sub);
         if (ok && sub == 0) {
             const double r = a.vcycle ? a.r[id] : s;
             ro[k] = r;
-            dd[k] = a.which ? a.d[id] : 0.0;
+            dd[k] = which ? a.d[id] : 0.0;
             qo[k] = 0.0;
             po[k] = 0.0;
             ibo[k] = inverse_target(a, id);
@@ -1302,7 +1303,7 @@ __device__ bool grid_cycle(const PcgArgs &a, Shared &sh, GridBar &bar, double *a
 }
 
 // A system shared by all blocks.  Returns the iterations, -1 when a barrier failed.
-__device__ int solve_grid_wide(const PcgArgs &a, Shared &sh, GridBar &bar, double trz, double tres, int cap) {
+__device__ int solve_grid_wide(const PcgArgs &a, Shared &sh, GridBar &bar, int which, double trz, double tres, int cap) {
     const HierView &v = a.v;
     Hier *H = v.H;
     const Rows &R = sh.lev[0];
@@ -1316,13 +1317,13 @@ __device__ int solve_grid_wide(const PcgArgs &a, Shared &sh, GridBar &bar, doubl
     for_items<8>(R.nrow, [&](bool ok, int sub, int k) {
         int id = 0;
         if (ok) id = here ? O.id[k] : any_row(v, R, k).id;
-        const double s = start_residual<8>(a, v, id, sub);
+        const double s = start_residual<8>(a, v, which, id, sub);
         if (ok && sub == 0) {
             const double r = a.vcycle ? a.r[id] : s, ib = inverse_target(a, id);
             a.p0[id] = 0.0;
             if (here) {
                 ro[k] = r;
-                dd[k] = a.which ? a.d[id] : 0.0;
+                dd[k] = which ? a.d[id] : 0.0;
                 qo[k] = 0.0;
                 po[k] = 0.0;
                 ibo[k] = ib;
@@ -1335,7 +1336,7 @@ __device__ int solve_grid_wide(const PcgArgs &a, Shared &sh, GridBar &bar, doubl
         }
     });
     if (!bar.sync()) return -1;
-    if (!here && !a.which && !a.vcycle)  // after the barrier: other rows' starts may read d
+    if (!here && !which && !a.vcycle)  // after the barrier: other rows' starts may read d
         for (int k = tid; k < R.nrow; k += kNT) a.d[any_row(v, R, k).id] = 0.0;
     double rz = 0.0, zq = 0.0;
     if (!grid_cycle(a, sh, bar, a.p1, rz, zq)) return -1;
@@ -1439,15 +1440,28 @@ __device__ __forceinline__ void own_vectors(Shared &sh, unsigned f, int n) {
     sh.ibo = f + 5 * s;
 }
 
-__global__ void __launch_bounds__(kSolveThreads, 1) k_pcg(PcgArgs a) {
+__global__ void __launch_bounds__(kSolveThreads, 1) k_pcg(const __grid_constant__ PcgArgs a) {
     __shared__ Shared sh;
     const HierView &v = a.v;
     Hier *H = v.H;
     const unsigned b = blockIdx.x, nb = gridDim.x;
     const unsigned rank = cluster_rank(), nr = cluster_size();
     const int tid = threadIdx.x;
-    GridBar bar(&H->bar[a.vcycle ? 3 : 1 + a.which], &H->err, nb);
-    if (__syncthreads_or(H->err)) return;  // an earlier barrier failed: nothing here can be relied on
+    const IpArgs &ip = a.ip;
+    GridBar bar(&H->bar[a.vcycle ? 2 : 1], &ip.st->err, nb);
+    // an earlier barrier failed: nothing here can be relied on; or the iterations have ended
+    if (__syncthreads_or(ip.st->err | (a.vcycle ? 0 : ip.st->stop))) return;
+    int *const notier = &H->notier[a.vcycle ? 1 : 0];
+    __shared__ IpShared ips;
+    int64_t r0, r1;
+    ip_range(ip.nc, b, nb, r0, r1);
+    const double mu = ip.st->mu, rp_max = ip.st->rp_max;
+    int cg = ip.st->cg;
+    const int done = ip.st->it;
+    if (!a.vcycle) {
+        if (b == 0 && tid == 0) H->bar[0] = 0;  // for the next build
+        ip_q<kIpLanes>(ip, r0, r1, 0, 0.0);
+    }
 
     // the levels: t0 is the first of the first cluster's (nlev: none), tr the first copied one
     if (tid == 0) {
@@ -1524,10 +1538,10 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_pcg(PcgArgs a) {
             }
         }
         __syncthreads();
-        if (!ok && tid == 0) atomicExch(&H->notier[a.vcycle ? 0 : 1 + a.which], 1);
+        if (!ok && tid == 0) atomicExch(notier, 1);
     }
     if (!bar.sync()) return;
-    if (*reinterpret_cast<volatile int *>(&H->notier[a.vcycle ? 0 : 1 + a.which])) {  // grid-uniform
+    if (*reinterpret_cast<volatile int *>(notier)) {  // grid-uniform
         if (tid == 0) sh.t0 = sh.nlev;
         p = 0;
         __syncthreads();
@@ -1568,43 +1582,44 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_pcg(PcgArgs a) {
         __syncthreads();
     }
 
-    const double trz = a.tol.rz_rel * a.scal[0];
-    const double tres = fmax(a.tol.res_rel * a.scal[1], a.tol.res_floor);
-    const int done_before = a.st->total;
-    const int cap = max(1, min(a.tol.max_iter, a.tol.max_total - done_before));
-    const int it = alone ? solve_small(a, sh, rank, nr, trz, tres, cap) : solve_grid_wide(a, sh, bar, trz, tres, cap);
-    if (it >= 0 && !a.vcycle) {
+    if (a.vcycle) {
+        alone ? solve_small(a, sh, rank, nr, 0, 0.0, 0.0, 1) : solve_grid_wide(a, sh, bar, 0, 0.0, 0.0, 1);
+        cluster_sync();
+        return;
+    }
+    ip_rhs<kIpLanes>(ip, r0, r1, 0, 0.0);
+    bool go = bar.sync();
+    for (int corr = 0; corr < 2 && go; ++corr) {
+        const SolveTol &tol = a.tol[corr];
+        const double trz = tol.rz_rel * mu, tres = fmax(tol.res_rel * rp_max, tol.res_floor);
+        const int cap = max(1, min(tol.max_iter, ip.max_cg - cg));
+        const int it = alone ? solve_small(a, sh, rank, nr, corr, trz, tres, cap)
+                             : solve_grid_wide(a, sh, bar, corr, trz, tres, cap);
+        cg += it;
+        go = it >= 0 && bar.sync();
+        if (!go) break;
         // back to the unknowns of rows and columns
-        bool go = true;
-        if (alone) {
-            __threadfence();
-            cluster_sync();
-        } else {
-            go = bar.sync();
-        }
-        if (go) {
-            if (a.schur) {
-                const int64_t ch = (a.nc + nb - 1) / nb;
-                const int64_t i0 = b * ch, i1 = i0 + ch < a.nc ? i0 + ch : a.nc;
-                for (int64_t i = i0 + tid; i < i1; i += kNT) {
-                    double s = a.rhs[i];
-                    for (int64_t e = a.row_ptr[i]; e < a.row_ptr[i + 1]; ++e) s += a.a2[e] * a.d[a.col[e]];
-                    a.dy[i] = s / a.diag[i];
-                    a.dy[a.nc + i] = -a.d[i];
-                }
-            } else {
-                const int64_t n = 2 * a.nc, ch = (n + nb - 1) / nb;
-                const int64_t i0 = b * ch, i1 = i0 + ch < n ? i0 + ch : n;
-                for (int64_t i = i0 + tid; i < i1; i += kNT) a.dy[i] = i < a.nc ? a.d[i] : -a.d[i];
+        if (a.schur)
+            ip_items<kIpLanes>(r0, r1, [&](bool ok, int sub, int64_t i) {
+                double s = 0.0;
+                if (ok)
+                    for (int64_t e = a.row_ptr[i] + sub; e < a.row_ptr[i + 1]; e += kIpLanes) s += a.a2[e] * a.d[a.col[e]];
+                s = ip_lanes<kIpLanes>(s);
+                if (ok && sub == 0) a.dy[i] = (a.rhs[i] + s) / a.diag[i];
+                if (ok && sub == 1) a.dy[a.nc + i] = -a.d[i];
+            });
+        else
+            for (int64_t i = r0 + tid; i < r1; i += kNT) {
+                a.dy[i] = a.d[i];
+                a.dy[a.nc + i] = -a.d[a.nc + i];
             }
-            if (b == 0 && tid == 0) {
-                a.st->rz = sh.rz;
-                a.st->res_max = sh.res_max;
-                a.st->iters = it;
-                a.st->converged = sh.conv;
-                a.st->total = done_before + it;
-            }
-        }
+        __syncthreads();
+        go = ip_steps(ip, bar, ips, r0, r1, a.d + (a.schur ? 0 : a.nc), -1.0);
+        if (go) go = corr ? ip_step(ip, bar, ips, r0, r1, cg, done + 1) : ip_corrector(ip, bar, ips, r0, r1) && bar.sync();
+    }
+    if (b == 0 && tid == 0) {
+        ip.st->levels = sh.nlev;
+        ip.st->coarsest = H->L[sh.nlev - 1].n;
     }
     cluster_sync();  // no block leaves while another may still store into its shared memory
 }
@@ -1648,7 +1663,6 @@ static PcgArgs pcg_args(bchar_mesh_t m) {
     }
     a.b_row = ptr<double>(m->bloc);
     a.volphi = ptr<double>(m->volphi);
-    a.st = ptr<SolveStat>(A.stat);
     return a;
 }
 
@@ -1701,21 +1715,21 @@ int solve_blocks_resident() {
     return n < 1 ? kWideCluster : n * kWideCluster;
 }
 
-void pcg_launch(bchar_mesh_t m, int which, const double *scal, const SolveTol &tol) {
+void pcg_launch(bchar_mesh_t m, const IpArgs &ip, const SolveTol (&tol)[2]) {
     PcgArgs a = pcg_args(m);
-    a.scal = scal;
-    a.tol = tol;
-    a.which = which;
+    a.ip = ip;
+    a.tol[0] = tol[0];
+    a.tol[1] = tol[1];
     launch_pcg(m, a);
 }
 
 void amg_vcycle_once(bchar_mesh_t m) {
     PcgArgs a = pcg_args(m);
-    a.scal = ptr<double>(m->partials);  // unused by a V-cycle
+    a.ip.st = ip_scalars(m);
     a.vcycle = 1;
     Hier *H = ptr<Hier>(m->amg.hier);
-    cudaMemsetAsync(&H->bar[3], 0, sizeof(unsigned), m->stream);
-    cudaMemsetAsync(&H->notier[0], 0, sizeof(int), m->stream);
+    cudaMemsetAsync(&H->bar[2], 0, sizeof(unsigned), m->stream);
+    cudaMemsetAsync(&H->notier[1], 0, sizeof(int), m->stream);
     launch_pcg(m, a);
 }
 

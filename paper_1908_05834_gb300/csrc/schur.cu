@@ -221,10 +221,10 @@ bool schur_pattern(bchar_mesh_t m) {
     const int64_t *row_ptr = ptr<int64_t>(m->row_ptr), *col_ptr = ptr<int64_t>(m->col_ptr);
     const int32_t *col = ptr<int32_t>(m->col), *csc_row = ptr<int32_t>(m->csc_row), *csc_src = ptr<int32_t>(m->csc_src);
     if (!ensure(m, A.hier, sizeof(Hier)) || !ensure(m, A.seg, sizeof(Seg) * kMaxLevels * kMaxCtas) ||
-        !ensure(m, A.stat, sizeof(SolveStat) + sizeof(PairStat)) || !ensure(m, A.raw_cnt, sizeof(int32_t) * nc) ||
+        !ensure(m, A.stat, sizeof(PairStat)) || !ensure(m, A.raw_cnt, sizeof(int32_t) * nc) ||
         !ensure(m, A.raw_off, sizeof(int64_t) * (nc + 1)))
         return false;
-    PairStat *st = reinterpret_cast<PairStat *>(ptr<SolveStat>(A.stat) + 1);
+    PairStat *st = ptr<PairStat>(A.stat);
     cudaMemsetAsync(st, 0, sizeof(PairStat), s);
     k_pair_counts<<<blocks_for(nc), kThreads, 0, s>>>(nc, row_ptr, col_ptr, csc_row, ptr<int32_t>(A.raw_cnt), st);
     ++m->launches;

@@ -17,12 +17,15 @@
 // All sums run in a fixed order (no floating-point atomics), so a step is
 // bitwise reproducible.
 #include <math.h>
+#include <stddef.h>
 #include <stdio.h>
 #include <stdlib.h>
+#include <string.h>
 #include <time.h>
 
 #include "amg.cuh"
 #include "device.cuh"
+#include "ip.cuh"
 #include "tiles.cuh"
 
 namespace bchar {
@@ -409,10 +412,6 @@ void launch_scaling_once(bchar_mesh_t m) {
 // step's pattern with edge weights a_e^2 D_e and that diagonal shift, by the
 // conjugate gradients below with the aggregation multigrid.
 
-__global__ void k_qp_gather_cols(int64_t nnz, const int32_t *csc_src, const double *a2, double *a2c) {
-    GRID_STRIDE(p, nnz) a2c[p] = a2[csc_src[p]];
-}
-
 // Preconditioned conjugate gradients on (A-hat A-hat^T + W) d = F.  Every
 // kernel returns at once when the solve has converged, so that batches of
 // iterations can be queued without reading the state back each time.
@@ -444,12 +443,6 @@ __global__ void k_dot(int64_t n, const double *a, const double *b, double *parti
     GRID_STRIDE(i, n) acc += a[i] * b[i];
     acc = block_sum(acc);
     if (threadIdx.x == 0) partials[blockIdx.x] = acc;
-}
-
-// The target b_l of constraint node l: |K_l|_phi-balanced row target for a
-// row node, |M_j|_phi for a column node.
-__device__ __forceinline__ double ip_target(int64_t nc, int64_t l, const double *b_row, const double *volphi) {
-    return l < nc ? b_row[l] : volphi[l - nc];
 }
 
 // Start of a solve: z.res of the initial residual, the two stopping targets
@@ -527,7 +520,7 @@ __global__ void k_cg_update(int64_t n2, const double *p, const double *q, double
         rp[l] = r0;
         const double r = r0 - alpha * q[l];
         res[l] = r;
-        mx = fmax(mx, fabs(r) / ip_target(nc, l, b_row, volphi));
+        mx = fmax(mx, fabs(r) / (l < nc ? b_row[l] : volphi[l - nc]));
     }
     mx = block_max(mx);
     if (threadIdx.x == 0) partials[blockIdx.x] = mx;
@@ -581,389 +574,46 @@ __global__ void k_cg_pupdate(int64_t n2, const double *z, double *p, const CgSta
     GRID_STRIDE(l, n2) p[l] = z[l] + beta * p[l];
 }
 
-// Scalars of one interior-point iteration, reduced over blocks (kRedBlocks
-// partial slots each) and read back once.
-struct IpScalars {
-    double mu;          // mean complementarity (the solves read it and rp_max, in this order)
-    double rp_max;      // max_l |rp_l| / b_l (the scaled constraint residual)
-    double rd_max;      // max_e |rd_e|
-    double rpq_max;     // max_l of the stationarity residuals of p and n
-    double dual_max;    // max(max_l |y_l| b_l, max zl, max zh)
-    double comp;        // sum of the complementarity products of all pairs
-    double rp_l1;       // sum_l |rp_l| (unscaled)
-    double ap, ad;      // largest primal / dual step to the boundary (<= 1)
-    double comp_aff;    // the same sum after the predictor's steps
-    double sigma_mu;    // the corrector's complementarity target
-    int err;            // a solver kernel's barrier failed
-};
+// Parts of an iteration as one cooperative kernel each: the start of the
+// minimisation, and the passes around solves that run as kernels of their own
+// (qp_precond = 0; with the multigrid an iteration is the two kernels of amg.cu
+// and pcg.cu).
+enum IpPart { kIpStart, kIpBegin, kIpMid, kIpEnd };
+constexpr int kIpThreads = 1024, kIpBlocks = 152;  // at 10^6 cells the loads in flight bound it
 
-constexpr int kIpSlots = 8;  // partial-sum slots per block in the reduction scratch
-
-__device__ __forceinline__ double ip_rd(double f, double zl, double zh, double gty) { return f - 1.0 - gty - zl + zh; }
-
-// Entry pass (thread per row): stationarity residuals rd and the entries'
-// complementarity sum; slots 0 (max |rd|), 1 (max multiplier), 2 (sum).
-__global__ void k_ip_entries(int64_t nc, const int64_t *row_ptr, const int32_t *col, const double *a,
-                             const double *y, const double *f, const double *u, const double *zl, const double *zh,
-                             double *part) {
-    dep_enter();
-    double rd_max = 0.0, comp = 0.0, zmax = 0.0;
-    GRID_STRIDE(i, nc) {
-        const double yi = y[i];
-        for (int64_t e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
-            rd_max = fmax(rd_max, fabs(ip_rd(f[e], zl[e], zh[e], a[e] * (yi + y[nc + col[e]]))));
-            comp += f[e] * zl[e] + u[e] * zh[e];
-            zmax = fmax(zmax, fmax(zl[e], zh[e]));
-        }
-    }
-    rd_max = block_max(rd_max);
-    zmax = block_max(zmax);
-    comp = block_sum(comp);
-    if (threadIdx.x == 0) {
-        double *pb = part + kIpSlots * blockIdx.x;
-        pb[0] = rd_max;
-        pb[1] = zmax;
-        pb[2] = comp;
+__global__ void __launch_bounds__(kIpThreads, 1) k_ip(const __grid_constant__ IpArgs A, int part, IpStart at) {
+    __shared__ IpShared S;
+    const unsigned b = blockIdx.x, nb = gridDim.x;
+    GridBar bar(&A.st->bar, &A.st->err, nb);
+    int64_t r0, r1;
+    ip_range(A.nc, b, nb, r0, r1);
+    const int done = A.st->it;
+    if (part == kIpStart) {
+        ip_check<true>(A, bar, S, r0, r1, 0, 0, at);
+    } else if (part == kIpBegin) {
+        if (!ip_weights(A, bar, r0, r1)) return;
+        ip_q<kIpLanes>(A, r0, r1, 0, 0.0);
+        if (bar.sync()) ip_rhs<kIpLanes>(A, r0, r1, 0, 0.0);
+    } else if (ip_steps(A, bar, S, r0, r1, A.dy + A.nc, 1.0)) {
+        if (part == kIpMid) ip_corrector(A, bar, S, r0, r1);
+        else ip_step(A, bar, S, r0, r1, 0, done + 1);
     }
 }
 
-// Node l: its constraint sum (row l by CSR, column l - n_c by CSC).
-__device__ __forceinline__ double ip_node_sum(int64_t nc, int64_t l, const int64_t *row_ptr, const int64_t *col_ptr,
-                                              const int32_t *csc_src, const double *a, const double *v) {
-    double s = 0.0;
-    if (l < nc) {
-        for (int64_t e = row_ptr[l]; e < row_ptr[l + 1]; ++e) s += a[e] * v[e];
-    } else {
-        for (int64_t k = col_ptr[l - nc]; k < col_ptr[l - nc + 1]; ++k) {
-            const int32_t e = csc_src[k];
-            s += a[e] * v[e];
-        }
-    }
-    return s;
-}
-
-// Node pass: constraint residual rp_l = b_l - (A-hat f)_l - eps^2 b_l^2 y_l - b_l (p_l - n_l),
-// the stationarity residuals gamma -+ b y - z of p and n, their complementarity;
-// slots 3 (max |rp| / b), 4 (max |rdp|, |rdn|), 5 (max |y| b), 6 (sum).
-__global__ void k_ip_nodes(int64_t nc, const int64_t *row_ptr, const int64_t *col_ptr, const int32_t *csc_src,
-                           const double *a, const double *b_row, const double *volphi, double eps2, double gamma,
-                           const double *y, const double *f, const double *p, const double *n, const double *zp,
-                           const double *zn, double *rp, double *part) {
-    dep_enter();
-    double rp_max = 0.0, rpq_max = 0.0, ymax = 0.0, comp = 0.0, rp_l1 = 0.0;
-    GRID_STRIDE(l, 2 * nc) {
-        const double bl = ip_target(nc, l, b_row, volphi);
-        const double ys = y[l] * bl;
-        const double r = bl - ip_node_sum(nc, l, row_ptr, col_ptr, csc_src, a, f) - eps2 * bl * ys - bl * (p[l] - n[l]);
-        rp[l] = r;
-        rp_l1 += fabs(r);
-        rp_max = fmax(rp_max, fabs(r) / bl);
-        rpq_max = fmax(rpq_max, fmax(fabs(gamma - ys - zp[l]), fabs(gamma + ys - zn[l])));
-        ymax = fmax(ymax, fabs(ys));
-        comp += p[l] * zp[l] + n[l] * zn[l];
-    }
-    rp_max = block_max(rp_max);
-    rpq_max = block_max(rpq_max);
-    ymax = block_max(ymax);
-    comp = block_sum(comp);
-    rp_l1 = block_sum(rp_l1);
-    if (threadIdx.x == 0) {
-        double *pb = part + kIpSlots * blockIdx.x;
-        pb[3] = rp_max;
-        pb[4] = rpq_max;
-        pb[5] = ymax;
-        pb[6] = comp;
-        pb[7] = rp_l1;
-    }
-}
-
-__global__ void k_ip_reduce_resid(const double *part, int nparts, double pairs, const int *solver_err, IpScalars *st) {
-    double rd = 0.0, rp = 0.0, rpq = 0.0, dm = 0.0, comp = 0.0, l1 = 0.0;
-    for (int k = threadIdx.x; k < nparts; k += blockDim.x) {
-        const double *pb = part + kIpSlots * k;
-        l1 += pb[7];
-        rd = fmax(rd, pb[0]);
-        dm = fmax(dm, fmax(pb[1], pb[5]));
-        comp += pb[2] + pb[6];
-        rp = fmax(rp, pb[3]);
-        rpq = fmax(rpq, pb[4]);
-    }
-    rd = block_max(rd);
-    rp = block_max(rp);
-    rpq = block_max(rpq);
-    dm = block_max(dm);
-    comp = block_sum(comp);
-    l1 = block_sum(l1);
-    if (threadIdx.x == 0) {
-        st->rp_l1 = l1;
-        st->rd_max = rd;
-        st->rp_max = rp;
-        st->rpq_max = rpq;
-        st->dual_max = dm;
-        st->comp = comp;
-        st->mu = comp / pairs;
-        st->err = solver_err ? *solver_err : 0;
-    }
-}
-
-// Normal-equation weights: D_e, a2_e = a_e^2 D_e, and per node
-// exc_l = b_l^2 (eps^2 + p_l / zp_l + n_l / zn_l) and diag_l = sum a^2 D + exc_l;
-// with g, t also the factors of the system with the rows eliminated,
-// g_e = a2_e / sqrt(diag_row) and t_row = exc_row / diag_row.
-__global__ void k_ip_weights(int64_t nc, const int64_t *row_ptr, const int64_t *col_ptr, const int32_t *csc_src,
-                             const double *a, const double *b_row, const double *volphi, double eps2,
-                             const double *f, const double *u, const double *zl, const double *zh, const double *p,
-                             const double *n, const double *zp, const double *zn, double *D, double *a2, double *diag,
-                             double *exc, double *g, double *t) {
-    dep_enter();
-    GRID_STRIDE(l, 2 * nc) {
-        double d = 0.0;
-        if (l < nc) {
-            for (int64_t e = row_ptr[l]; e < row_ptr[l + 1]; ++e) {
-                const double De = 1.0 / (1.0 + zl[e] / f[e] + zh[e] / u[e]);
-                D[e] = De;
-                a2[e] = a[e] * a[e] * De;
-                d += a2[e];
-            }
-        } else {
-            for (int64_t k = col_ptr[l - nc]; k < col_ptr[l - nc + 1]; ++k) {
-                const int32_t e = csc_src[k];
-                d += a[e] * a[e] / (1.0 + zl[e] / f[e] + zh[e] / u[e]);
-            }
-        }
-        const double bl = ip_target(nc, l, b_row, volphi);
-        const double x = bl * bl * (eps2 + p[l] / zp[l] + n[l] / zn[l]);
-        diag[l] = d + x;
-        exc[l] = x;
-        if (g && l < nc) {
-            const double w = 1.0 / sqrt(d + x);
-            for (int64_t e = row_ptr[l]; e < row_ptr[l + 1]; ++e) g[e] = a2[e] * w;
-            t[l] = x / (d + x);
-        }
-    }
-}
-
-// Reduced right-hand side per entry for the predictor (corrector = 0) or the
-// corrector (st->sigma_mu = sigma * mu, with the predictor's direction in df..dzh):
-//   cl = target of f zl, ch = target of u zh,
-//   q = -rd + cl / f - ch / u + (zh / u) ru.
-__global__ void k_ip_q(int64_t nc, const int64_t *row_ptr, const int32_t *col, const double *a, const double *y,
-                       const double *f, const double *u, const double *zl, const double *zh, int corrector,
-                       const IpScalars *st, const double *df, const double *du, const double *dzl, const double *dzh,
-                       double *cl, double *ch, double *q) {
-    dep_enter();
-    const double sigma_mu = corrector ? st->sigma_mu : 0.0;
-    GRID_STRIDE(i, nc) {
-        const double yi = y[i];
-        for (int64_t e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
-            const double fe = f[e], ue = u[e], zle = zl[e], zhe = zh[e];
-            const double rd = ip_rd(fe, zle, zhe, a[e] * (yi + y[nc + col[e]]));
-            const double ru = 2.0 - fe - ue;
-            double c_lo = -fe * zle, c_hi = -ue * zhe;
-            if (corrector) {
-                c_lo += sigma_mu - df[e] * dzl[e];
-                c_hi += sigma_mu - du[e] * dzh[e];
-            }
-            cl[e] = c_lo;
-            ch[e] = c_hi;
-            q[e] = -rd + c_lo / fe - c_hi / ue + (zhe / ue) * ru;
-        }
-    }
-}
-
-// Per node: the targets of p zp and n zn, and
-// rhs_l = rp_l - (A-hat (D q))_l - b_l (p/zp sp - n/zn sn),
-// sp = -(gamma - b y - zp) + cp / p, sn = -(gamma + b y - zn) + cn / n.
-__global__ void k_ip_rhs(int64_t nc, const int64_t *row_ptr, const int64_t *col_ptr, const int32_t *csc_src,
-                         const double *a, const double *D, const double *q, const double *rp, const double *b_row,
-                         const double *volphi, double gamma, const double *y, const double *p, const double *n,
-                         const double *zp, const double *zn, int corrector, const IpScalars *st, const double *dp,
-                         const double *dn, const double *dzp, const double *dzn, double *cp, double *cn, double *rhs) {
-    dep_enter();
-    const double sigma_mu = corrector ? st->sigma_mu : 0.0;
-    GRID_STRIDE(l, 2 * nc) {
-        double s = 0.0;
-        if (l < nc) {
-            for (int64_t e = row_ptr[l]; e < row_ptr[l + 1]; ++e) s += a[e] * D[e] * q[e];
-        } else {
-            for (int64_t k = col_ptr[l - nc]; k < col_ptr[l - nc + 1]; ++k) {
-                const int32_t e = csc_src[k];
-                s += a[e] * D[e] * q[e];
-            }
-        }
-        const double bl = ip_target(nc, l, b_row, volphi);
-        const double ys = y[l] * bl;
-        double c_p = -p[l] * zp[l], c_n = -n[l] * zn[l];
-        if (corrector) {
-            c_p += sigma_mu - dp[l] * dzp[l];
-            c_n += sigma_mu - dn[l] * dzn[l];
-        }
-        cp[l] = c_p;
-        cn[l] = c_n;
-        const double sp = -(gamma - ys - zp[l]) + c_p / p[l];
-        const double sn = -(gamma + ys - zn[l]) + c_n / n[l];
-        rhs[l] = rp[l] - s - bl * (p[l] / zp[l] * sp - n[l] / zn[l] * sn);
-    }
-}
-
-// Direction per entry from dy, and the ratio tests (largest steps <= 1 that
-// keep f, u, zl, zh positive), reduced per block as their reciprocals
-// max(1, -dv / v) into slots 0 (primal) and 1 (dual).
-__global__ void k_ip_dir(int64_t nc, const int64_t *row_ptr, const int32_t *col, const double *a, const double *dy,
-                         const double *f, const double *u, const double *zl, const double *zh, const double *D,
-                         const double *q, const double *cl, const double *ch, double *df, double *du, double *dzl,
-                         double *dzh, double *part) {
-    dep_enter();
-    double ap_inv = 1.0, ad_inv = 1.0;
-    GRID_STRIDE(i, nc) {
-        const double di = dy[i];
-        for (int64_t e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
-            const double fe = f[e], ue = u[e];
-            const double d_f = D[e] * (q[e] + a[e] * (di + dy[nc + col[e]]));
-            const double ru = 2.0 - fe - ue;
-            const double d_u = ru - d_f;
-            const double d_zl = (cl[e] - zl[e] * d_f) / fe;
-            const double d_zh = (ch[e] - zh[e] * d_u) / ue;
-            df[e] = d_f;
-            du[e] = d_u;
-            dzl[e] = d_zl;
-            dzh[e] = d_zh;
-            ap_inv = fmax(ap_inv, fmax(-d_f / fe, -d_u / ue));
-            ad_inv = fmax(ad_inv, fmax(-d_zl / zl[e], -d_zh / zh[e]));
-        }
-    }
-    ap_inv = block_max(ap_inv);  // block_max pads with 0: only for non-negative values
-    ad_inv = block_max(ad_inv);
-    if (threadIdx.x == 0) {
-        part[kIpSlots * blockIdx.x] = ap_inv;
-        part[kIpSlots * blockIdx.x + 1] = ad_inv;
-    }
-}
-
-// The same per node for p, n and their multipliers (dy scaled: b_l dy_l),
-// into slots 2 (primal) and 3 (dual).
-__global__ void k_ip_dir_nodes(int64_t nc, const double *b_row, const double *volphi, double gamma, const double *y,
-                               const double *dy, const double *p, const double *n, const double *zp, const double *zn,
-                               const double *cp, const double *cn, double *dp, double *dn, double *dzp, double *dzn,
-                               double *part) {
-    dep_enter();
-    double ap_inv = 1.0, ad_inv = 1.0;
-    GRID_STRIDE(l, 2 * nc) {
-        const double bl = ip_target(nc, l, b_row, volphi);
-        const double ys = y[l] * bl, dys = dy[l] * bl;
-        const double sp = -(gamma - ys - zp[l]) + cp[l] / p[l];
-        const double sn = -(gamma + ys - zn[l]) + cn[l] / n[l];
-        const double d_p = p[l] / zp[l] * (sp + dys);
-        const double d_n = n[l] / zn[l] * (sn - dys);
-        const double d_zp = (cp[l] - zp[l] * d_p) / p[l];
-        const double d_zn = (cn[l] - zn[l] * d_n) / n[l];
-        dp[l] = d_p;
-        dn[l] = d_n;
-        dzp[l] = d_zp;
-        dzn[l] = d_zn;
-        ap_inv = fmax(ap_inv, fmax(-d_p / p[l], -d_n / n[l]));
-        ad_inv = fmax(ad_inv, fmax(-d_zp / zp[l], -d_zn / zn[l]));
-    }
-    ap_inv = block_max(ap_inv);
-    ad_inv = block_max(ad_inv);
-    if (threadIdx.x == 0) {
-        part[kIpSlots * blockIdx.x + 2] = ap_inv;
-        part[kIpSlots * blockIdx.x + 3] = ad_inv;
-    }
-}
-
-__global__ void k_ip_reduce_steps(const double *part, int nparts, IpScalars *st) {
-    double ap_inv = 1.0, ad_inv = 1.0;
-    for (int k = threadIdx.x; k < nparts; k += blockDim.x) {
-        const double *pb = part + kIpSlots * k;
-        ap_inv = fmax(ap_inv, fmax(pb[0], pb[2]));
-        ad_inv = fmax(ad_inv, fmax(pb[1], pb[3]));
-    }
-    ap_inv = block_max(ap_inv);
-    ad_inv = block_max(ad_inv);
-    if (threadIdx.x == 0) {
-        st->ap = 1.0 / ap_inv;
-        st->ad = 1.0 / ad_inv;
-    }
-}
-
-// Complementarity after the predictor's steps to the boundary: entries into
-// slot 4, nodes into slot 5.
-__global__ void k_ip_comp_aff(int64_t nnz, int64_t n2, const double *f, const double *u, const double *zl,
-                              const double *zh, const double *df, const double *du, const double *dzl,
-                              const double *dzh, const double *p, const double *n, const double *zp, const double *zn,
-                              const double *dp, const double *dn, const double *dzp, const double *dzn,
-                              const IpScalars *st, double *part) {
-    dep_enter();
-    const double ap = st->ap, ad = st->ad;
-    double s = 0.0, t = 0.0;
-    GRID_STRIDE(e, nnz > n2 ? nnz : n2) {
-        if (e < nnz)
-            s += (f[e] + ap * df[e]) * (zl[e] + ad * dzl[e]) + (u[e] + ap * du[e]) * (zh[e] + ad * dzh[e]);
-        if (e < n2)
-            t += (p[e] + ap * dp[e]) * (zp[e] + ad * dzp[e]) + (n[e] + ap * dn[e]) * (zn[e] + ad * dzn[e]);
-    }
-    s = block_sum(s);
-    t = block_sum(t);
-    if (threadIdx.x == 0) {
-        part[kIpSlots * blockIdx.x + 4] = s;
-        part[kIpSlots * blockIdx.x + 5] = t;
-    }
-}
-
-// Mehrotra's centring target (comp_aff / comp)^3 mu, not below the floor.
-__global__ void k_ip_reduce_comp_aff(const double *part, int nparts, double mu_floor, IpScalars *st) {
-    double s = 0.0;
-    for (int k = threadIdx.x; k < nparts; k += blockDim.x) s += part[kIpSlots * k + 4] + part[kIpSlots * k + 5];
-    s = block_sum(s);
-    if (threadIdx.x == 0) {
-        const double r = s / st->comp;
-        st->comp_aff = s;
-        st->sigma_mu = fmax(fmin(1.0, r * r * r) * st->mu, mu_floor);
-    }
-}
-
-// Step with fraction 0.99 of the way to the boundary.
-__global__ void k_ip_update(int64_t nnz, int64_t n2, const IpScalars *st, double frac, const double *df,
-                            const double *du, const double *dzl, const double *dzh, const double *dy, const double *dp,
-                            const double *dn, const double *dzp, const double *dzn, double *f, double *u, double *zl,
-                            double *zh, double *y, double *p, double *n, double *zp, double *zn) {
-    dep_enter();
-    const double ap = frac * st->ap, ad = frac * st->ad;
-    GRID_STRIDE(e, nnz > n2 ? nnz : n2) {
-        if (e < nnz) {
-            f[e] += ap * df[e];
-            u[e] += ap * du[e];
-            zl[e] += ad * dzl[e];
-            zh[e] += ad * dzh[e];
-        }
-        if (e < n2) {
-            y[e] += ad * dy[e];
-            p[e] += ap * dp[e];
-            n[e] += ap * dn[e];
-            zp[e] += ad * dzp[e];
-            zn[e] += ad * dzn[e];
-        }
-    }
-}
-
-__global__ void k_ip_init(int64_t nnz, int64_t n2, double z0, double p0, double zp0, double *f, double *u,
-                          double *zl, double *zh, double *y, double *p, double *n, double *zp, double *zn) {
-    GRID_STRIDE(e, nnz > n2 ? nnz : n2) {
-        if (e < nnz) {
-            f[e] = 1.0;
-            u[e] = 1.0;
-            zl[e] = z0;
-            zh[e] = z0;
-        }
-        if (e < n2) {
-            y[e] = 0.0;
-            p[e] = p0;
-            n[e] = p0;
-            zp[e] = zp0;
-            zn[e] = zp0;
-        }
-    }
+static void launch_ip(bchar_mesh_t m, const IpArgs &A, IpPart part, const IpStart &start = IpStart{}) {
+    cudaMemsetAsync(&A.st->bar, 0, sizeof(unsigned), m->stream);
+    int64_t grid = (A.nc + 63) / 64;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(static_cast<unsigned>(grid < kIpBlocks ? (grid < 1 ? 1 : grid) : kIpBlocks));
+    cfg.blockDim = dim3(kIpThreads);
+    cfg.stream = m->stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_ip, A, static_cast<int>(part), start);
+    ++m->launches;
 }
 
 // x_e = f_e - 1 (kept in qx for the bounds / column-fix stage) and the count
@@ -1136,136 +786,129 @@ bchar_status launch_minimise(bchar_mesh_t m, int *cg_iters, int *ip_iters) {
                   &m->ip_dzp, &m->ip_dzn};
     for (Buf *b : nod)
         if (!ensure(m, *b, nb)) return BCHAR_ERR_OUT_OF_MEMORY;
-    static_assert(kIpSlots * kRedBlocks <= 152 * 64, "interior-point partials fit the first scratch section");
-    cudaStream_t s = m->stream;
-    const double eps2 = m->opt.penalty * m->opt.penalty;
-    const double gamma = kLinearFrom / eps2;
-    const int64_t *row_ptr = ptr<int64_t>(m->row_ptr), *col_ptr = ptr<int64_t>(m->col_ptr);
-    const int32_t *col = ptr<int32_t>(m->col), *csc_src = ptr<int32_t>(m->csc_src);
-    const double *a = ptr<double>(m->aN), *brow = ptr<double>(m->bloc), *volphi = ptr<double>(m->volphi);
-    double *f = ptr<double>(m->ip_f), *u = ptr<double>(m->ip_u), *zl = ptr<double>(m->ip_zl),
-           *zh = ptr<double>(m->ip_zh), *D = ptr<double>(m->ip_D), *q = ptr<double>(m->ip_q),
-           *cl = ptr<double>(m->ip_cl), *ch = ptr<double>(m->ip_ch), *df = ptr<double>(m->ip_df),
-           *du = ptr<double>(m->ip_du), *dzl = ptr<double>(m->ip_dzl), *dzh = ptr<double>(m->ip_dzh);
-    double *p = ptr<double>(m->ip_p), *n = ptr<double>(m->ip_n), *zp = ptr<double>(m->ip_zp),
-           *zn = ptr<double>(m->ip_zn), *cp = ptr<double>(m->ip_cp), *cn = ptr<double>(m->ip_cn),
-           *dp = ptr<double>(m->ip_dp), *dn = ptr<double>(m->ip_dn), *dzp = ptr<double>(m->ip_dzp),
-           *dzn = ptr<double>(m->ip_dzn);
-    double *y = ptr<double>(m->qy), *rp = ptr<double>(m->F), *rhs = ptr<double>(m->rhs), *dy = ptr<double>(m->cg_d);
-    double *part = ptr<double>(m->partials);
-    IpScalars *st = reinterpret_cast<IpScalars *>(ptr<CgState>(m->cg) + 1);
+    static_assert(5 * kMaxCtas <= 4 * 152 * 64, "interior-point partials fit the scratch");
     static_assert(sizeof(CgState) + sizeof(IpScalars) <= 256, "both scalar blocks fit the cg buffer");
-    IpScalars hs{};
-    const int blr = kRedBlocks;  // the entry and node passes are grid-stride over kRedBlocks blocks
-    const int bl2 = blocks_for(n2);
-    const int blm = blocks_for(nnz > n2 ? nnz : n2);
-    const double pairs = 2.0 * static_cast<double>(nnz) + 2.0 * static_cast<double>(n2);
+    cudaStream_t s = m->stream;
     const bool use_amg = m->opt.qp_precond == 1;
-    bool have_pattern = false;  // the finest level's pattern of this step
-    SolveStat *stat = nullptr, solve{};
-    const int *solver_err = nullptr;
-
-    k_ip_init<<<blm, kThreads, 0, s>>>(nnz, n2, kIpStartViol * gamma, kIpStartViol, gamma, f, u, zl, zh, y, p, n, zp,
-                                       zn);
-    ++m->launches;
-    int it = 0, total_cg = 0;
-    bool converged = false;
-    for (it = 0; it <= m->opt.qp_max_refine; ++it) {
-        launch_dep(k_ip_entries, blr, kThreads, s, nc, row_ptr, col, a, y, f, u, zl, zh, part);
-        launch_dep(k_ip_nodes, blr, kThreads, s, nc, row_ptr, col_ptr, csc_src, a, brow, volphi, eps2, gamma, y, f, p,
-                   n, zp, zn, rp, part);
-        k_ip_reduce_resid<<<1, 1024, 0, s>>>(part, blr, pairs, have_pattern ? solver_err : nullptr, st);
-        m->launches += 3;
-        cudaMemcpyAsync(&hs, st, sizeof hs, cudaMemcpyDeviceToHost, s);
-        if (have_pattern) cudaMemcpyAsync(&solve, stat, sizeof solve, cudaMemcpyDeviceToHost, s);
-        if (cudaStreamSynchronize(s) != cudaSuccess) break;  // the caller reads the error
-        if (cudaPeekAtLastError() != cudaSuccess) break;     // a launch failed: likewise
-        if (have_pattern) total_cg = solve.total;
-        if (hs.err) {
-            m->err = "a solver kernel's grid barrier timed out";
-            return BCHAR_ERR_CUDA;
-        }
-        const double mu = hs.mu;
-        if (trace)
+    const double eps2 = m->opt.penalty * m->opt.penalty;
+    IpArgs A{};
+    A.nc = nc;
+    A.nnz = nnz;
+    A.row_ptr = ptr<int64_t>(m->row_ptr);
+    A.col_ptr = ptr<int64_t>(m->col_ptr);
+    A.col = ptr<int32_t>(m->col);
+    A.csc_src = ptr<int32_t>(m->csc_src);
+    A.a = ptr<double>(m->aN);
+    A.b_row = ptr<double>(m->bloc);
+    A.volphi = ptr<double>(m->volphi);
+    A.eps2 = eps2;
+    A.gamma = kLinearFrom / eps2;
+    A.pairs = 2.0 * static_cast<double>(nnz) + 2.0 * static_cast<double>(n2);
+    A.mu_floor = kIpMuFloor;
+    A.step = kIpStep;
+    A.qp_tol = m->opt.qp_tol;
+    A.mu_tol = kIpMuTol;
+    A.rd_rel = kIpRdRel;
+    A.max_it = m->opt.qp_max_refine;
+    A.max_cg = m->opt.qp_max_iter;
+    double **ent_p[] = {&A.f, &A.u, &A.zl, &A.zh, &A.D, &A.q, &A.cl, &A.ch, &A.df, &A.du, &A.dzl, &A.dzh};
+    for (int k = 0; k < 12; ++k) *ent_p[k] = ptr<double>(*ent[k]);
+    double **nod_p[] = {&A.p, &A.n, &A.zp, &A.zn, &A.cp, &A.cn, &A.dp, &A.dn, &A.dzp, &A.dzn};
+    for (int k = 0; k < 10; ++k) *nod_p[k] = ptr<double>(*nod[k]);
+    A.y = ptr<double>(m->qy);
+    A.rp = ptr<double>(m->F);
+    A.rhs = ptr<double>(m->rhs);
+    A.dy = ptr<double>(m->cg_d);
+    A.a2 = ptr<double>(m->a2);
+    A.a2c = ptr<double>(m->a2c);
+    A.diag = ptr<double>(m->diag);
+    A.exc = ptr<double>(m->qexc);
+    A.part = ptr<double>(m->partials);
+    A.st = ip_scalars(m);
+    // the scalars after iteration k arrive in the host's copy k % 2
+    for (cudaEvent_t &e : m->ip_ev)
+        if (!e && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) e = nullptr;
+    unsigned char *const copies = static_cast<unsigned char *>(m->info_host.p) + sizeof(DevInfo) + sizeof(CgState);
+    auto read_back = [&](int k) {
+        cudaMemcpyAsync(copies + (k & 1) * kIpScalarBytes, A.st, sizeof(IpScalars), cudaMemcpyDeviceToHost, s);
+        cudaEventRecord(m->ip_ev[k & 1], s);
+    };
+    IpScalars hs{};
+    auto wait_for = [&](int k) {  // false: an error that the caller reads
+        const bool ok = cudaEventSynchronize(m->ip_ev[k & 1]) == cudaSuccess && cudaPeekAtLastError() == cudaSuccess;
+        memcpy(&hs, copies + (k & 1) * kIpScalarBytes, sizeof hs);
+        if (ok && trace)
             fprintf(stderr, "[bchar] ip %d rp %.3e rd %.3e rpq %.3e mu %.3e dual %.3e ap %.3e ad %.3e cg %d (%.1f ms)\n",
-                    it, hs.rp_max, hs.rd_max, hs.rpq_max, mu, hs.dual_max, hs.ap, hs.ad, total_cg,
-                    trace_ms() - t_start);
-        if (hs.rp_max <= m->opt.qp_tol && mu <= kIpMuTol && hs.rd_max <= kIpRdRel * (1.0 + hs.dual_max) &&
-            hs.rpq_max <= kIpRdRel * (1.0 + gamma)) {
-            converged = true;
-            break;
+                    hs.it, hs.rp_max, hs.rd_max, hs.rpq_max, hs.mu, hs.dual_max, hs.ap, hs.ad, hs.cg, trace_ms() - t_start);
+        return ok;
+    };
+    // the corrector's direction is solved until its squared energy-norm error is about
+    // <= 1e-2 mu (then every entry's step error stays about <= 0.1 of its distance to the
+    // bound) and the constraint residual it leaves is, relative to each target, <= half
+    // the current one (which the step then reduces), but not below half the stopping
+    // tolerance.  The predictor's only sets the centring and the second-order terms, and
+    // a thousand times looser it does that as well: 2 631 -> 1 999 CG iterations at 128^2
+    // stretched, 819 -> 559 on a porous 24^3 mesh, 279 -> 139 at 32^2, with at most one to
+    // three more interior-point iterations.  The corrector's system differs from the
+    // predictor's only in its right-hand side: its solve starts from the predictor's direction.
+    const double half = 0.5 * m->opt.qp_tol;
+    const SolveTol tols[2] = {{1e1, 5e2, 1e3 * half, kIpCgPerSolve}, {1e-2, 0.5, half, kIpCgPerSolve}};
+
+    cudaMemsetAsync(A.st, 0, sizeof(IpScalars), s);
+    launch_ip(m, A, kIpStart, {kIpStartViol * A.gamma, kIpStartViol, A.gamma});
+    read_back(0);
+    bool ok = wait_for(0), have_pattern = false;
+    int total_cg = 0;
+    if (ok && !hs.stop && !hs.err && use_amg) {
+        if (!schur_pattern(m)) return BCHAR_ERR_OUT_OF_MEMORY;
+        have_pattern = true;
+        cudaMemsetAsync(m->amg.hier.p, 0, offsetof(Hier, L), s);
+        if (m->amg.schur) {
+            A.g = ptr<double>(m->amg.g);
+            A.t = ptr<double>(m->amg.t);
         }
-        if (it == m->opt.qp_max_refine || total_cg >= m->opt.qp_max_iter) break;
-        if (use_amg && !have_pattern) {
-            if (!schur_pattern(m)) return BCHAR_ERR_OUT_OF_MEMORY;
-            have_pattern = true;
-            stat = ptr<SolveStat>(m->amg.stat);
-            solver_err = &ptr<Hier>(m->amg.hier)->err;
-            cudaMemsetAsync(stat, 0, sizeof(SolveStat), s);
+        // An iteration is queued before the scalars of the one before it are read, so that the
+        // device does not wait for the host; the kernels of one queued in vain return at once.
+        // The aggregates are found anew every other iteration (no effect on the CG iterations,
+        // where every third costs up to 30 % more of them: the weights change by orders of
+        // magnitude).
+        int queued = 0;
+        while (ok && !hs.stop && !hs.err) {
+            for (; queued < hs.it + 2 && queued < A.max_it; ++queued) {
+                amg_build(m, A, queued % 2 == 1);
+                pcg_launch(m, A, tols);
+                read_back(queued + 1);
+            }
+            ok = wait_for(hs.it + 1);
         }
-        // normal-equation matrix and its preconditioner; the aggregates are found anew every
-        // other iteration (no effect on the CG iterations, where every third costs up to
-        // 30 % more of them: the weights change by orders of magnitude)
-        const bool schur = use_amg && m->amg.schur;
-        launch_dep(k_ip_weights, bl2, kThreads, s, nc, row_ptr, col_ptr, csc_src, a, brow, volphi, eps2, f, u, zl, zh, p,
-                   n, zp, zn, D, ptr<double>(m->a2), ptr<double>(m->diag), ptr<double>(m->qexc),
-                   schur ? ptr<double>(m->amg.g) : nullptr, schur ? ptr<double>(m->amg.t) : nullptr);
-        k_qp_gather_cols<<<blocks_for(nnz), kThreads, 0, s>>>(nnz, csc_src, ptr<double>(m->a2), ptr<double>(m->a2c));
-        m->launches += 2;
-        if (use_amg) amg_build(m, it % 2 == 1);
-        // the corrector's direction is solved until its squared energy-norm error is about
-        // <= 1e-2 mu (then every entry's step error stays about <= 0.1 of its distance to the
-        // bound) and the constraint residual it leaves is, relative to each target, <= half
-        // the current one (which the step then reduces), but not below half the stopping
-        // tolerance.  The predictor's only sets the centring and the second-order terms, and
-        // a thousand times looser it does that as well: 2 631 -> 1 999 CG iterations at 128^2
-        // stretched, 819 -> 559 on a porous 24^3 mesh, 279 -> 139 at 32^2, with at most one to
-        // three more interior-point iterations.
-        const double half = 0.5 * m->opt.qp_tol;
-        const SolveTol tols[2] = {{1e1, 5e2, 1e3 * half, kIpCgPerSolve, m->opt.qp_max_iter},
-                                  {1e-2, 0.5, half, kIpCgPerSolve, m->opt.qp_max_iter}};
+        total_cg = hs.cg;
+    }
+    while (ok && !hs.stop && !hs.err && !use_amg) {
+        launch_ip(m, A, kIpBegin);
         cudaGraphExec_t exec = nullptr;
         int graph_launches = 0;
         for (int corr = 0; corr < 2; ++corr) {
-            launch_dep(k_ip_q, blr, kThreads, s, nc, row_ptr, col, a, y, f, u, zl, zh, corr, st, df, du, dzl, dzh, cl,
-                       ch, q);
-            launch_dep(k_ip_rhs, bl2, kThreads, s, nc, row_ptr, col_ptr, csc_src, a, D, q, rp, brow, volphi, gamma, y,
-                       p, n, zp, zn, corr, st, dp, dn, dzp, dzn, cp, cn, rhs);
-            m->launches += 2;
-            // the corrector's system differs from the predictor's only in its right-hand
-            // side (the centring and second-order terms): its solve starts from the
-            // predictor's direction
-            const SolveTol &tol = tols[corr];
-            if (use_amg) {
-                pcg_launch(m, corr, &st->mu, tol);
-            } else {
-                const int left = m->opt.qp_max_iter - total_cg;
-                const int cap = left < kIpCgPerSolve ? left : kIpCgPerSolve;
-                total_cg += pcg_solve(m, rhs, tol.rz_rel * mu, fmax(tol.res_rel * hs.rp_max, tol.res_floor), corr == 1,
-                                      cap > 0 ? cap : 1, &exec, &graph_launches);
-            }
-            launch_dep(k_ip_dir, blr, kThreads, s, nc, row_ptr, col, a, dy, f, u, zl, zh, D, q, cl, ch, df, du, dzl,
-                       dzh, part);
-            launch_dep(k_ip_dir_nodes, blr, kThreads, s, nc, brow, volphi, gamma, y, dy, p, n, zp, zn, cp, cn, dp, dn,
-                       dzp, dzn, part);
-            k_ip_reduce_steps<<<1, 1024, 0, s>>>(part, blr, st);
-            m->launches += 3;
-            if (!corr) {
-                launch_dep(k_ip_comp_aff, blr, kThreads, s, nnz, n2, f, u, zl, zh, df, du, dzl, dzh, p, n, zp, zn, dp,
-                           dn, dzp, dzn, st, part);
-                k_ip_reduce_comp_aff<<<1, 1024, 0, s>>>(part, blr, kIpMuFloor, st);
-                m->launches += 2;
-            }
+            const int left = m->opt.qp_max_iter - total_cg;
+            const int cap = left < kIpCgPerSolve ? left : kIpCgPerSolve;
+            total_cg += pcg_solve(m, A.rhs, 1e-2 * hs.mu, fmax(0.1 * hs.rp_max, half), corr == 1, cap > 0 ? cap : 1,
+                                  &exec, &graph_launches);
+            launch_ip(m, A, corr ? kIpEnd : kIpMid);
         }
         if (exec) cudaGraphExecDestroy(exec);
-        launch_dep(k_ip_update, blm, kThreads, s, nnz, n2, st, kIpStep, df, du, dzl, dzh, dy, dp, dn, dzp, dzn, f, u,
-                   zl, zh, y, p, n, zp, zn);
-        ++m->launches;
+        read_back(hs.it + 1);
+        ok = wait_for(hs.it + 1);
+        if (total_cg >= m->opt.qp_max_iter) break;
     }
-    k_ip_finish<<<blocks_for(nnz), kThreads, 0, s>>>(nnz, f, ptr<double>(m->qx), ptr<DevInfo>(m->dinfo));
+    if (hs.err) {
+        m->err = "a solver kernel's grid barrier timed out";
+        return BCHAR_ERR_CUDA;
+    }
+    const bool converged = hs.converged != 0;
+    const int it = hs.it;
+    k_ip_finish<<<blocks_for(nnz), kThreads, 0, s>>>(nnz, A.f, ptr<double>(m->qx), ptr<DevInfo>(m->dinfo));
     ++m->launches;
     DevInfo *di = ptr<DevInfo>(m->dinfo);
-    cudaMemcpyAsync(&di->kkt_l1, &st->rp_max, sizeof(double), cudaMemcpyDeviceToDevice, s);
+    cudaMemcpyAsync(&di->kkt_l1, &A.st->rp_max, sizeof(double), cudaMemcpyDeviceToDevice, s);
     if (trace) {
         cudaStreamSynchronize(s);
         fprintf(stderr, "[bchar] interior point: %d iterations, %d CG iterations, %s, %.3f ms\n", it, total_cg,
@@ -1275,19 +918,8 @@ bchar_status launch_minimise(bchar_mesh_t m, int *cg_iters, int *ip_iters) {
     m->ip_converged = converged;
     *cg_iters = total_cg;
     *ip_iters = it;
-    m->amg_levels = 0;
-    m->amg_coarsest = 0;
-    if (have_pattern) {
-        Hier *H = ptr<Hier>(m->amg.hier);
-        LevelInfo L[kMaxLevels];
-        int nlev = 0;
-        cudaMemcpyAsync(&nlev, &H->nlev, sizeof nlev, cudaMemcpyDeviceToHost, s);
-        cudaMemcpyAsync(L, H->L, sizeof L, cudaMemcpyDeviceToHost, s);
-        if (cudaStreamSynchronize(s) == cudaSuccess && nlev > 0 && nlev <= kMaxLevels) {
-            m->amg_levels = nlev;
-            m->amg_coarsest = L[nlev - 1].n;
-        }
-    }
+    m->amg_levels = have_pattern ? hs.levels : 0;
+    m->amg_coarsest = have_pattern ? hs.coarsest : 0;
     return BCHAR_OK;
 }
 
