@@ -29,23 +29,17 @@ __device__ __forceinline__ void relocate(const MeshView &m, int a, int &c, real 
     const int n = m.n[a];
 #pragma unroll 1
     for (int it = 0; it < 64; ++it) {  // one face per stage under the substep rule
-        if (xi >= real(1)) {
-            if (c >= n - 1) {
-                xi = real(1);
-                return;
-            }
-            xi = (xi - real(1)) * w[c] / w[c + 1];
-            ++c;
-        } else if (xi < real(0)) {
-            if (c <= 0) {
-                xi = real(0);
-                return;
-            }
-            xi = real(1) + xi * w[c] / w[c - 1];
-            --c;
-        } else {
+        const bool up = xi >= real(1);
+        if (!up && !(xi < real(0))) return;
+        // one path for both directions: the lanes of a warp that leave their cells share the division
+        const int cn = up ? c + 1 : c - 1;
+        if (cn < 0 || cn >= n) {
+            xi = up ? real(1) : real(0);
             return;
         }
+        const real t = (up ? xi - real(1) : xi) * w[c] / w[cn];
+        xi = up ? t : real(1) + t;
+        c = cn;
     }
     xi = xi < real(0) ? real(0) : (xi > real(1) ? real(1) : xi);
 }
@@ -69,6 +63,8 @@ template <> struct Stage<double> {
         wr[0] = e.x, wr[1] = e.y, wr[2] = f.x;
     }
     static __device__ __forceinline__ double per_phi(double u, double phi) { return u / phi; }
+    // acc + u / phi
+    static __device__ __forceinline__ double add_per_phi(double acc, double u, double phi) { return acc + u / phi; }
     // d over the width held in a record
     static __device__ __forceinline__ double by_width(double wr, double d) { return d / wr; }
 };
@@ -84,6 +80,9 @@ template <> struct Stage<float> {
         wr[0] = c.x, wr[1] = c.y, wr[2] = c.z;
     }
     static __device__ __forceinline__ float per_phi(float u, float inv_phi) { return u * inv_phi; }
+    static __device__ __forceinline__ float add_per_phi(float acc, float u, float inv_phi) {
+        return __fmaf_rn(u, inv_phi, acc);
+    }
     // d times the inverse width held in a record (the same value as m.wif)
     static __device__ __forceinline__ float by_width(float wr, float d) { return d * wr; }
 };
@@ -93,84 +92,70 @@ template <int DIM> __device__ __forceinline__ int64_t cell_of(const MeshView &m,
     return DIM == 2 ? c[0] + m.n[0] * c[1] : c[0] + m.n[0] * (c[1] + m.n[1] * c[2]);
 }
 
-// f = sign u(p) / phi(p) at the point (c, xi): one record load.  The axis
-// count is a template parameter so that every per-point array stays in
-// registers (all loops unroll).
+// su = sign u(p) at the point (c, xi) and the record's phi term (f = sign u / phi):
+// one record load.  The axis count is a template parameter so that every
+// per-point array stays in registers (all loops unroll).
 template <class real, int DIM>
 __device__ __forceinline__ void flow(const MeshView &m, const VelView &v, const int (&c)[3], const real (&xi)[3],
-                                     real sign, real (&f)[3]) {
+                                     real sign, real (&su)[3], real &phi) {
     real r[7];
     Stage<real>::load(v, cell_of<DIM>(m, c), r);
-    f[2] = real(0);
+    phi = r[6];
 #pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-        const real u = r[2 * a] + xi[a] * (r[2 * a + 1] - r[2 * a]);
-        f[a] = sign * Stage<real>::per_phi(u, r[6]);
-    }
+    for (int a = 0; a < DIM; ++a) su[a] = sign * (r[2 * a] + xi[a] * (r[2 * a + 1] - r[2 * a]));
 }
 
-// (c2, x2) = (c, xi) moved by the physical displacement s * k; wb holds the
-// width terms of cell c (from its record).
-template <class real, int DIM>
-__device__ __forceinline__ void moved(const MeshView &m, const int (&c)[3], const real (&xi)[3], real s,
-                                      const real (&k)[3], const real (&wb)[3], int (&c2)[3], real (&x2)[3]) {
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        c2[a] = c[a];
-        x2[a] = xi[a];
-    }
-#pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-        x2[a] = xi[a] + Stage<real>::by_width(wb[a], s * k[a]);
-        relocate<real>(m, a, c2[a], x2[a]);
-    }
-}
-
+// Bound by instruction issue (88 % of the slots on the porous 3D workload, FP32).
+// The four stages are unrolled: as one loop body, the selects between them cost
+// 12 to 16 % more time than the instruction cache gives back.  A move has one
+// path for both directions with one division; with two, and all 32 lanes of a
+// warp at work instead of 28, 7.1 million balls of seven points took 29.3 ms
+// over 37 substeps, now 22.7.
 template <class real, int DIM, int P>
-__device__ void rk4(const MeshView &m, const VelView &v, int (&c)[P][3], real (&xi)[P][3], real h, int substeps,
-                    real sign) {
-    const real half = real(0.5) * h;
+__device__ __forceinline__ void rk4(const MeshView &m, const VelView &v, int (&c)[P][3], real (&xi)[P][3], real h,
+                                    int substeps, real sign) {
+    const real half = real(0.5) * h, sixth = h / real(6);
+#pragma unroll 1
     for (int st = 0; st < substeps; ++st) {
-        real acc[P][3], k[P][3], x2[P][3], wb[P][3];
+        real acc[P][3], x2[P][3], wb[P][3];
         int c2[P][3];
 #pragma unroll
         for (int p = 0; p < P; ++p) {
-            flow<real, DIM>(m, v, c[p], xi[p], sign, k[p]);
             Stage<real>::load_widths(v, cell_of<DIM>(m, c[p]), wb[p]);
-        }
 #pragma unroll
-        for (int p = 0; p < P; ++p) {
-#pragma unroll
-            for (int a = 0; a < 3; ++a) acc[p][a] = k[p][a];
-            moved<real, DIM>(m, c[p], xi[p], half, k[p], wb[p], c2[p], x2[p]);
-        }
-#pragma unroll
-        for (int p = 0; p < P; ++p) flow<real, DIM>(m, v, c2[p], x2[p], sign, k[p]);
-#pragma unroll
-        for (int p = 0; p < P; ++p) {
-#pragma unroll
-            for (int a = 0; a < 3; ++a) acc[p][a] = acc[p][a] + real(2) * k[p][a];
-            moved<real, DIM>(m, c[p], xi[p], half, k[p], wb[p], c2[p], x2[p]);
-        }
-#pragma unroll
-        for (int p = 0; p < P; ++p) flow<real, DIM>(m, v, c2[p], x2[p], sign, k[p]);
-#pragma unroll
-        for (int p = 0; p < P; ++p) {
-#pragma unroll
-            for (int a = 0; a < 3; ++a) acc[p][a] = acc[p][a] + real(2) * k[p][a];
-            moved<real, DIM>(m, c[p], xi[p], h, k[p], wb[p], c2[p], x2[p]);
-        }
-#pragma unroll
-        for (int p = 0; p < P; ++p) flow<real, DIM>(m, v, c2[p], x2[p], sign, k[p]);
-#pragma unroll
-        for (int p = 0; p < P; ++p) {
-#pragma unroll
-            for (int a = 0; a < DIM; ++a) {
-                const real d = h / real(6) * (acc[p][a] + k[p][a]);
-                xi[p][a] = xi[p][a] + Stage<real>::by_width(wb[p][a], d);
-                relocate<real>(m, a, c[p][a], xi[p][a]);
+            for (int a = 0; a < 3; ++a) {
+                c2[p][a] = c[p][a];
+                x2[p][a] = xi[p][a];
+                acc[p][a] = real(0);
             }
         }
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            const real len = s < 2 ? half : (s == 2 ? h : sixth), wgt = s == 0 ? real(1) : real(2);
+            real su[P][3], phi[P];
+#pragma unroll
+            for (int p = 0; p < P; ++p) flow<real, DIM>(m, v, c2[p], x2[p], sign, su[p], phi[p]);
+#pragma unroll
+            for (int p = 0; p < P; ++p) {
+#pragma unroll
+                for (int a = 0; a < DIM; ++a) {
+                    // the last stage moves by h/6 (k1 + 2 k2 + 2 k3 + k4), the others by their own k
+                    const real k = Stage<real>::per_phi(su[p][a], phi[p]);
+                    const real d = len * (s < 3 ? k : Stage<real>::add_per_phi(acc[p][a], su[p][a], phi[p]));
+                    acc[p][a] = acc[p][a] + wgt * k;
+                    c2[p][a] = c[p][a];
+                    x2[p][a] = xi[p][a] + Stage<real>::by_width(wb[p][a], d);
+                    relocate<real>(m, a, c2[p][a], x2[p][a]);
+                }
+            }
+        }
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) {
+                c[p][a] = c2[p][a];
+                xi[p][a] = x2[p][a];
+            }
     }
 }
 
@@ -194,30 +179,79 @@ __device__ __forceinline__ void ball_start(const MeshView &m, int64_t b, int64_t
     for (int a = 0; a < DIM; ++a) xi0[a] = (real(sub[a]) + real(0.5)) / real(cnt[a]);
 }
 
-// phi constant: r_hat = r_K, only the centres move; each thread tracks
-// kBallsPerThread balls side by side (the last group repeats its last ball).
-constexpr int kBallsPerThread = 4;
+// The balls of a block's kGroupCells consecutive cells, by their number within
+// the cell and then by cell: the lanes of a warp track the same ball of
+// neighbouring cells, which cross faces at the same stages.  In ball order (the
+// balls of a cell side by side) the lanes diverged in almost every move, with 20
+// of 32 active in the mean; with both changes 5.3 million balls take 1.27 ms over
+// 20 substeps instead of 1.87.
+constexpr int kGroupCells = 32;
+constexpr int kListBalls = kGroupCells * kMaxBallsPerCell;  // a mesh with fuller cells is refused
+
+struct BallList {
+    int64_t first;  // first ball of the group
+    int total;
+    unsigned short at[kListBalls];  // list entry -> ball - first
+    // every thread of the block
+    __device__ void build(const MeshView &m) {
+        if (threadIdx.x < 32) {
+            const int lane = threadIdx.x;
+            const int64_t K0 = static_cast<int64_t>(blockIdx.x) * kGroupCells, K = K0 + lane;
+            const int64_t o0 = m.ball_off[K0];
+            const int64_t o = m.ball_off[K < m.nc ? K : m.nc];
+            const int n = static_cast<int>(m.ball_off[K + 1 < m.nc ? K + 1 : m.nc] - o);
+            int tot = n, most = n;
+            for (int d = 16; d > 0; d >>= 1) {
+                tot += __shfl_xor_sync(0xffffffffu, tot, d);
+                most = max(most, __shfl_xor_sync(0xffffffffu, most, d));
+            }
+            int base = 0;
+            for (int s = 0; s < most; ++s) {
+                const unsigned mask = __ballot_sync(0xffffffffu, n > s);
+                const int to = base + __popc(mask & ((1u << lane) - 1u));
+                if (n > s && to < kListBalls) at[to] = static_cast<unsigned short>(o - o0 + s);
+                base += __popc(mask);
+            }
+            if (lane == 0) {
+                first = o0;
+                total = min(tot, kListBalls);
+            }
+        }
+        __syncthreads();
+    }
+    __device__ int64_t ball(int i) const { return first + at[i]; }
+};
+static_assert(kGroupCells == 32, "a lane per cell");
+
+// phi constant: r_hat = r_K, only the centres move; a warp tracks chunks of
+// 32 kBallsPerThread balls, kBallsPerThread per lane side by side (past the end
+// of the list the last ball again).
+constexpr int kBallsPerThread = 2;
+constexpr int kCentreThreads = 128;
 
 template <class real, int DIM>
-__global__ void k_track_centres(MeshView m, VelView v, real h, int substeps, int64_t nballs, int32_t *out_cell,
-                                real *out_xi, real *out_rhat) {
-    const int64_t ngroups = (nballs + kBallsPerThread - 1) / kBallsPerThread;
-    for (int64_t g = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; g < ngroups;
-         g += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+__global__ void __launch_bounds__(kCentreThreads, sizeof(real) == 4 ? 7 : 4)
+    k_track_centres(MeshView m, VelView v, real h, int substeps, int32_t *out_cell, real *out_xi, real *out_rhat) {
+    __shared__ BallList list;
+    list.build(m);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    constexpr int W = kCentreThreads / 32;
+    for (int i0 = (static_cast<int>(blockIdx.y) * W + wid) * 32 * kBallsPerThread; i0 < list.total;
+         i0 += static_cast<int>(gridDim.y) * W * 32 * kBallsPerThread) {
         int c[kBallsPerThread][3];
         real xi[kBallsPerThread][3];
-        int64_t Ks[kBallsPerThread];
+        int64_t Ks[kBallsPerThread], bs[kBallsPerThread];
 #pragma unroll
         for (int p = 0; p < kBallsPerThread; ++p) {
-            int64_t b = g * kBallsPerThread + p;
-            if (b >= nballs) b = nballs - 1;
-            ball_start<real, DIM>(m, b, Ks[p], c[p], xi[p]);
+            const int i = i0 + p * 32 + lane;
+            bs[p] = list.ball(i < list.total ? i : list.total - 1);
+            ball_start<real, DIM>(m, bs[p], Ks[p], c[p], xi[p]);
         }
         rk4<real, DIM, kBallsPerThread>(m, v, c, xi, h, substeps, real(-1));
 #pragma unroll
         for (int p = 0; p < kBallsPerThread; ++p) {
-            const int64_t b = g * kBallsPerThread + p;
-            if (b >= nballs) break;
+            if (i0 + p * 32 + lane >= list.total) break;
+            const int64_t b = bs[p];
             out_cell[b] = static_cast<int32_t>(cell_of<DIM>(m, c[p]));
 #pragma unroll
             for (int a = 0; a < 3; ++a) out_xi[3 * b + a] = xi[p][a];
@@ -226,63 +260,56 @@ __global__ void k_track_centres(MeshView m, VelView v, real h, int substeps, int
     }
 }
 
-// phi varying: the centre and the 2 DIM axis points C +- r e_a of one ball
-// are tracked by 1 + 2 DIM adjacent lanes, one point per lane (a small
-// single-point RK4, so few registers and many warps per SM); the lanes then
-// exchange positions by shuffles and the centre's lane forms r_hat, the mean
-// distance, summing the axis points in order.
+// phi varying: the centre and the 2 DIM axis points C +- r e_a are tracked;
+// warp p of a block tracks point p of 32 consecutive balls (one point per lane: a
+// small single-point RK4, so few registers and many warps per SM, and all lanes
+// of every warp have a point), then the axis points' distances to the centres go
+// through shared memory to the centres' warp, which sums them in order.  The
+// points of a warp leave their cells at different stages in any order of the
+// balls; in this one they read few cells' records.
 template <class real, int DIM>
-__global__ void k_track_balls(MeshView m, VelView v, real h, int substeps, int64_t nballs, int32_t *out_cell,
-                              real *out_xi, real *out_rhat) {
-    constexpr int G = 1 + 2 * DIM;   // lanes (points) per ball
-    constexpr int PER_WARP = 32 / G;  // balls per warp
-    const int lane = threadIdx.x & 31;
-    const int g = lane / G, p = lane % G;
-    const int base = g * G;
-    const int64_t warp = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
-    const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-    const int64_t nw_needed = (nballs + PER_WARP - 1) / PER_WARP;
-    for (int64_t w = warp; w < nw_needed; w += nwarps) {  // warp-uniform loop
-        int64_t b = w * PER_WARP + g;
-        const bool valid = g < PER_WARP && b < nballs;
-        if (!valid) b = nballs - 1;  // idle lanes track a copy and write nothing
+__global__ void __launch_bounds__(32 * (1 + 2 * DIM), (sizeof(real) == 4 ? 1400 : 900) / (32 * (1 + 2 * DIM)))
+    k_track_balls(MeshView m, VelView v, real h, int substeps, int64_t nballs, int32_t *out_cell, real *out_xi,
+                  real *out_rhat) {
+    constexpr int G = 1 + 2 * DIM;  // points per ball
+    __shared__ double cen[3][32], dist[G][32];
+    const int lane = threadIdx.x & 31, p = threadIdx.x >> 5;
+    for (int64_t i0 = static_cast<int64_t>(blockIdx.x) * 32; i0 < nballs; i0 += static_cast<int64_t>(gridDim.x) * 32) {
+        const bool valid = i0 + lane < nballs;
+        const int64_t b = valid ? i0 + lane : nballs - 1;  // idle lanes track a copy and write nothing
         int64_t K;
-        int c0[3];
-        real xi0[3];
-        ball_start<real, DIM>(m, b, K, c0, xi0);
-        const real r = Real<real>::rad(m, K);
-        int c[1][3] = {{c0[0], c0[1], c0[2]}};
-        real xi[1][3] = {{xi0[0], xi0[1], xi0[2]}};
+        int c[1][3];
+        real xi[1][3];
+        ball_start<real, DIM>(m, b, K, c[0], xi[0]);
         {  // point p > 0: axis (p - 1) / 2, sign - for odd p, + for even p
+            const real r = Real<real>::rad(m, K);
             const real sg = (p & 1) ? real(-1) : real(1);
 #pragma unroll
             for (int q = 0; q < DIM; ++q)
-                if (p > 0 && (p - 1) / 2 == q) xi[0][q] = xi0[q] + sg * r / Real<real>::w(m, q)[c0[q]];
+                if (p > 0 && (p - 1) / 2 == q) xi[0][q] = xi[0][q] + sg * r / Real<real>::w(m, q)[c[0][q]];
         }
         rk4<real, DIM, 1>(m, v, c, xi, h, substeps, real(-1));
         double pos[3] = {0.0, 0.0, 0.0};
 #pragma unroll
         for (int q = 0; q < DIM; ++q) pos[q] = position<real>(m, q, c[0][q], xi[0][q]);
-        double cen[3] = {0.0, 0.0, 0.0};
+        if (p == 0)
 #pragma unroll
-        for (int q = 0; q < DIM; ++q) cen[q] = __shfl_sync(0xffffffffu, pos[q], base < 32 ? base : 0);
-        double dist = 0.0;
-        {
+            for (int q = 0; q < DIM; ++q) cen[q][lane] = pos[q];
+        __syncthreads();
+        if (p > 0) {
             double d2 = 0.0;
 #pragma unroll
             for (int q = 0; q < DIM; ++q) {
-                const double dq = pos[q] - cen[q];
+                const double dq = pos[q] - cen[q][lane];
                 d2 += dq * dq;
             }
-            dist = sqrt(d2);
+            dist[p][lane] = sqrt(d2);
         }
-        double sum = 0.0;
+        __syncthreads();
+        if (p == 0 && valid) {
+            double sum = 0.0;
 #pragma unroll
-        for (int q = 1; q < G; ++q) {
-            const int src = base + q < 32 ? base + q : 0;
-            sum += __shfl_sync(0xffffffffu, dist, src);
-        }
-        if (valid && p == 0) {
+            for (int q = 1; q < G; ++q) sum += dist[q][lane];
             out_cell[b] = static_cast<int32_t>(cell_of<DIM>(m, c[0]));
 #pragma unroll
             for (int a = 0; a < 3; ++a) out_xi[3 * b + a] = xi[0][a];
@@ -298,21 +325,22 @@ template <class real>
 static void track_in(bchar_mesh_t m, real h, int substeps, int32_t *cell, real *xi, real *rhat) {
     MeshView mv = full_view(m);
     VelView vv = vel_view(m);
+    const int64_t most = 0x7fffffff, n32 = (m->nballs + 31) / 32;
+    const unsigned chunks = static_cast<unsigned>(n32 < 1 ? 1 : (n32 > most ? most : n32));
     if (m->phi_const) {
-        const int64_t groups = (m->nballs + kBallsPerThread - 1) / kBallsPerThread;
+        // a block column per group of cells, and as many blocks per group as it has chunks in the mean
+        const unsigned groups = static_cast<unsigned>((m->nc + kGroupCells - 1) / kGroupCells);
+        const int64_t chunk = kCentreThreads * kBallsPerThread, y = ((m->nballs + groups - 1) / groups + chunk - 1) / chunk;
+        const dim3 grid(groups, static_cast<unsigned>(y < 1 ? 1 : (y > 64 ? 64 : y)));
         if (m->dim == 2)
-            k_track_centres<real, 2><<<blocks_for(groups, 128), 128, 0, m->stream>>>(mv, vv, h, substeps, m->nballs,
-                                                                                      cell, xi, rhat);
+            k_track_centres<real, 2><<<grid, kCentreThreads, 0, m->stream>>>(mv, vv, h, substeps, cell, xi, rhat);
         else
-            k_track_centres<real, 3><<<blocks_for(groups, 128), 128, 0, m->stream>>>(mv, vv, h, substeps, m->nballs,
-                                                                                      cell, xi, rhat);
-    } else if (m->dim == 2) {  // 6 balls per warp
-        const int64_t threads = (m->nballs + 5) / 6 * 32;
-        k_track_balls<real, 2><<<blocks_for(threads, 128), 128, 0, m->stream>>>(mv, vv, h, substeps, m->nballs, cell,
+            k_track_centres<real, 3><<<grid, kCentreThreads, 0, m->stream>>>(mv, vv, h, substeps, cell, xi, rhat);
+    } else if (m->dim == 2) {
+        k_track_balls<real, 2><<<chunks, 160, 0, m->stream>>>(mv, vv, h, substeps, m->nballs, cell,
                                                                                   xi, rhat);
-    } else {  // 4 balls per warp
-        const int64_t threads = (m->nballs + 3) / 4 * 32;
-        k_track_balls<real, 3><<<blocks_for(threads, 128), 128, 0, m->stream>>>(mv, vv, h, substeps, m->nballs, cell,
+    } else {
+        k_track_balls<real, 3><<<chunks, 224, 0, m->stream>>>(mv, vv, h, substeps, m->nballs, cell,
                                                                                   xi, rhat);
     }
     ++m->launches;
