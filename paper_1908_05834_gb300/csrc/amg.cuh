@@ -13,11 +13,12 @@ constexpr int kSolveThreads = 512;   // threads per block of the conjugate gradi
 constexpr int kBuildThreads = 1024;  // threads per block of the hierarchy build
 constexpr int kDense = 32;           // a coarsest level of at most this many nodes is solved by its inverse
 
-// Levels of at most this many off-diagonal entries and nodes are built and
-// cycled by block 0 alone, between block barriers, from shared memory.
-constexpr int kBlockEntries = 4000;
+// Levels of at most this many off-diagonal entries and nodes are built by block 0
+// alone, between block barriers.  (At 4 000 the first such level took it 33 us for
+// the values and 52 in full, against 9 and 35 for a level across the grid.)
+constexpr int kBlockEntries = 1200;
 constexpr int kBlockNodes = 1500;
-constexpr int kBlockTotalNodes = 2600;  // nodes of all such levels (their vectors must fit shared memory)
+constexpr int kBlockTotalNodes = 2600;  // nodes of all such levels at most
 
 // Where one block's share of a level is: its rows (the members of its
 // aggregates, in aggregate order, then its nodes without a coarse counterpart)

@@ -21,6 +21,8 @@ namespace bchar {
 
 constexpr int kWarpPairs = 512;    // contributions of a column sorted by one warp
 constexpr int kBlockPairs = 8192;  // by one block
+static_assert(kWarpPairs >= 32 && (kWarpPairs & (kWarpPairs - 1)) == 0 && (kBlockPairs & (kBlockPairs - 1)) == 0,
+              "the sorts pad to a power of two of at least 32");
 // S then holds about six entries per entry of A where the product through the
 // two views touches two; the recipes' matrices have 1.5 to 8.
 constexpr int64_t kMaxPairs = 12;
