@@ -523,8 +523,8 @@ __device__ int coarse_rows(const BuildArgs &a, int64_t noff, int64_t noff2, int 
 // to ex_i, f = w_ik / d_k -- sums of positive terms, so a shift of 1e-14 of the
 // weights keeps its relative precision.  The same steps applied to the unit
 // matrix give M, and inv = sum_k M_k M_k^T / d_k, again sums of positive terms
-(its lower triangle, with the division folded into one factor: a third of the
-FP64 instructions, 10 of the 25 us that 32 nodes took).
+// (its lower triangle, with the division folded into one factor: a third of the
+// FP64 instructions, 10 of the 25 us that 32 nodes took).
 // Row i holds w_ij for j above the pivot and M_ij below it, one warp per row and
 // one lane per column: only the rows below the pivot issue FP64 instructions.
 __device__ void dense_inverse(const HierView &v, int64_t noff, int n, double *sm) {
