@@ -571,7 +571,8 @@ __device__ void dense_inverse(const HierView &v, int64_t noff, int n, double *sm
 
 // ---- the build
 
-template <int LPR> __global__ void __launch_bounds__(kBuildThreads, 1) k_amg_build(const __grid_constant__ BuildArgs a) {
+// ONE: the grid is one cluster.
+template <int LPR, bool ONE> __global__ void __launch_bounds__(kBuildThreads, 1) k_amg_build(const __grid_constant__ BuildArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned long long *keys = reinterpret_cast<unsigned long long *>(smem);
     double *vals = reinterpret_cast<double *>(smem + sizeof(unsigned long long) * kBlockRaw);
@@ -584,7 +585,7 @@ template <int LPR> __global__ void __launch_bounds__(kBuildThreads, 1) k_amg_bui
     Hier *H = v.H;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     int nb = gridDim.x, b = blockIdx.x;
-    GridBar bar(&H->bar[0], &a.ip.st->err, gridDim.x);
+    GridBarT<ONE> bar(&H->bar[0], &a.ip.st->err, gridDim.x);
     if (__syncthreads_or(a.ip.st->stop | a.ip.st->err)) return;
     if (b == 0) {  // the control block's values, for this build (behind the weights' barrier) and the solves
         if (!a.same && tid < kMaxLevels) {
@@ -596,6 +597,7 @@ template <int LPR> __global__ void __launch_bounds__(kBuildThreads, 1) k_amg_bui
             if (!a.same) H->ecur = static_cast<unsigned long long>(a.e0);
             H->bar[1] = 0;
             H->notier[0] = 0;
+            H->general = 0;
         }
     }
     {
@@ -816,16 +818,25 @@ SolveShape solve_shape(bchar_mesh_t m) {
     return {static_cast<int>(g), kWideCluster, 0};
 }
 
+// All blocks resident at once: one cluster, or a cooperative launch.
 template <typename... P, typename... A>
-static void launch_cooperative(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t s, A... args) {
+static void launch_resident(void (*kernel)(P...), int grid, bool cluster, int block, size_t smem, cudaStream_t s,
+                            A... args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeCooperative;
-    at[0].val.cooperative = 1;
+    if (cluster) {
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = grid;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+    } else {
+        at[0].id = cudaLaunchAttributeCooperative;
+        at[0].val.cooperative = 1;
+    }
     cfg.attrs = at;
     cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
@@ -881,17 +892,20 @@ void amg_build(bchar_mesh_t m, const IpArgs &ip, bool same_aggregates) {
     }
     a.ip = ip;
     a.same = same_aggregates ? 1 : 0;
-    static bool attrs = false;  // the shared-memory opt-in (harmless to repeat)
+    static bool attrs = false;  // opt-ins of the kernels (harmless to repeat)
     if (!attrs) {
-        cudaFuncSetAttribute(k_amg_build<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBuildSmem));
-        cudaFuncSetAttribute(k_amg_build<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBuildSmem));
+        void (*const all[])(BuildArgs) = {k_amg_build<4, false>, k_amg_build<16, false>, k_amg_build<4, true>, k_amg_build<16, true>};
+        for (auto k : all) {
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBuildSmem));
+            cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        }
         attrs = true;
     }
-    const int grid = solve_shape(m).grid;
-    if (A.e0 <= 10 * A.n0)
-        launch_cooperative(k_amg_build<4>, grid, kBuildThreads, kBuildSmem, m->stream, a);
-    else
-        launch_cooperative(k_amg_build<16>, grid, kBuildThreads, kBuildSmem, m->stream, a);
+    const SolveShape shape = solve_shape(m);
+    const bool few = A.e0 <= 10 * A.n0;  // lanes per row
+    launch_resident(shape.small ? (few ? k_amg_build<4, true> : k_amg_build<16, true>)
+                                : (few ? k_amg_build<4, false> : k_amg_build<16, false>),
+                    shape.grid, shape.small, kBuildThreads, kBuildSmem, m->stream, a);
     ++m->launches;
 }
 

@@ -39,6 +39,7 @@ struct LevelInfo {
 struct Hier {
     unsigned bar[3];          // barrier counters: build (zeroed by the solves), solves (by the build), stage timing
     int notier[2];            // (solves, stage timing) the first cluster's levels do not fit its shared memory
+    int general;              // a block's rows of the finest level do not fit its shared memory (zeroed by the build)
     // set by a build with new aggregates
     int overflow;             // the entry arrays are full: coarsening stops
     unsigned long long ecur;  // entries in use

@@ -15,20 +15,27 @@ constexpr long long kSpinClocks = 10000000000LL;
 // block's earlier writes visible to all threads of every block.  About 2 350
 // clocks on 16 to 152 blocks (1.2 us), against ~2.5 us for a dependent kernel
 // launch; with one block it is the block barrier alone (~160 clocks).
-struct GridBar {
+// A grid that is one cluster (CLUSTER) has the hardware's barrier, about 450 clocks.
+template <bool CLUSTER> struct GridBarT {
+    static constexpr bool kCluster = CLUSTER;
     unsigned *cnt;
     int *err;
     unsigned nb, target = 0;
-    __device__ GridBar(unsigned *c, int *e, unsigned n) : cnt(c), err(e), nb(n) {}
+    __device__ GridBarT(unsigned *c, int *e, unsigned n) : cnt(c), err(e), nb(n) {}
     // false (in every thread of the block): the wait ran out, or another block's did
     __device__ bool sync() {
+        if (CLUSTER && nb > 1) {
+            asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+            return true;
+        }
         target += nb;
         __syncthreads();
         if (nb == 1) return true;
         int ok = 1;
         if (threadIdx.x == 0) {
             unsigned v;
-            asm volatile("atom.add.release.gpu.global.u32 %0, [%1], 1;" : "=r"(v) : "l"(cnt) : "memory");
+            // a reduction: an atomic's result would be waited for before the first poll
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(cnt) : "memory");
             const long long t0 = clock64();
             for (unsigned polls = 1;; ++polls) {
                 asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
@@ -44,5 +51,6 @@ struct GridBar {
         return __syncthreads_and(ok) != 0;
     }
 };
+using GridBar = GridBarT<false>;
 
 }  // namespace bchar

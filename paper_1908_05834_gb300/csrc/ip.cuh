@@ -411,7 +411,8 @@ __device__ __forceinline__ void ip_totals(IpShared &S, const double *part, int s
 constexpr int kIpLanes = 4;  // lanes per row: the rows of the recipes hold 3 to 7 entries in the mean
 
 // Weights; the normal equations' right-hand side of the predictor or corrector.
-static __device__ __noinline__ bool ip_weights(const IpArgs &A, GridBar &bar, int64_t r0, int64_t r1) {
+template <class Bar>
+static __device__ __noinline__ bool ip_weights(const IpArgs &A, Bar &bar, int64_t r0, int64_t r1) {
     ip_weights_rows<kIpLanes>(A, r0, r1);
     if (!bar.sync()) return false;
     ip_weights_cols<kIpLanes>(A, r0, r1);
@@ -419,7 +420,8 @@ static __device__ __noinline__ bool ip_weights(const IpArgs &A, GridBar &bar, in
 }
 
 // The direction's steps to the boundary, S.ap and S.ad.
-static __device__ __noinline__ bool ip_steps(const IpArgs &A, GridBar &bar, IpShared &S, int64_t r0, int64_t r1,
+template <class Bar>
+static __device__ __noinline__ bool ip_steps(const IpArgs &A, Bar &bar, IpShared &S, int64_t r0, int64_t r1,
                                          const double *dc, double sgn) {
     long long mx[2] = {sbits(1.0), sbits(1.0)};
     ip_dir<kIpLanes>(A, r0, r1, dc, sgn, mx[0], mx[1]);
@@ -433,7 +435,8 @@ static __device__ __noinline__ bool ip_steps(const IpArgs &A, GridBar &bar, IpSh
 
 // Mehrotra's centring target (comp_aff / comp)^3 mu, not below the floor, and
 // the corrector's right-hand side.
-static __device__ __noinline__ bool ip_corrector(const IpArgs &A, GridBar &bar, IpShared &S, int64_t r0, int64_t r1) {
+template <class Bar>
+static __device__ __noinline__ bool ip_corrector(const IpArgs &A, Bar &bar, IpShared &S, int64_t r0, int64_t r1) {
     const long long none[1] = {0};
     ip_partials<true, 1>(S, A.part, ip_comp_aff(A, r0, r1, S.ap, S.ad), none);
     if (!bar.sync()) return false;
@@ -451,8 +454,8 @@ static __device__ __noinline__ bool ip_corrector(const IpArgs &A, GridBar &bar, 
 
 // Residuals of the iterate, the scalars and the stopping test; cg: the solves'
 // conjugate-gradient iterations so far (of block 0), done: iterations done.
-template <bool START>
-static __device__ __noinline__ bool ip_check(const IpArgs &A, GridBar &bar, IpShared &S, int64_t r0, int64_t r1, int cg,
+template <bool START, class Bar>
+static __device__ __noinline__ bool ip_check(const IpArgs &A, Bar &bar, IpShared &S, int64_t r0, int64_t r1, int cg,
                                              int done, const IpStart &at) {
     IpResid R;
     ip_residual<kIpLanes, START>(A, r0, r1, at, R);
@@ -480,7 +483,8 @@ static __device__ __noinline__ bool ip_check(const IpArgs &A, GridBar &bar, IpSh
 }
 
 // The step, a fraction of the way to the boundary, then the check.
-static __device__ __noinline__ bool ip_step(const IpArgs &A, GridBar &bar, IpShared &S, int64_t r0, int64_t r1, int cg,
+template <class Bar>
+static __device__ __noinline__ bool ip_step(const IpArgs &A, Bar &bar, IpShared &S, int64_t r0, int64_t r1, int cg,
                                         int done) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         A.st->ap = S.ap;

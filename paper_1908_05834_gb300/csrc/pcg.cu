@@ -1,5 +1,6 @@
 // Preconditioned conjugate gradients on the normal equations of the
-// minimisation, one cooperative kernel per solve.
+// minimisation: one kernel for both solves of an interior-point iteration, with
+// the iteration's passes over the entries around them (ip.cuh).
 //
 // Each iteration is a product with the finest level, a vector update and one
 // V-cycle (a damped-Jacobi sweep before and after the coarse correction, the
@@ -9,8 +10,8 @@
 // with 40 sweeps at the bottom: 0.13 ms per iteration at 32^2, 0.22 ms at
 // 128^2, 0.35 ms at 24^3, for 5 to 30 us of arithmetic and memory traffic.
 //
-// Here a solve is one launch, and what bounds it is, per pass, the barrier after
-// it (2 350 clocks across the grid, about 600 within a cluster), one round trip
+// In one launch what bounds a solve is, per pass, the barrier after
+// it (2 350 clocks across the grid, about 450 within a cluster), one round trip
 // to L2 (~800 clocks), and the FP64 pipe: a warp instruction of it takes 19
 // clocks of its SM however many lanes are active, so work is spread over many
 // SMs even when there is little of it, sums take one thread per row, and scalars
@@ -58,7 +59,6 @@ struct PcgArgs {
     int n0;
     int64_t e0;
     int schur;
-    int small;  // one cluster does it all
     int64_t nc;
     const int64_t *row_ptr, *col_ptr;
     const int32_t *col, *csc_row;
@@ -512,9 +512,12 @@ struct Row {
     double dg, om;
 };
 
-__device__ __forceinline__ Row any_row(const HierView &v, const Rows &R, int k) {
+// HERE: from shared memory.  As a template parameter of the passes: with a pointer
+// that may be to either memory (generic loads) a system whose rows fit but for the
+// gathered values took 325 ms a step instead of 277 (32^3, rows of 5 to 40).
+template <bool HERE> __device__ __forceinline__ Row row_at(const HierView &v, const Rows &R, int k) {
     Row r;
-    if (R.here) {
+    if (HERE) {
         const int o = at_i(R.off)[k];
         r.id = at_i(R.id)[k];
         r.len = at_i(R.off)[k + 1] - o;
@@ -532,6 +535,11 @@ __device__ __forceinline__ Row any_row(const HierView &v, const Rows &R, int k) 
     r.dg = v.dg[R.noff + r.id];
     r.om = v.om[R.noff + r.id];
     return r;
+}
+
+__device__ __forceinline__ int row_id(const HierView &v, const Rows &R, int k) {
+    if (R.here) return at_i(R.id)[k];
+    return R.whole ? R.i0 + k : v.own[R.noff + (k < R.nmem ? R.m0 + k : R.l0 + k - R.nmem)];
 }
 
 template <int LPR> __device__ __forceinline__ double lanes_sum(double s) {
@@ -565,27 +573,40 @@ template <int LPR, class F> __device__ __forceinline__ void for_items(int n, F f
     }
 }
 
-#define WITH_LANES(L, CALL)                             \
-    switch (L) {                                        \
-    case 1: { constexpr int LPR = 1; CALL; } break;     \
-    case 2: { constexpr int LPR = 2; CALL; } break;     \
-    case 4: { constexpr int LPR = 4; CALL; } break;     \
-    case 8: { constexpr int LPR = 8; CALL; } break;     \
-    default: { constexpr int LPR = 16; CALL; } break;   \
+// Lanes per row of the general passes: with many rows per block, else they are in
+// shared memory.  A single cluster's system comes here only when its levels do not
+// fit: one variant is enough.
+#define WITH_LANES(L, H, CALL)                                  \
+    if constexpr (Bar::kCluster) {                              \
+        constexpr bool HERE = false;                            \
+        constexpr int LPR = 4;                                  \
+        CALL;                                                   \
+    } else if (H) {                                             \
+        constexpr bool HERE = true;                             \
+        WITH_LANES_OF(L, CALL)                                  \
+    } else {                                                    \
+        constexpr bool HERE = false;                            \
+        WITH_LANES_OF(L, CALL)                                  \
+    }
+#define WITH_LANES_OF(L, CALL)                                  \
+    switch (L) {                                                \
+    case 1: { constexpr int LPR = 1; CALL; } break;             \
+    case 2: { constexpr int LPR = 2; CALL; } break;             \
+    default: { constexpr int LPR = 4; CALL; } break;            \
     }
 
 // b and x of the next level: the residual b - L x summed over each aggregate,
 // and that level's first sweep from zero.
-template <int LPR>
+template <int LPR, bool HERE>
 __device__ void general_down(const HierView &v, const Rows &R, const double *bl, const double *x, double *bc, double *xc) {
     const int64_t noff2 = R.noff + R.n;
     for_items<LPR>(R.ngrp, [&](bool ok, int sub, int g) {
         double s = 0.0;
         if (ok) {
-            const int k0 = R.here ? at_i(R.gst)[g] : v.gs[noff2 + R.i0 + g] - R.m0;
-            const int k1 = R.here ? at_i(R.gst)[g + 1] : k0 + v.gc[noff2 + R.i0 + g];
+            const int k0 = HERE ? at_i(R.gst)[g] : v.gs[noff2 + R.i0 + g] - R.m0;
+            const int k1 = HERE ? at_i(R.gst)[g + 1] : k0 + v.gc[noff2 + R.i0 + g];
             for (int k = k0; k < k1; ++k) {
-                const Row r = any_row(v, R, k);
+                const Row r = row_at<HERE>(v, R, k);
                 if (sub == 0) s += bl[r.id] - r.dg * x[r.id];
                 s += lane_dot<LPR>(r, sub, x);
             }
@@ -606,14 +627,14 @@ __device__ __forceinline__ void prolong(const HierView &v, int64_t noff, int64_t
 }
 
 // The sweep after the coarse correction, prolonged into the finer level.
-template <int LPR>
+template <int LPR, bool HERE>
 __device__ void general_up(const HierView &v, const Rows &R, const double *bl, const double *x, int64_t fine, double *xf) {
     for_items<LPR>(R.nrow, [&](bool ok, int sub, int k) {
         double s = 0.0;
         Row r{};
         double xi = 0.0, bi = 0.0;
         if (ok) {
-            r = any_row(v, R, k);
+            r = row_at<HERE>(v, R, k);
             xi = x[r.id];
             bi = bl[r.id];
             s = lane_dot<LPR>(r, sub, x);
@@ -624,7 +645,7 @@ __device__ void general_up(const HierView &v, const Rows &R, const double *bl, c
 }
 
 // The same on the finest level: z, and this thread's parts of z.r and z.q.
-template <int LPR>
+template <int LPR, bool HERE>
 __device__ void general_top(const HierView &v, const Rows &R, const double *r_, const double *q_, const double *x, double *z,
                             double &rz, double &zq) {
     for_items<LPR>(R.nrow, [&](bool ok, int sub, int k) {
@@ -632,7 +653,7 @@ __device__ void general_top(const HierView &v, const Rows &R, const double *r_, 
         Row r{};
         double xi = 0.0, bi = 0.0, qi = 0.0;
         if (ok) {
-            r = any_row(v, R, k);
+            r = row_at<HERE>(v, R, k);
             xi = x[r.id];
             bi = r_[r.id];
             qi = q_[r.id];
@@ -649,13 +670,13 @@ __device__ void general_top(const HierView &v, const Rows &R, const double *r_, 
 }
 
 // One Jacobi sweep of a coarsest level shared by all blocks.
-template <int LPR>
+template <int LPR, bool HERE>
 __device__ void general_sweep(const HierView &v, const Rows &R, const double *bl, const double *x, double *xo) {
     for_items<LPR>(R.nrow, [&](bool ok, int sub, int k) {
         double s = 0.0;
         Row r{};
         if (ok) {
-            r = any_row(v, R, k);
+            r = row_at<HERE>(v, R, k);
             s = lane_dot<LPR>(r, sub, x);
         }
         s = lanes_sum<LPR>(s);
@@ -668,14 +689,14 @@ __device__ void general_sweep(const HierView &v, const Rows &R, const double *bl
 
 // q = L p and this thread's part of p.q.  FUSED: p = z + beta pold is formed by
 // its readers and stored by its owner.
-template <int LPR, bool FUSED>
+template <int LPR, bool HERE, bool FUSED>
 __device__ void general_product(const HierView &v, const Rows &R, const double *z, const double *pold, double beta,
                                 double *p, double *q, double &pq) {
     for_items<LPR>(R.nrow, [&](bool ok, int sub, int k) {
         double s = 0.0, pi = 0.0;
         Row r{};
         if (ok) {
-            r = any_row(v, R, k);
+            r = row_at<HERE>(v, R, k);
             if (FUSED) {
                 pi = z[r.id] + beta * pold[r.id];
                 int e = sub;
@@ -848,8 +869,9 @@ __device__ void fast_top(const Shared &sh, const View R, const double *x, double
     });
 }
 
+// yq (or null): gets om q, for fast_first.
 __device__ void fast_product(const Shared &sh, const View R, const double *z, const double *pold, double beta, double *p,
-                             double &pq) {
+                             double *yq, double &pq) {
     const int tid = threadIdx.x;
     double *const xg = at_d(sh.xg), *const po = at_d(sh.po), *const qo = at_d(sh.qo);
     const double *const zo = at_d(sh.zo);
@@ -867,9 +889,52 @@ __device__ void fast_product(const Shared &sh, const View R, const double *z, co
             p[R.id[k]] = pi;
             const double qi = R.dg[k] * pi - s;
             qo[k] = qi;
+            if (yq) yq[R.id[k]] = R.om[k] * qi;
             pq += pi * qi;
         }
     });
+}
+
+// The step of the conjugate gradients and the finest level's way down in one
+// pass: the neighbours' new smoothed values are xr - alpha yq, with xr = om r
+// and yq = om q of before (the owner's own differs from that in its last bits
+// at most, and only the preconditioner sees it).  A pass and a grid barrier
+// less per iteration: a step at 96^2 82.1 ms instead of 85.2, at 320^2 502 instead
+// of 531.
+__device__ void fast_first(const Shared &sh, const View R, const double *xr, const double *yq, double alpha, double *xrn,
+                           double *x, double *bc, double *xc, unsigned long long &mx) {
+    const int tid = threadIdx.x;
+    double *const xg = at_d(sh.xg), *const ro = at_d(sh.ro), *const dd = at_d(sh.dd);
+    const double *const qo = at_d(sh.qo), *const po = at_d(sh.po), *const ibo = at_d(sh.ibo);
+    for (int e = tid; e < R.ents; e += kNT) {
+        const int c = R.col[e];
+        xg[e] = xr[c] - alpha * yq[c];
+    }
+    for (int k = tid; k < R.nrow; k += kNT) {
+        dd[k] += alpha * po[k];
+        const double r = ro[k] - alpha * qo[k], v = R.om[k] * r;
+        ro[k] = r;
+        R.bo[k] = r;
+        R.res[k] = v;
+        xrn[R.id[k]] = v;
+        x[R.id[k]] = v;
+        mx = max_bits(mx, bits_of(fabs(r) * ibo[k]));
+    }
+    __syncthreads();
+    for_rows(R.nrow, R.lg, [&](bool ok, int sub, int t) {
+        const int k = ok ? R.ord[t] : 0;
+        const bool in = ok && k < R.nmem;
+        double s = 0.0;
+        if (in) s = row_sum(R, k, sub, xg, sub ? 0.0 : R.bo[k] - R.dg[k] * R.res[k]);
+        s = lanes_total(s, R.lg);
+        if (in && sub == 0) R.res[k] = s;
+    });
+    __syncthreads();
+    for (int g = tid; g < R.ngrp; g += kNT) {
+        const double s = group_sum(R, g);
+        bc[R.i0 + g] = s;
+        xc[R.i0 + g] = R.omc[g] * s;
+    }
 }
 
 // ---------------------------------------------------------------- the first cluster's levels
@@ -1207,18 +1272,21 @@ __device__ int solve_small(const PcgArgs &a, Shared &sh, unsigned rank, unsigned
 }
 
 // One V-cycle across the grid; x of the finest level holds om r on entry, alt is
-// a free vector of its size.  This thread's parts of z.r, z.q.
-__device__ bool grid_cycle(const PcgArgs &a, Shared &sh, GridBar &bar, double *alt, double &rz, double &zq) {
+// a free vector of its size; first = 1: level 0's way down is done.  This
+// thread's parts of z.r, z.q.
+template <class Bar>
+__device__ bool grid_cycle(const PcgArgs &a, Shared &sh, Bar &bar, int first, double *alt, double &rz,
+                                        double &zq) {
     const HierView &v = a.v;
     const int nlev = sh.nlev, t0 = sh.t0;
     const int nd = t0 < nlev ? t0 : nlev - 1;  // shared levels that are aggregated
-    for (int l = 0; l < nd; ++l) {
+    for (int l = first; l < nd; ++l) {
         const Rows &R = sh.lev[l];
         double *bc = v.b + (R.noff + R.n), *xc = v.x + (R.noff + R.n);
         if (R.here == 1)
             fast_down(sh, view(R), l ? v.b + R.noff : nullptr, v.x + R.noff, bc, xc);
         else
-            WITH_LANES(R.lprg, (general_down<LPR>(v, R, l ? v.b + R.noff : a.r, v.x + R.noff, bc, xc)));
+            WITH_LANES(R.lprg, R.here, (general_down<LPR, HERE>(v, R, l ? v.b + R.noff : a.r, v.x + R.noff, bc, xc)));
         if (!bar.sync()) return false;
     }
     if (t0 < nlev) {
@@ -1266,7 +1334,7 @@ __device__ bool grid_cycle(const PcgArgs &a, Shared &sh, GridBar &bar, double *a
             if (!bar.sync()) return false;
         } else {
             for (int k = 0; k < sh.sweeps; ++k) {
-                WITH_LANES(R.lpr, (general_sweep<LPR>(v, R, bl, (k & 1) ? alt : x, (k & 1) ? x : alt)));
+                WITH_LANES(R.lpr, R.here, (general_sweep<LPR, HERE>(v, R, bl, (k & 1) ? alt : x, (k & 1) ? x : alt)));
                 if (!bar.sync()) return false;
             }
         }
@@ -1291,19 +1359,20 @@ __device__ bool grid_cycle(const PcgArgs &a, Shared &sh, GridBar &bar, double *a
         if (R.here == 1)
             fast_up(sh, view(R), v.x + R.noff, v.x + fine);
         else
-            WITH_LANES(R.lpr, (general_up<LPR>(v, R, v.b + R.noff, v.x + R.noff, fine, v.x + fine)));
+            WITH_LANES(R.lpr, R.here, (general_up<LPR, HERE>(v, R, v.b + R.noff, v.x + R.noff, fine, v.x + fine)));
         if (!bar.sync()) return false;
     }
     const Rows &R = sh.lev[0];
     if (R.here == 1)
         fast_top(sh, view(R), v.x + 0, a.z, rz, zq);
     else
-        WITH_LANES(R.lpr, (general_top<LPR>(v, R, a.r, a.q, v.x + 0, a.z, rz, zq)));
+        WITH_LANES(R.lpr, R.here, (general_top<LPR, HERE>(v, R, a.r, a.q, v.x + 0, a.z, rz, zq)));
     return true;
 }
 
 // A system shared by all blocks.  Returns the iterations, -1 when a barrier failed.
-__device__ int solve_grid_wide(const PcgArgs &a, Shared &sh, GridBar &bar, int which, double trz, double tres, int cap) {
+template <class Bar>
+__device__ int solve_grid_wide(const PcgArgs &a, Shared &sh, Bar &bar, int which, double trz, double tres, int cap) {
     const HierView &v = a.v;
     Hier *H = v.H;
     const Rows &R = sh.lev[0];
@@ -1314,9 +1383,14 @@ __device__ int solve_grid_wide(const PcgArgs &a, Shared &sh, GridBar &bar, int w
     const int tid = threadIdx.x;
     double *pbuf[2] = {a.p0, a.p1};
     const bool here = R.here == 1;
+    // rows of every block in shared memory: the vectors there leave a.ib, a.r (om r, in turns)
+    // and a.q (om q) free for fast_first
+    const bool fused = a.e0 <= kFuseEntries * nb;
+    const bool lean = fused && sh.nlev > 1 && !a.vcycle && *reinterpret_cast<volatile int *>(&H->general) == 0;
+    double *xr[2] = {a.ib, a.r};
     for_items<8>(R.nrow, [&](bool ok, int sub, int k) {
         int id = 0;
-        if (ok) id = here ? O.id[k] : any_row(v, R, k).id;
+        if (ok) id = here ? O.id[k] : row_id(v, R, k);
         const double s = start_residual<8>(a, v, which, id, sub);
         if (ok && sub == 0) {
             const double r = a.vcycle ? a.r[id] : s, ib = inverse_target(a, id);
@@ -1333,27 +1407,33 @@ __device__ int solve_grid_wide(const PcgArgs &a, Shared &sh, GridBar &bar, int w
                 a.ib[id] = ib;
             }
             v.x[id] = v.om[id] * r;
+            if (lean) a.ib[id] = v.om[id] * r;
         }
     });
     if (!bar.sync()) return -1;
     if (!here && !which && !a.vcycle)  // after the barrier: other rows' starts may read d
-        for (int k = tid; k < R.nrow; k += kNT) a.d[any_row(v, R, k).id] = 0.0;
-    double rz = 0.0, zq = 0.0;
-    if (!grid_cycle(a, sh, bar, a.p1, rz, zq)) return -1;
-    if (a.vcycle) return 0;
-    block_partials(sh, 1, here ? R.nrow << R.lg : kNT, rz, 0.0, 0);
-    if (tid == 0) H->part[1][b] = sh.out[0];
-    if (!bar.sync()) return -1;
-    block_totals(sh, H->part[1], kMaxCtas, 1, nb);
-    if (tid == 0) {
-        sh.rz = sh.out[0];
-        sh.beta = 0.0;
-        sh.conv = sh.out[0] == 0.0 ? 1 : 0;
-    }
-    __syncthreads();
-    const bool fused = a.e0 <= kFuseEntries * nb;
+        for (int k = tid; k < R.nrow; k += kNT) a.d[row_id(v, R, k)] = 0.0;
     int it = 0;
-    while (!sh.conv && it < cap) {
+    unsigned long long mx = 0;
+    for (;;) {
+        double rz = 0.0, zq = 0.0;
+        if (!grid_cycle(a, sh, bar, lean && it ? 1 : 0, pbuf[(it + 1) & 1], rz, zq)) return -1;
+        if (a.vcycle) return 0;
+        block_partials(sh, 3, here ? R.nrow << R.lg : kNT, rz, zq, mx);
+        if (tid < 3) H->part[1 + tid][b] = sh.out[tid];
+        if (!bar.sync()) return -1;
+        block_totals(sh, H->part[1], kMaxCtas, 3, nb);
+        if (tid == 0) {
+            if (it == 0) {
+                sh.rz = sh.out[0];
+                sh.beta = 0.0;
+                sh.conv = sh.out[0] == 0.0 ? 1 : 0;
+            } else {
+                set_beta(sh, trz, tres);
+            }
+        }
+        __syncthreads();
+        if (sh.conv || it >= cap) break;
         ++it;
         invert_rz(sh);
         const double beta = sh.beta;
@@ -1362,7 +1442,7 @@ __device__ int solve_grid_wide(const PcgArgs &a, Shared &sh, GridBar &bar, int w
         double pq = 0.0;
         if (!fused) {  // grid-uniform
             for (int k = tid; k < R.nrow; k += kNT) {
-                const int i = here ? O.id[k] : any_row(v, R, k).id;
+                const int i = here ? O.id[k] : row_id(v, R, k);
                 pn[i] = a.z[i] + beta * pold[i];
             }
             if (!bar.sync()) return -1;
@@ -1380,12 +1460,12 @@ __device__ int solve_grid_wide(const PcgArgs &a, Shared &sh, GridBar &bar, int w
                     }
                 });
             } else {
-                WITH_LANES(R.lpr, (general_product<LPR, false>(v, R, a.z, pold, beta, pn, a.q, pq)));
+                WITH_LANES(R.lpr, R.here, (general_product<LPR, HERE, false>(v, R, a.z, pold, beta, pn, a.q, pq)));
             }
         } else if (here) {
-            fast_product(sh, O, a.z, pold, beta, pn, pq);
+            fast_product(sh, O, a.z, pold, beta, pn, lean ? a.q : nullptr, pq);
         } else {
-            WITH_LANES(R.lpr, (general_product<LPR, true>(v, R, a.z, pold, beta, pn, a.q, pq)));
+            WITH_LANES(R.lpr, R.here, (general_product<LPR, HERE, true>(v, R, a.z, pold, beta, pn, a.q, pq)));
         }
         block_partials(sh, 1, here ? R.nrow << R.lg : kNT, pq, 0.0, 0);
         if (tid == 0) H->part[0][b] = sh.out[0];
@@ -1394,8 +1474,12 @@ __device__ int solve_grid_wide(const PcgArgs &a, Shared &sh, GridBar &bar, int w
         if (tid == 0) set_alpha(sh, sh.out[0]);
         __syncthreads();
         const double alpha = sh.alpha;
-        unsigned long long mx = 0;
-        for (int k = tid; k < R.nrow; k += kNT) {
+        mx = 0;
+        if (lean) {
+            const int64_t c = R.noff + R.n;  // the next level's nodes
+            fast_first(sh, O, xr[(it + 1) & 1], a.q, alpha, xr[it & 1], v.x + 0, v.b + c, v.x + c, mx);
+        }
+        for (int k = lean ? R.nrow : tid; k < R.nrow; k += kNT) {
             if (here) {
                 dd[k] += alpha * po[k];
                 const double r = ro[k] - alpha * qo[k];
@@ -1403,7 +1487,7 @@ __device__ int solve_grid_wide(const PcgArgs &a, Shared &sh, GridBar &bar, int w
                 v.x[O.id[k]] = O.om[k] * r;
                 mx = max_bits(mx, bits_of(fabs(r) * ibo[k]));
             } else {
-                const int i = any_row(v, R, k).id;
+                const int i = row_id(v, R, k);
                 a.d[i] += alpha * pn[i];
                 const double r = a.r[i] - alpha * a.q[i];
                 a.r[i] = r;
@@ -1412,14 +1496,6 @@ __device__ int solve_grid_wide(const PcgArgs &a, Shared &sh, GridBar &bar, int w
             }
         }
         if (!bar.sync()) return -1;
-        rz = zq = 0.0;
-        if (!grid_cycle(a, sh, bar, const_cast<double *>(pold), rz, zq)) return -1;
-        block_partials(sh, 3, here ? R.nrow << R.lg : kNT, rz, zq, mx);
-        if (tid < 3) H->part[1 + tid][b] = sh.out[tid];
-        if (!bar.sync()) return -1;
-        block_totals(sh, H->part[1], kMaxCtas, 3, nb);
-        if (tid == 0) set_beta(sh, trz, tres);
-        __syncthreads();
     }
     if (here)
         for (int k = tid; k < R.nrow; k += kNT) {
@@ -1440,7 +1516,8 @@ __device__ __forceinline__ void own_vectors(Shared &sh, unsigned f, int n) {
     sh.ibo = f + 5 * s;
 }
 
-__global__ void __launch_bounds__(kSolveThreads, 1) k_pcg(const __grid_constant__ PcgArgs a) {
+// ONE: the grid is one cluster, for a small system.
+template <bool ONE> __global__ void __launch_bounds__(kSolveThreads, 1) k_pcg(const __grid_constant__ PcgArgs a) {
     __shared__ Shared sh;
     const HierView &v = a.v;
     Hier *H = v.H;
@@ -1448,7 +1525,7 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_pcg(const __grid_constant_
     const unsigned rank = cluster_rank(), nr = cluster_size();
     const int tid = threadIdx.x;
     const IpArgs &ip = a.ip;
-    GridBar bar(&H->bar[a.vcycle ? 2 : 1], &ip.st->err, nb);
+    GridBarT<ONE> bar(&H->bar[a.vcycle ? 2 : 1], &ip.st->err, nb);
     // an earlier barrier failed: nothing here can be relied on; or the iterations have ended
     if (__syncthreads_or(ip.st->err | (a.vcycle ? 0 : ip.st->stop))) return;
     int *const notier = &H->notier[a.vcycle ? 1 : 0];
@@ -1467,11 +1544,11 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_pcg(const __grid_constant_
     if (tid == 0) {
         const int nlev = H->nlev;
         int t0 = nlev;
-        for (int l = nlev - 1; l >= (a.small ? 0 : 1); --l) {
-            if (!a.small && (H->L[l].nnz > kTierEntries || H->L[l].n > kTierNodes)) break;
+        for (int l = nlev - 1; l >= (ONE ? 0 : 1); --l) {
+            if (!ONE && (H->L[l].nnz > kTierEntries || H->L[l].n > kTierNodes)) break;
             t0 = l;
         }
-        if (a.small && nlev == 1) t0 = nlev;
+        if (ONE && nlev == 1) t0 = nlev;
         int tr = nlev - 1;
         while (tr - 1 > t0 && H->L[tr - 1].n <= kCopyNodes && H->L[tr - 1].nnz <= kCopyEntries) --tr;
         sh.nlev = nlev;
@@ -1546,7 +1623,7 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_pcg(const __grid_constant_
         p = 0;
         __syncthreads();
     }
-    const bool alone = sh.t0 == 0;
+    const bool alone = ONE && sh.t0 == 0;
     if (!alone) {
         // shared levels, the finest first; the gathered values of a pass go to the end of the arrays
         const int ns = sh.t0 < sh.nlev ? sh.t0 : sh.nlev;
@@ -1560,7 +1637,8 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_pcg(const __grid_constant_
                 own = static_cast<size_t>(g.mlen + g.llen) * 48 + 128;
             }
             const bool got = !coarsest && load_rows(v, sh, l, kGrid, static_cast<int>(b), static_cast<int>(nb), p, end,
-                                                    own, most) && sh.lev[l].here;
+                                                    own, most) &&
+                             (ONE ? sh.lev[l].here == 1 : sh.lev[l].here != 0);
             if (coarsest) {
                 unsigned q = p;  // rows are read from global memory: only the description is wanted
                 load_rows(v, sh, l, kGrid, static_cast<int>(b), static_cast<int>(nb), q, q, 1, 0);
@@ -1578,7 +1656,10 @@ __global__ void __launch_bounds__(kSolveThreads, 1) k_pcg(const __grid_constant_
             }
             __syncthreads();
         }
-        if (tid == 0) sh.xg = p;
+        if (tid == 0) {
+            sh.xg = p;
+            if (!a.vcycle && sh.lev[0].here != 1) atomicExch(&H->general, 1);
+        }
         __syncthreads();
     }
 
@@ -1669,33 +1750,33 @@ static PcgArgs pcg_args(bchar_mesh_t m) {
 static void launch_pcg(bchar_mesh_t m, PcgArgs &a) {
     static bool attrs = false;  // opt-ins of the kernel (harmless to repeat)
     if (!attrs) {
-        cudaFuncSetAttribute(k_pcg, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSolveSmem));
-        cudaFuncSetAttribute(k_pcg, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        cudaFuncSetAttribute(k_pcg<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSolveSmem));
+        cudaFuncSetAttribute(k_pcg<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSolveSmem));
+        cudaFuncSetAttribute(k_pcg<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         attrs = true;
     }
     const SolveShape s = solve_shape(m);
-    a.small = s.small;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(s.grid);
     cfg.blockDim = dim3(kSolveThreads);
     cfg.dynamicSmemBytes = kSolveSmem;
     cfg.stream = m->stream;
     cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeCooperative;
-    at[0].val.cooperative = 1;
-    at[1].id = cudaLaunchAttributeClusterDimension;
-    at[1].val.clusterDim.x = s.cluster;
-    at[1].val.clusterDim.y = 1;
-    at[1].val.clusterDim.z = 1;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = s.cluster;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeCooperative;
+    at[1].val.cooperative = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 2;
-    cudaLaunchKernelEx(&cfg, k_pcg, a);
+    cfg.numAttrs = s.small ? 1 : 2;  // one cluster is resident as a whole
+    cudaLaunchKernelEx(&cfg, s.small ? k_pcg<true> : k_pcg<false>, a);
     ++m->launches;
 }
 
 // Blocks of 8-block clusters that the device holds at once (one block per SM).
 int solve_blocks_resident() {
-    cudaFuncSetAttribute(k_pcg, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSolveSmem));
+    cudaFuncSetAttribute(k_pcg<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSolveSmem));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(kWideCluster);
     cfg.blockDim = dim3(kSolveThreads);
@@ -1708,7 +1789,7 @@ int solve_blocks_resident() {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, k_pcg, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, k_pcg<false>, &cfg) != cudaSuccess) {
         cudaGetLastError();
         n = 1;
     }
