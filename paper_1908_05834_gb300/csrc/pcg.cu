@@ -592,7 +592,9 @@ template <int LPR, class F> __device__ __forceinline__ void for_items(int n, F f
     switch (L) {                                                \
     case 1: { constexpr int LPR = 1; CALL; } break;             \
     case 2: { constexpr int LPR = 2; CALL; } break;             \
-    default: { constexpr int LPR = 4; CALL; } break;            \
+    case 4: { constexpr int LPR = 4; CALL; } break;             \
+    case 8: { constexpr int LPR = 8; CALL; } break;             \
+    default: { constexpr int LPR = 16; CALL; } break;           \
     }
 
 // b and x of the next level: the residual b - L x summed over each aggregate,
