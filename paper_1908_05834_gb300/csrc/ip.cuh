@@ -353,10 +353,16 @@ struct IpShared {
 };
 
 // The block's parts of a sum (slot 0) and of NM maxima (slots 1 .. NM, bits).
+// Every block reads the slots of all blocks, so a slot may be written only behind
+// a grid barrier that follows its last read:
+//   ip_steps to ip_corrector: 1 and 2 were read with no barrier since; 0 is written;
+//   ip_corrector to ip_steps: 0 was read; barriers follow (and 1 and 2 are written);
+//   ip_steps to ip_step: 1 and 2 were read; the barrier behind the update precedes
+//     the check, which writes all of them.
 template <bool SUM, int NM>
-__device__ void ip_partials(IpShared &S, double *part, double sum, const long long (&mx)[NM]) {
+__device__ void ip_partials(IpShared &S, double *part, double sum, const long long *mx) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    long long m[NM];
+    long long m[NM > 0 ? NM : 1];
 #pragma unroll
     for (int k = 0; k < NM; ++k) m[k] = mx[k];
     for (int o = 16; o > 0; o >>= 1) {
@@ -437,8 +443,7 @@ static __device__ __noinline__ bool ip_steps(const IpArgs &A, Bar &bar, IpShared
 // the corrector's right-hand side.
 template <class Bar>
 static __device__ __noinline__ bool ip_corrector(const IpArgs &A, Bar &bar, IpShared &S, int64_t r0, int64_t r1) {
-    const long long none[1] = {0};
-    ip_partials<true, 1>(S, A.part, ip_comp_aff(A, r0, r1, S.ap, S.ad), none);
+    ip_partials<true, 0>(S, A.part, ip_comp_aff(A, r0, r1, S.ap, S.ad), nullptr);
     if (!bar.sync()) return false;
     ip_totals(S, A.part, 0, 1);
     if (threadIdx.x == 0) {
