@@ -110,6 +110,16 @@ __device__ __forceinline__ int high_word(double w) { return __double2hiint(w); }
 constexpr int kStrengthHi = 3483294;  // -log2(kStrength) = 3.3219, in those units
 constexpr int kAttachHi = 2 << 20;    // -log2(kAttach)
 static_assert(kStrength == 0.1 && kAttach == 0.25, "the constants above follow them");
+// Whether an edge of weight w is strong between diagonals di and dj, w >= kStrength
+// sqrt(di dj); whether it carries kAttach of di.  The sum of two high words passes
+// 2^31 from weights of 0.2 on (a mesh given in metres, or in cell widths): with 32
+// bits a 96^2 step on a square of side 1 024 took 3.6 times the CG iterations.
+__device__ __forceinline__ bool strong_edge(int w, int di, int dj) {
+    return 2ll * w + 2 * kStrengthHi >= static_cast<long long>(di) + dj;
+}
+__device__ __forceinline__ bool carries_diagonal(int w, int di) {
+    return static_cast<long long>(w) + kAttachHi >= di;
+}
 
 // The higher-ranked of (key, j) and (k2, j2); j < 0 is none; ties go to the smaller node.
 __device__ __forceinline__ void take_higher(unsigned long long &key, int &j, unsigned long long k2, int j2) {
@@ -239,8 +249,7 @@ __device__ void rank_round(const BuildArgs &a, int64_t noff, int i0, int i1, int
                         wmax = max(wmax, w);
                         take_higher(akey, aj, k, j);
                     }
-                    // strong: w >= kStrength sqrt(d_i d_j)
-                    if (2 * (w + kStrengthHi) >= di + high_word(v.dg[noff + j])) take_higher(key, bj, k, j);
+                    if (strong_edge(w, di, high_word(v.dg[noff + j]))) take_higher(key, bj, k, j);
                 }
             }
         }
@@ -258,7 +267,7 @@ __device__ void rank_round(const BuildArgs &a, int64_t noff, int i0, int i1, int
             } else {
                 // one-sided on purpose: a leaf hanging off a hub by an edge that is most of
                 // its own diagonal but little of the hub's should follow the hub
-                a.att[i] = (aj >= 0 && wmax + kAttachHi >= di) ? aj : -1;
+                a.att[i] = (aj >= 0 && carries_diagonal(wmax, di)) ? aj : -1;
                 a.cnt[i] = 0;
                 a.cap[i] = 0;
             }
