@@ -601,6 +601,7 @@ template <int LPR, bool ONE> __global__ void __launch_bounds__(kBuildThreads, 1)
             H->mcur[tid] = 0;
             H->nnzacc[tid] = 0;
         }
+        if (tid < kMaxCtas / kWideCluster) H->left[0][tid] = 0;
         if (tid == 0) {
             if (!a.same) H->overflow = 0;
             if (!a.same) H->ecur = static_cast<unsigned long long>(a.e0);

@@ -9,6 +9,8 @@ namespace bchar {
 
 constexpr int kMaxLevels = 40;
 constexpr int kMaxCtas = 256;        // blocks of the cooperative kernels at most
+constexpr int kWideCluster = 8;      // blocks per cluster of a solve across the grid
+constexpr int kSmallCluster = 16;    // of a solve by one cluster alone
 constexpr int kSolveThreads = 512;   // threads per block of the conjugate gradients
 constexpr int kBuildThreads = 1024;  // threads per block of the hierarchy build
 constexpr int kDense = 32;           // a coarsest level of at most this many nodes is solved by its inverse
@@ -39,6 +41,7 @@ struct LevelInfo {
 struct Hier {
     unsigned bar[3];          // barrier counters: build (zeroed by the solves), solves (by the build), stage timing
     int notier[2];            // (solves, stage timing) the first cluster's levels do not fit its shared memory
+    unsigned left[2][kMaxCtas / kWideCluster];  // (solves, stage timing) blocks at their end, per cluster (zeroed by the build)
     int general;              // a block's rows of the finest level do not fit its shared memory (zeroed by the build)
     // set by a build with new aggregates
     int overflow;             // the entry arrays are full: coarsening stops
@@ -74,8 +77,6 @@ struct SolveShape {
     int grid, cluster, small;
 };
 struct IpArgs;  // ip.cuh
-constexpr int kWideCluster = 8;    // blocks per cluster of a solve across the grid
-constexpr int kSmallCluster = 16;  // of a solve by one cluster alone
 SolveShape solve_shape(bchar_mesh_t m);
 int solve_blocks_resident();  // pcg.cu
 

@@ -53,4 +53,40 @@ template <bool CLUSTER> struct GridBarT {
 };
 using GridBar = GridBarT<false>;
 
+// The end of a block of a cluster whose blocks read and write one another's
+// shared memory and wait at the cluster's barrier.  A grid barrier that runs out
+// may fail in some of its blocks and not in others (a late block completes it), and
+// those go on until their next grid barrier: a failed block stays, and arrives at
+// every cluster barrier, until the whole cluster has come here.  The others need one
+// barrier: behind the last grid barrier nothing is exchanged.  C: done() counts
+// this block among those that are here, barrier() is the cluster's, all_done()
+// tells whether every block of the cluster has been counted.
+template <class C> __host__ __device__ inline void leave_cluster(C &c, bool failed) {
+    c.done();
+    // every round but the last accompanies one barrier of another block: a few hundred at
+    // most, the limit is for a block that is never counted
+    for (int k = 0; k < (1 << 22); ++k) {
+        c.barrier();
+        if (!failed || c.all_done()) break;
+    }
+}
+
+// On the device: `here` is a counter per cluster in global memory, zero at launch.
+struct ClusterEnd {
+    unsigned *here;
+    unsigned blocks;
+    __device__ void done() {
+        __syncthreads();
+        if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(here) : "memory");
+    }
+    __device__ void barrier() {
+        asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+    }
+    __device__ bool all_done() {
+        unsigned v = 0;
+        if (threadIdx.x == 0) asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(here) : "memory");
+        return __syncthreads_or(v >= blocks) != 0;
+    }
+};
+
 }  // namespace bchar

@@ -1528,8 +1528,13 @@ template <bool ONE> __global__ void __launch_bounds__(kSolveThreads, 1) k_pcg(co
     const int tid = threadIdx.x;
     const IpArgs &ip = a.ip;
     GridBarT<ONE> bar(&H->bar[a.vcycle ? 2 : 1], &ip.st->err, nb);
+    // formed where it is used: held through the solves it costs a register too many
+    auto end_of_block = [&]() { return ClusterEnd{&v.H->left[a.vcycle ? 1 : 0][blockIdx.x / cluster_size()], cluster_size()}; };
     // an earlier barrier failed: nothing here can be relied on; or the iterations have ended
-    if (__syncthreads_or(ip.st->err | (a.vcycle ? 0 : ip.st->stop))) return;
+    if (__syncthreads_or(ip.st->err | (a.vcycle ? 0 : ip.st->stop))) {
+        end_of_block().done();
+        return;
+    }
     int *const notier = &H->notier[a.vcycle ? 1 : 0];
     __shared__ IpShared ips;
     int64_t r0, r1;
@@ -1619,14 +1624,14 @@ template <bool ONE> __global__ void __launch_bounds__(kSolveThreads, 1) k_pcg(co
         __syncthreads();
         if (!ok && tid == 0) atomicExch(notier, 1);
     }
-    if (!bar.sync()) return;
-    if (*reinterpret_cast<volatile int *>(notier)) {  // grid-uniform
+    bool go = bar.sync();
+    if (go && *reinterpret_cast<volatile int *>(notier)) {  // grid-uniform
         if (tid == 0) sh.t0 = sh.nlev;
         p = 0;
         __syncthreads();
     }
     const bool alone = ONE && sh.t0 == 0;
-    if (!alone) {
+    if (go && !alone) {
         // shared levels, the finest first; the gathered values of a pass go to the end of the arrays
         const int ns = sh.t0 < sh.nlev ? sh.t0 : sh.nlev;
         int most = 0;
@@ -1665,14 +1670,13 @@ template <bool ONE> __global__ void __launch_bounds__(kSolveThreads, 1) k_pcg(co
         __syncthreads();
     }
 
-    if (a.vcycle) {
-        alone ? solve_small(a, sh, rank, nr, 0, 0.0, 0.0, 1) : solve_grid_wide(a, sh, bar, 0, 0.0, 0.0, 1);
-        cluster_sync();
-        return;
+    if (go && a.vcycle) {
+        go = (alone ? solve_small(a, sh, rank, nr, 0, 0.0, 0.0, 1) : solve_grid_wide(a, sh, bar, 0, 0.0, 0.0, 1)) >= 0;
+    } else if (go) {
+        ip_rhs<kIpLanes>(ip, r0, r1, 0, 0.0);
+        go = bar.sync();
     }
-    ip_rhs<kIpLanes>(ip, r0, r1, 0, 0.0);
-    bool go = bar.sync();
-    for (int corr = 0; corr < 2 && go; ++corr) {
+    for (int corr = 0; corr < 2 && go && !a.vcycle; ++corr) {
         const SolveTol &tol = a.tol[corr];
         const double trz = tol.rz_rel * mu, tres = fmax(tol.res_rel * rp_max, tol.res_floor);
         const int cap = max(1, min(tol.max_iter, ip.max_cg - cg));
@@ -1700,11 +1704,13 @@ template <bool ONE> __global__ void __launch_bounds__(kSolveThreads, 1) k_pcg(co
         go = ip_steps(ip, bar, ips, r0, r1, a.d + (a.schur ? 0 : a.nc), -1.0);
         if (go) go = corr ? ip_step(ip, bar, ips, r0, r1, cg, done + 1) : ip_corrector(ip, bar, ips, r0, r1) && bar.sync();
     }
-    if (b == 0 && tid == 0) {
+    if (b == 0 && tid == 0 && !a.vcycle) {
         ip.st->levels = sh.nlev;
         ip.st->coarsest = H->L[sh.nlev - 1].n;
     }
-    cluster_sync();  // no block leaves while another may still store into its shared memory
+    // no block leaves while another may still store into its shared memory
+    ClusterEnd here = end_of_block();
+    leave_cluster(here, !go);
 }
 
 // One damped-Jacobi sweep of the finest level (timing).
@@ -1813,6 +1819,7 @@ void amg_vcycle_once(bchar_mesh_t m) {
     Hier *H = ptr<Hier>(m->amg.hier);
     cudaMemsetAsync(&H->bar[2], 0, sizeof(unsigned), m->stream);
     cudaMemsetAsync(&H->notier[1], 0, sizeof(int), m->stream);
+    cudaMemsetAsync(H->left[1], 0, sizeof H->left[1], m->stream);
     launch_pcg(m, a);
 }
 
