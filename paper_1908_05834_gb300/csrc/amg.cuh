@@ -86,14 +86,17 @@ bool schur_pattern(bchar_mesh_t m);
 // hierarchy for them; with same_aggregates the values alone, on the aggregates
 // of the build before.
 void amg_build(bchar_mesh_t m, const IpArgs &ip, bool same_aggregates);
-// Its predictor and corrector, the step and the residuals after it.  The
-// tolerances of the two solves: z.res <= rz_rel mu, max |res_l| / b_l <=
-// max(res_rel rp_max, res_floor).
+// Its predictor and corrector, the step and the residuals after it.  A solve stops at
+// z.res <= rz_rel mu, max |res_l| / b_l <= max(res_rel rp_max, res_floor).
 struct SolveTol {
     double rz_rel, res_rel, res_floor;
-    int max_iter;   // of this solve
 };
-void pcg_launch(bchar_mesh_t m, const IpArgs &ip, const SolveTol (&tol)[2]);
+struct SolveTols {
+    SolveTol predictor, corrector, last;  // last: the corrector's once mu <= last_mu
+    double last_mu;
+    int max_iter;   // of one solve
+};
+void pcg_launch(bchar_mesh_t m, const IpArgs &ip, const SolveTols &tols);
 void amg_release(Amg &amg);
 HierView hier_view(bchar_mesh_t m);
 // Timing aids: one damped-Jacobi sweep of the finest level; one V-cycle.

@@ -67,7 +67,7 @@ struct PcgArgs {
     double *d, *r, *p0, *p1, *q, *z, *ib;     // finest level; ib: 1 / target of each constraint
     const double *b_row, *volphi;
     IpArgs ip;
-    SolveTol tol[2];  // predictor (from zero), corrector (from the predictor's d)
+    SolveTols tols;   // predictor (from zero), corrector (from the predictor's d)
     int vcycle;       // 1: one V-cycle only (timing)
 };
 
@@ -1677,9 +1677,9 @@ template <bool ONE> __global__ void __launch_bounds__(kSolveThreads, 1) k_pcg(co
         go = bar.sync();
     }
     for (int corr = 0; corr < 2 && go && !a.vcycle; ++corr) {
-        const SolveTol &tol = a.tol[corr];
+        const SolveTol &tol = corr ? (mu <= a.tols.last_mu ? a.tols.last : a.tols.corrector) : a.tols.predictor;
         const double trz = tol.rz_rel * mu, tres = fmax(tol.res_rel * rp_max, tol.res_floor);
-        const int cap = max(1, min(tol.max_iter, ip.max_cg - cg));
+        const int cap = max(1, min(a.tols.max_iter, ip.max_cg - cg));
         const int it = alone ? solve_small(a, sh, rank, nr, corr, trz, tres, cap)
                              : solve_grid_wide(a, sh, bar, corr, trz, tres, cap);
         cg += it;
@@ -1804,11 +1804,10 @@ int solve_blocks_resident() {
     return n < 1 ? kWideCluster : n * kWideCluster;
 }
 
-void pcg_launch(bchar_mesh_t m, const IpArgs &ip, const SolveTol (&tol)[2]) {
+void pcg_launch(bchar_mesh_t m, const IpArgs &ip, const SolveTols &tols) {
     PcgArgs a = pcg_args(m);
     a.ip = ip;
-    a.tol[0] = tol[0];
-    a.tol[1] = tol[1];
+    a.tols = tols;
     launch_pcg(m, a);
 }
 
