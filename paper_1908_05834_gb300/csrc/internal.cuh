@@ -174,6 +174,7 @@ struct bchar_mesh_s {
     int amg_levels = 0;
     int64_t amg_coarsest = 0;
     bool have_step = false;
+    int ip_resident = 0;     // blocks of the interior point's own kernel the device holds at once (0: not asked yet)
     int ip_iters = 0;        // interior-point iterations of the last minimisation
     bool ip_converged = false;
     int launches = 0;

@@ -39,6 +39,13 @@ static_assert(sizeof(IpScalars) <= kIpScalarBytes, "room in the host's copies");
 // After the conjugate gradients' scalars in their buffer.
 inline IpScalars *ip_scalars(bchar_mesh_t m) { return reinterpret_cast<IpScalars *>(ptr<CgState>(m->cg) + 1); }
 
+// Blocks of a kernel of these passes alone (k_ip): one per 64 rows, and never more
+// than the device holds at once, because a cooperative launch beyond that is refused.
+inline int ip_grid(int64_t nc, int resident) {
+    const int64_t most = resident < kMaxCtas ? resident : kMaxCtas, want = (nc + 63) / 64;
+    return static_cast<int>(want < 1 || most < 1 ? 1 : (want < most ? want : most));
+}
+
 struct IpArgs {
     int64_t nc, nnz;
     const int64_t *row_ptr, *col_ptr;

@@ -579,7 +579,7 @@ __global__ void k_cg_pupdate(int64_t n2, const double *z, double *p, const CgSta
 // (qp_precond = 0; with the multigrid an iteration is the two kernels of amg.cu
 // and pcg.cu).
 enum IpPart { kIpStart, kIpBegin, kIpMid, kIpEnd };
-constexpr int kIpThreads = 1024, kIpBlocks = 152;  // at 10^6 cells the loads in flight bound it
+constexpr int kIpThreads = 1024;  // one block per SM: at 10^6 cells the loads in flight bound it
 
 __global__ void __launch_bounds__(kIpThreads, 1) k_ip(const __grid_constant__ IpArgs A, int part, IpStart at) {
     __shared__ IpShared S;
@@ -600,11 +600,22 @@ __global__ void __launch_bounds__(kIpThreads, 1) k_ip(const __grid_constant__ Ip
     }
 }
 
+// The SMs of the handle's device (or of the part of it that the process may use).
+static int ip_blocks_resident(bchar_mesh_t m) {
+    int sms = 0, per_sm = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ip, kIpThreads, 0) != cudaSuccess) {
+        cudaGetLastError();
+        return 1;
+    }
+    return per_sm > 0 && sms > 0 ? sms : 1;
+}
+
 static void launch_ip(bchar_mesh_t m, const IpArgs &A, IpPart part, const IpStart &start = IpStart{}) {
     cudaMemsetAsync(&A.st->bar, 0, sizeof(unsigned), m->stream);
-    int64_t grid = (A.nc + 63) / 64;
+    if (!m->ip_resident) m->ip_resident = ip_blocks_resident(m);
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(static_cast<unsigned>(grid < kIpBlocks ? (grid < 1 ? 1 : grid) : kIpBlocks));
+    cfg.gridDim = dim3(static_cast<unsigned>(ip_grid(A.nc, m->ip_resident)));
     cfg.blockDim = dim3(kIpThreads);
     cfg.stream = m->stream;
     cudaLaunchAttribute at[1];
