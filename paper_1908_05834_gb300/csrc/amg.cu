@@ -805,27 +805,14 @@ template <int LPR, bool ONE> __global__ void __launch_bounds__(kBuildThreads, 1)
 
 // ---- host side
 
-// A finest level of at most this size is solved by one cluster: a pass of its
-// kSmallCluster blocks takes about 1 300 clocks plus 19 per FP64 warp instruction
-// (0.06 clocks per entry), one across the grid about 4 000.  Three more clusters
-// that share the passes over A's entries took 3 % off a 64^2 step alone, but a
-// batch of seven small meshes took 58 ms instead of 36: their launches no longer
-// fit side by side.
-constexpr int64_t kSmallEntries = 40000;
-constexpr int64_t kSmallNodes = 4096;
-
 SolveShape solve_shape(bchar_mesh_t m) {
     Amg &A = m->amg;
     if (!A.resident) {
-        const int n = solve_blocks_resident();
-        A.resident = n > kMaxCtas ? kMaxCtas / kWideCluster * kWideCluster : n;
+        const SolveRoom r = solve_room();
+        A.resident = r.blocks;
+        A.small_fits = r.small && build_cluster_fits();
     }
-    if (A.e0 <= kSmallEntries && A.n0 <= kSmallNodes) return {kSmallCluster, kSmallCluster, 1};
-    // one block per ~300 entries (two warps of rows), as many as the device holds
-    int64_t g = (A.e0 / 300 + kWideCluster - 1) / kWideCluster * kWideCluster;
-    if (g < 2 * kWideCluster) g = 2 * kWideCluster;
-    if (g > A.resident) g = A.resident;
-    return {static_cast<int>(g), kWideCluster, 0};
+    return solve_shape_of(A.e0, A.n0, {A.resident, A.small_fits});
 }
 
 // All blocks resident at once: one cluster, or a cooperative launch.
@@ -850,6 +837,17 @@ static void launch_resident(void (*kernel)(P...), int grid, bool cluster, int bl
     cfg.attrs = at;
     cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+bool build_cluster_fits() {
+    int n = 0, least = 1 << 30;
+    for (auto k : {k_amg_build<4, true>, k_amg_build<16, true>}) {
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBuildSmem));
+        cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (!clusters_resident(k, kSmallCluster, kBuildThreads, kBuildSmem, &n)) return false;
+        least = n < least ? n : least;
+    }
+    return least >= 1;
 }
 
 HierView hier_view(bchar_mesh_t m) {

@@ -77,8 +77,51 @@ struct SolveShape {
     int grid, cluster, small;
 };
 struct IpArgs;  // ip.cuh
+// The clusters of a kernel that the current device holds at once (false: it refuses the shape).
+template <class K> inline bool clusters_resident(K kernel, int cluster, int threads, size_t smem, int *n) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(cluster);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cluster;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(n, kernel, &cfg) == cudaSuccess) return true;
+    cudaGetLastError();
+    return false;
+}
+// What a device holds at once of the solve and build kernels.
+struct SolveRoom {
+    int blocks = 0;       // of clusters of kWideCluster, one block per SM (0: not asked yet)
+    bool small = false;   // one cluster of kSmallCluster
+};
+SolveRoom solve_room();  // pcg.cu (asks the device)
+bool build_cluster_fits();  // amg.cu: one cluster of kSmallCluster of the build
 SolveShape solve_shape(bchar_mesh_t m);
-int solve_blocks_resident();  // pcg.cu
+
+// A finest level of at most this size is solved by one cluster: a pass of its
+// kSmallCluster blocks takes about 1 300 clocks plus 19 per FP64 warp instruction
+// (0.06 clocks per entry), one across the grid about 4 000.  Three more clusters
+// that share the passes over A's entries took 3 % off a 64^2 step alone, but a
+// batch of seven small meshes took 58 ms instead of 36: their launches no longer
+// fit side by side.
+constexpr int64_t kSmallEntries = 40000;
+constexpr int64_t kSmallNodes = 4096;
+
+inline SolveShape solve_shape_of(int64_t e0, int64_t n0, const SolveRoom &room) {
+    if (room.small && e0 <= kSmallEntries && n0 <= kSmallNodes) return {kSmallCluster, kSmallCluster, 1};
+    // one block per ~300 entries (two warps of rows), as many as the device holds
+    int64_t g = (e0 / 300 + kWideCluster - 1) / kWideCluster * kWideCluster;
+    if (g < 2 * kWideCluster) g = 2 * kWideCluster;
+    const int most = kMaxCtas / kWideCluster * kWideCluster;
+    if (g > most) g = most;
+    if (g > room.blocks) g = room.blocks;
+    return {static_cast<int>(g), kWideCluster, 0};
+}
 
 // Once per step: the finest level's pattern (false: out of memory).
 bool schur_pattern(bchar_mesh_t m);

@@ -109,7 +109,8 @@ struct Amg {
     Buf scratch, vec;                                     // matching scratch; vectors of the conjugate gradients
     int64_t n0 = 0, e0 = 0;      // nodes and entries of the finest level
     int64_t capn = 0, cape = 0;  // room in the level arrays
-    int resident = 0;            // blocks of the solve kernel the device holds at once
+    int resident = 0;            // blocks of the solve kernel the device holds at once (0: not asked yet)
+    bool small_fits = false;     // whether it holds the cluster that small systems are solved by
     bool schur = false;          // finest level: the columns, rows eliminated (else rows and columns)
 };
 

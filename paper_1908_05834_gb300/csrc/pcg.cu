@@ -1782,26 +1782,16 @@ static void launch_pcg(bchar_mesh_t m, PcgArgs &a) {
     ++m->launches;
 }
 
-// Blocks of 8-block clusters that the device holds at once (one block per SM).
-int solve_blocks_resident() {
+SolveRoom solve_room() {
+    cudaFuncSetAttribute(k_pcg<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSolveSmem));
     cudaFuncSetAttribute(k_pcg<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSolveSmem));
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(kWideCluster);
-    cfg.blockDim = dim3(kSolveThreads);
-    cfg.dynamicSmemBytes = kSolveSmem;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = kWideCluster;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cudaFuncSetAttribute(k_pcg<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    SolveRoom r;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, k_pcg<false>, &cfg) != cudaSuccess) {
-        cudaGetLastError();
-        n = 1;
-    }
-    return n < 1 ? kWideCluster : n * kWideCluster;
+    r.blocks = kWideCluster;
+    if (clusters_resident(k_pcg<false>, kWideCluster, kNT, kSolveSmem, &n) && n > 1) r.blocks = n * kWideCluster;
+    r.small = clusters_resident(k_pcg<true>, kSmallCluster, kNT, kSolveSmem, &n) && n >= 1;
+    return r;
 }
 
 void pcg_launch(bchar_mesh_t m, const IpArgs &ip, const SolveTols &tols) {

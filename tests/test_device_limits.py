@@ -39,3 +39,27 @@ int main() {
         assert grid <= max(1, (cells + 63) // 64)
         if resident <= 152:
             assert grid == min(resident, (cells + 63) // 64)
+
+
+@needs_nvcc
+def test_solver_grid_fits_the_device(tmp_path):
+    """Small systems take one cluster of 16 blocks only where the device holds one; else
+    they, like the larger ones, take clusters of 8, no more blocks than fit."""
+    for fits, blocks, entries, nodes, grid, cluster, small in _run(tmp_path, r"""
+#include <cstdio>
+#include "amg.cuh"
+int main() {
+    for (int fits : {0, 1})
+        for (int blocks : {8, 24, 144, 152, 400})
+            for (long long e0 : {0ll, 1ll, 40000ll, 40001ll, 6000000ll})
+                for (long long n0 : {1ll, 4096ll, 4097ll}) {
+                    const bchar::SolveShape s = bchar::solve_shape_of(e0, n0, {blocks, fits != 0});
+                    std::printf("%d %d %lld %lld %d %d %d\n", fits, blocks, e0, n0, s.grid, s.cluster, s.small);
+                }
+}
+"""):
+        assert small == (fits and entries <= 40000 and nodes <= 4096)
+        if small:
+            assert (grid, cluster) == (16, 16)
+        else:
+            assert cluster == 8 and grid % 8 == 0 and 8 <= grid <= min(blocks, 256)
