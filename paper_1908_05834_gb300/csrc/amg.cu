@@ -839,11 +839,16 @@ static void launch_resident(void (*kernel)(P...), int grid, bool cluster, int bl
     cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+void amg_opt_in() {
+    for (auto k : {k_amg_build<4, false>, k_amg_build<16, false>, k_amg_build<4, true>, k_amg_build<16, true>}) {
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBuildSmem));
+        cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    }
+}
+
 bool build_cluster_fits() {
     int n = 0, least = 1 << 30;
     for (auto k : {k_amg_build<4, true>, k_amg_build<16, true>}) {
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBuildSmem));
-        cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (!clusters_resident(k, kSmallCluster, kBuildThreads, kBuildSmem, &n)) return false;
         least = n < least ? n : least;
     }
@@ -900,15 +905,6 @@ void amg_build(bchar_mesh_t m, const IpArgs &ip, bool same_aggregates) {
     }
     a.ip = ip;
     a.same = same_aggregates ? 1 : 0;
-    static bool attrs = false;  // opt-ins of the kernels (harmless to repeat)
-    if (!attrs) {
-        void (*const all[])(BuildArgs) = {k_amg_build<4, false>, k_amg_build<16, false>, k_amg_build<4, true>, k_amg_build<16, true>};
-        for (auto k : all) {
-            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBuildSmem));
-            cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        }
-        attrs = true;
-    }
     const SolveShape shape = solve_shape(m);
     const bool few = A.e0 <= 10 * A.n0;  // lanes per row
     launch_resident(shape.small ? (few ? k_amg_build<4, true> : k_amg_build<16, true>)

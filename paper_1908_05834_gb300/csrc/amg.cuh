@@ -99,6 +99,8 @@ struct SolveRoom {
     int blocks = 0;       // of clusters of kWideCluster, one block per SM (0: not asked yet)
     bool small = false;   // one cluster of kSmallCluster
 };
+void pcg_opt_in();  // before the first launch on a device, like tiles_opt_in
+void amg_opt_in();
 SolveRoom solve_room();  // pcg.cu (asks the device)
 bool build_cluster_fits();  // amg.cu: one cluster of kSmallCluster of the build
 SolveShape solve_shape(bchar_mesh_t m);

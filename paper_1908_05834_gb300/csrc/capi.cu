@@ -396,6 +396,12 @@ bchar_status bchar_step(bchar_mesh_t m, double dt, const void *c_in, void *c_out
         for (cudaEvent_t &e : m->stage_ev)
             if (cudaEventCreate(&e) != cudaSuccess) return cuda_check(m);
     cudaEvent_t *ev = m->stage_ev;
+    if (!m->opted_in) {
+        tiles_opt_in();
+        amg_opt_in();
+        pcg_opt_in();
+        m->opted_in = true;
+    }
     cudaEventRecord(ev[0], m->stream);
 
     // substeps: the smallest s with dt * vmax / s <= cfl * hmin

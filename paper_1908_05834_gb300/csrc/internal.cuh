@@ -175,6 +175,7 @@ struct bchar_mesh_s {
     int amg_levels = 0;
     int64_t amg_coarsest = 0;
     bool have_step = false;
+    bool opted_in = false;   // the kernels' opt-ins are set (an attribute of a function is one device's)
     int ip_resident = 0;     // blocks of the interior point's own kernel the device holds at once (0: not asked yet)
     int ip_iters = 0;        // interior-point iterations of the last minimisation
     bool ip_converged = false;
@@ -258,6 +259,7 @@ VelView vel_view(bchar_mesh_t m);
 // sparse.cu
 void scan_i32_to_i64(bchar_mesh_t m, const int32_t *in, int64_t *out, int64_t n);  // out has n + 1 entries
 void launch_transpose(bchar_mesh_t m);
+void tiles_opt_in();  // the opt-ins of the kernels with large shared memory or clusters, on the current device
 bool launch_tiles(bchar_mesh_t m);  // tile boundaries of both views (false: out of memory)
 bool launch_balance(bchar_mesh_t m);  // components.cu
 void launch_scaling(bchar_mesh_t m);

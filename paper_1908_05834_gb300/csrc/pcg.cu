@@ -1756,13 +1756,6 @@ static PcgArgs pcg_args(bchar_mesh_t m) {
 }
 
 static void launch_pcg(bchar_mesh_t m, PcgArgs &a) {
-    static bool attrs = false;  // opt-ins of the kernel (harmless to repeat)
-    if (!attrs) {
-        cudaFuncSetAttribute(k_pcg<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSolveSmem));
-        cudaFuncSetAttribute(k_pcg<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSolveSmem));
-        cudaFuncSetAttribute(k_pcg<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        attrs = true;
-    }
     const SolveShape s = solve_shape(m);
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(s.grid);
@@ -1782,10 +1775,13 @@ static void launch_pcg(bchar_mesh_t m, PcgArgs &a) {
     ++m->launches;
 }
 
-SolveRoom solve_room() {
+void pcg_opt_in() {
     cudaFuncSetAttribute(k_pcg<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSolveSmem));
     cudaFuncSetAttribute(k_pcg<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSolveSmem));
     cudaFuncSetAttribute(k_pcg<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+}
+
+SolveRoom solve_room() {
     SolveRoom r;
     int n = 0;
     r.blocks = kWideCluster;

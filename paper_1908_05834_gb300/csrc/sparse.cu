@@ -236,16 +236,15 @@ __global__ void k_cg_matvec(LineView Vr, LineView Vc, const double *diag, const 
                             double *partials, const CgState *st);
 template <class T> __global__ void k_spmv(LineView V, const double *volphi, const T *c_in, T *c_out, double *partials);
 
+void tiles_opt_in() {
+    allow_tile_smem(k_scale_tiles);
+    allow_tile_smem(k_scaled_col_error);
+    allow_tile_smem(k_cg_matvec);
+    allow_tile_smem(k_spmv<float>);
+    allow_tile_smem(k_spmv<double>);
+}
+
 bool launch_tiles(bchar_mesh_t m) {
-    static bool attrs = false;  // the shared-memory opt-in of the tile kernels (per process; harmless to repeat)
-    if (!attrs) {
-        allow_tile_smem(k_scale_tiles);
-        allow_tile_smem(k_scaled_col_error);
-        allow_tile_smem(k_cg_matvec);
-        allow_tile_smem(k_spmv<float>);
-        allow_tile_smem(k_spmv<double>);
-        attrs = true;
-    }
     m->ntile = tile_count(m->nnz);
     const size_t b = sizeof(int32_t) * (m->ntile + 1);
     if (!ensure(m, m->tile_r, b) || !ensure(m, m->tile_c, b)) return false;

@@ -2,6 +2,7 @@
 constants were chosen on: the sizes of the resident grids, as host functions.
 """
 import os
+import re
 import shutil
 import subprocess
 
@@ -63,3 +64,16 @@ int main() {
             assert (grid, cluster) == (16, 16)
         else:
             assert cluster == 8 and grid % 8 == 0 and 8 <= grid <= min(blocks, 256)
+
+
+def test_opt_ins_are_not_kept_per_process():
+    """A function's attributes are one device's: a flag that outlives the handle would
+    leave them unset on the second device that a process uses (and its threads would race on it)."""
+    flag = re.compile(r"^\s+static (?!const\b|constexpr\b|__|std::mutex\b)\w[\w<>:\s*]*?(\w+)\s*(\[\w*\])?\s*(=|;|\{\})", re.M)
+    for name in sorted(os.listdir(CSRC)):
+        with open(os.path.join(CSRC, name)) as f:
+            found = [m.group(0).strip() for m in flag.finditer(f.read())]
+        if name == "noalloc.cu":  # an address per device, behind a lock
+            assert found == ["static double *addr[256] ="]
+        else:
+            assert not found, (name, found)
