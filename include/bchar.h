@@ -268,10 +268,11 @@ bchar_status bchar_device_bytes(bchar_mesh_t m, int64_t *now, int64_t *peak);
 
 /* A-priori estimate (bytes) of the device memory a handle created with these
  * arguments will hold after its steps, for admission control before any
- * allocation: per cell (mesh arrays, minimisation vectors, row slab,
- * multigrid), per ball (the tight packing, counted here from the widths)
- * and per matrix entry, with the entries bounded by a 3^d neighbourhood per
- * row (9 in 2D, 27 in 3D), plus 10 %.  Rows wider than the slab's 24 (2D)
+ * allocation: per cell (mesh arrays, minimisation vectors, row slab), per
+ * ball (the tight packing, counted here from the widths), per matrix entry,
+ * with the entries bounded by a 3^d neighbourhood per row (9 in 2D, 27 in
+ * 3D), and the linear solver's, at the limits of the rule that chooses its
+ * form, plus 10 %.  Rows wider than the slab's 24 (2D)
  * or 64 (3D) entries are held at their exact length in a spill area, which the
  * per-entry count covers.  Host only; no GPU work.  coords as for
  * bchar_create_mesh; opt NULL = defaults.

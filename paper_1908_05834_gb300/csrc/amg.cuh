@@ -125,6 +125,31 @@ inline SolveShape solve_shape_of(int64_t e0, int64_t n0, const SolveRoom &room) 
     return {static_cast<int>(g), kWideCluster, 0};
 }
 
+// The limits of the system with the rows eliminated, per entry of A (schur.cu): the
+// contributions (pairs of entries of one row of A), and its entries.  At 12 pairs it
+// holds about five entries per entry of A where the product through the two views
+// touches two (measured 4.1 to 5.3 between 9 and 17 pairs); the recipes' matrices have
+// 2 to 5.  The second limit only bounds the memory.
+constexpr int64_t kMaxPairs = 12, kMaxFill = 6;
+// Room in the level arrays: all levels together, of the finest level's nodes and entries.
+constexpr int64_t kRoomNodes10 = 26, kRoomEntries = 4;
+
+// Bytes per cell of schur_pattern's buffers, at most, where A's rows hold `rows` entries
+// in the mean and an entry of A costs per_entry bytes besides: the larger of the two
+// forms, as the difference to per_entry * rows.  Buffers have an eighth to spare.
+inline double solver_bytes_per_cell(double rows, double per_entry) {
+    // per node: rs, three or five arrays of each type (72 bytes), eight of the matching's, seven vectors
+    const double node = 1.125 * (72.0 * kRoomNodes10 / 10 + 8 * 4 + 7 * 8);
+    const double cell = 8 + 4 + 8, entry = 1.125 * 8;  // t, counts and offsets of the contributions; g
+    const double both = 2 * node + cell + rows * (entry + 1.125 * 12 * kRoomEntries * 2);
+    // at most kMaxPairs contributions per entry: the squares of the row lengths sum to at most
+    // (kMaxPairs + 1) times their sum, so a row has at most kMaxPairs + 1 entries in the mean
+    const double r = rows < kMaxPairs + 1 ? rows : kMaxPairs + 1;
+    const double eliminated = node + cell + r * (entry + 1.125 * (12 * kMaxPairs + (12 * kRoomEntries + 4) * kMaxFill));
+    const double e = eliminated - per_entry * (rows - r);
+    return both > e ? both : e;
+}
+
 // Once per step: the finest level's pattern (false: out of memory).
 bool schur_pattern(bchar_mesh_t m);
 // An interior-point iteration: the weights of the normal equations and the

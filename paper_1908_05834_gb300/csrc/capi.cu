@@ -272,10 +272,10 @@ bchar_status bchar_create_mesh(int dim, const int64_t *n_cells, const double *co
          ensure(m, m->diag, sizeof(double) * 2 * nc) && ensure(m, m->rhs, sizeof(double) * 2 * nc) &&
          ensure(m, m->qexc, sizeof(double) * 2 * nc) &&
          ensure(m, m->qy, sizeof(double) * 2 * nc) && ensure(m, m->F, sizeof(double) * 2 * nc) &&
-         ensure(m, m->cg_d, sizeof(double) * 2 * nc) && ensure(m, m->cg_r, sizeof(double) * 2 * nc) &&
-         ensure(m, m->cg_z, sizeof(double) * 2 * nc) && ensure(m, m->cg_p, sizeof(double) * 2 * nc) &&
-         ensure(m, m->cg_q, sizeof(double) * 2 * nc) && ensure(m, m->cg_rp, sizeof(double) * 2 * nc) && ensure(m, m->partials, sizeof(double) * 4 * 152 * 64) &&
+         ensure(m, m->cg_d, sizeof(double) * 2 * nc) && ensure(m, m->partials, sizeof(double) * 4 * 152 * 64) &&
          ensure(m, m->dinfo, sizeof(DevInfo)) && ensure(m, m->cg, sizeof(CgState));
+    if (o.qp_precond == 0)  // the other vectors of that solver (the multigrid's are in its own buffers)
+        for (Buf *b : {&m->cg_r, &m->cg_z, &m->cg_p, &m->cg_q, &m->cg_rp}) ok = ok && ensure(m, *b, sizeof(double) * 2 * nc);
     if (ok && cudaMallocHost(&m->info_host.p, sizeof(DevInfo) + sizeof(CgState) + 2 * kIpScalarBytes) != cudaSuccess) {
         cudaGetLastError();
         m->info_host.p = nullptr;
@@ -585,21 +585,20 @@ bchar_status bchar_estimate_device_bytes(int dim, const int64_t *n_cells, const 
         nballs += cnt;
     }
     // bytes per cell, per ball and per matrix entry of every buffer a step holds:
-    // mesh and row arrays 116, minimisation vectors 2 x 11 x 8, union-find 80,
+    // mesh and row arrays 116, minimisation vectors 2 x 6 x 8, union-find 80,
     // face velocities 12 d, tracking records kRecordLen x precision, row slab
-    // 12 row_cap, matching scratch 48, multigrid level 0 144 and coarser levels
-    // ~154, interior-point state of the 2 constraint nodes 2 x 10 x 8, spill
-    // counts and offsets 12; per entry: CSR and column view 68, multigrid
-    // level 0 48 and coarser ~50, interior-point state 12 x 8, spill area at
-    // most 12; per ball 8 + 4 (3 + 1) x precision.
+    // 12 row_cap, interior-point state of the 2 constraint nodes 2 x 10 x 8, spill
+    // counts and offsets 12; per entry: CSR and column view 68, interior-point
+    // state 12 x 8, spill area at most 12; per ball 8 + 4 (3 + 1) x precision.
     const int row_cap = o.slab_width > 0 ? o.slab_width : (dim == 2 ? 24 : 64);
     const double rec = kRecordLen * (o.precision == BCHAR_FP32_SPLIT ? 4.0 : 8.0);
-    const double per_cell = 116 + 176 + 80 + 12.0 * dim + rec + 12.0 * row_cap + 48 + 144 + 154 + 160 + 12;
-    const double per_entry = 68 + 48 + 50 + 96 + 12;
+    const double per_cell = 116 + 96 + 80 + 12.0 * dim + rec + 12.0 * row_cap + 160 + 12;
+    const double per_entry = 68 + 96 + 12;
     const double per_ball = 8 + 4.0 * (o.precision == BCHAR_FP32_SPLIT ? 4 : 8);
-    const double nnz_bound = (dim == 2 ? 9.0 : 27.0) * nc;  // a 3^d neighbourhood per row
+    const double rows = dim == 2 ? 9.0 : 27.0;  // entries per row: a 3^d neighbourhood
+    const double solver = o.qp_precond == 0 ? 80.0 : solver_bytes_per_cell(rows, per_entry);
     const double fixed = 4.0 * 152 * 64 * 8 + 4096 * 8 + (1 << 20);
-    *bytes = static_cast<int64_t>(1.1 * (per_cell * nc + per_entry * nnz_bound + per_ball * nballs + fixed));
+    *bytes = static_cast<int64_t>(1.1 * ((per_cell + per_entry * rows + solver) * nc + per_ball * nballs + fixed));
     return BCHAR_OK;
 }
 
@@ -616,6 +615,16 @@ bchar_status bchar_time_stage(bchar_mesh_t m, int stage, int reps, float *mean_m
         release(cout);
         return BCHAR_ERR_OUT_OF_MEMORY;
     }
+    if (stage == BCHAR_STAGE_CG_MATVEC && !m->cg_p.p)  // a handle with the multigrid: the product's vectors are not there
+        for (Buf *b : {&m->cg_p, &m->cg_q}) {
+            if (!ensure(m, *b, sizeof(double) * 2 * m->nc)) {
+                release(st);
+                release(cin);
+                release(cout);
+                return BCHAR_ERR_OUT_OF_MEMORY;
+            }
+            cudaMemsetAsync(b->p, 0, sizeof(double) * 2 * m->nc, m->stream);
+        }
     cudaMemsetAsync(st.p, 0, sizeof(CgState), m->stream);
     cudaMemsetAsync(cin.p, 0, sizeof(double) * m->nc, m->stream);
     // the final weights are kept in wgt; the slab of the assembly is scratch

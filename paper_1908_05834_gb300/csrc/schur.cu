@@ -12,8 +12,8 @@
 // contributions of every entry (pairs of entries of one row of A) in a fixed
 // order; each interior-point iteration then only sums products (amg.cu).  A
 // matrix whose rows are so long that the products would outweigh the gain
-// (more than kMaxPairs contributions per entry of A), or one column collects
-// more than kBlockPairs, keeps rows and columns as they are.
+// (more than kMaxPairs contributions or kMaxFill entries per entry of A), or where
+// one column collects more than kBlockPairs, keeps rows and columns as they are.
 #include "amg.cuh"
 #include "device.cuh"
 
@@ -23,9 +23,6 @@ constexpr int kWarpPairs = 512;    // contributions of a column sorted by one wa
 constexpr int kBlockPairs = 8192;  // by one block
 static_assert(kWarpPairs >= 32 && (kWarpPairs & (kWarpPairs - 1)) == 0 && (kBlockPairs & (kBlockPairs - 1)) == 0,
               "the sorts pad to a power of two of at least 32");
-// S then holds about six entries per entry of A where the product through the
-// two views touches two; the recipes' matrices have 1.5 to 8.
-constexpr int64_t kMaxPairs = 12;
 constexpr size_t kBlockPairSmem = static_cast<size_t>(kBlockPairs) * (sizeof(unsigned long long) + sizeof(int2));
 
 struct PairStat {
@@ -216,76 +213,95 @@ static bool ensure_more(bchar_mesh_t m, Buf &b, size_t bytes) {
     return (b.p && b.bytes >= bytes) || ensure(m, b, bytes + bytes / 8);
 }
 
+// The arrays of a system of n0 nodes, its hierarchy and its conjugate gradients.
+static bool node_buffers(bchar_mesh_t m, int64_t n0) {
+    Amg &A = m->amg;
+    A.n0 = n0;
+    A.capn = n0 * kRoomNodes10 / 10 + 256;
+    const size_t cn = static_cast<size_t>(A.capn);
+    for (Buf *b : {&A.dg, &A.ex, &A.om, &A.x, &A.b})
+        if (!ensure_more(m, *b, sizeof(double) * cn)) return false;
+    for (Buf *b : {&A.rl, &A.own, &A.gs, &A.gc, &A.agg, &A.raw})
+        if (!ensure_more(m, *b, sizeof(int32_t) * cn)) return false;
+    return ensure_more(m, A.rs, sizeof(int64_t) * cn) && ensure_more(m, A.scratch, sizeof(int32_t) * 8 * n0) &&
+           ensure_more(m, A.vec, sizeof(double) * 7 * n0);
+}
+
+static bool entry_buffers(bchar_mesh_t m, int64_t e0) {
+    Amg &A = m->amg;
+    A.e0 = e0;
+    A.cape = kRoomEntries * e0 + 4096;
+    return ensure_more(m, A.ecol, sizeof(int32_t) * A.cape) && ensure_more(m, A.ew, sizeof(double) * A.cape);
+}
+
+// The system with the rows eliminated; A.schur is false on return when it has more
+// than kMaxFill entries per entry of A.  False: out of memory.
+static bool eliminated_form(bchar_mesh_t m, const PairStat &h) {
+    Amg &A = m->amg;
+    cudaStream_t s = m->stream;
+    const int64_t nc = m->nc;
+    const int64_t *row_ptr = ptr<int64_t>(m->row_ptr), *col_ptr = ptr<int64_t>(m->col_ptr);
+    const int32_t *col = ptr<int32_t>(m->col), *csc_row = ptr<int32_t>(m->csc_row), *csc_src = ptr<int32_t>(m->csc_src);
+    const size_t tot = h.total > 0 ? static_cast<size_t>(h.total) : 1;
+    if (!node_buffers(m, nc) || !ensure_more(m, A.raw_key, sizeof(int32_t) * tot) ||
+        !ensure_more(m, A.pair, sizeof(int2) * tot))
+        return false;
+    int32_t *cnt = ptr<int32_t>(A.raw_cnt), *key = ptr<int32_t>(A.raw_key), *rl = ptr<int32_t>(A.rl);
+    int64_t *off = ptr<int64_t>(A.raw_off), *rs = ptr<int64_t>(A.rs);
+    scan_i32_to_i64(m, cnt, off, nc);
+    k_schur_columns<<<blocks_for(nc * 32, 128), 128, 0, s>>>(nc, row_ptr, col, col_ptr, csc_row, csc_src, cnt, off, key,
+                                                             ptr<int2>(A.pair), rl);
+    ++m->launches;
+    if (h.most > kWarpPairs) {
+        cudaFuncSetAttribute(k_schur_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kBlockPairSmem));
+        k_schur_wide<<<static_cast<int>(nc < 152 ? nc : 152), 1024, kBlockPairSmem, s>>>(
+            nc, row_ptr, col, col_ptr, csc_row, csc_src, cnt, off, key, ptr<int2>(A.pair), rl);
+        ++m->launches;
+    }
+    scan_i32_to_i64(m, rl, rs, nc);
+    int64_t e0 = 0;
+    cudaMemcpyAsync(&e0, rs + nc, sizeof e0, cudaMemcpyDeviceToHost, s);
+    if (cudaStreamSynchronize(s) != cudaSuccess) return true;  // the caller reads the error
+    A.schur = e0 <= kMaxFill * m->nnz;
+    if (!A.schur) return true;
+    if (!entry_buffers(m, e0) || !ensure_more(m, A.cs, sizeof(uint32_t) * (e0 + 1))) return false;
+    k_schur_entries<<<blocks_for(nc * 32), kThreads, 0, s>>>(nc, cnt, off, key, rs, ptr<int32_t>(A.ecol), ptr<uint32_t>(A.cs));
+    ++m->launches;
+    return true;
+}
+
+static bool bipartite_form(bchar_mesh_t m) {
+    Amg &A = m->amg;
+    for (Buf *b : {&A.raw_key, &A.pair, &A.cs}) release(*b);  // of an eliminated system before
+    if (!node_buffers(m, 2 * m->nc) || !entry_buffers(m, 2 * m->nnz)) return false;
+    k_bipartite_rows<<<blocks_for(2 * m->nc), kThreads, 0, m->stream>>>(
+        m->nc, m->nnz, ptr<int64_t>(m->row_ptr), ptr<int32_t>(m->col), ptr<int64_t>(m->col_ptr), ptr<int32_t>(m->csc_row),
+        ptr<int64_t>(A.rs), ptr<int32_t>(A.rl), ptr<int32_t>(A.ecol));
+    ++m->launches;
+    return true;
+}
+
 bool schur_pattern(bchar_mesh_t m) {
     Amg &A = m->amg;
     cudaStream_t s = m->stream;
     const int64_t nc = m->nc, nnz = m->nnz;
-    const int64_t *row_ptr = ptr<int64_t>(m->row_ptr), *col_ptr = ptr<int64_t>(m->col_ptr);
-    const int32_t *col = ptr<int32_t>(m->col), *csc_row = ptr<int32_t>(m->csc_row), *csc_src = ptr<int32_t>(m->csc_src);
     if (!ensure(m, A.hier, sizeof(Hier)) || !ensure(m, A.seg, sizeof(Seg) * kMaxLevels * kMaxCtas) ||
         !ensure(m, A.stat, sizeof(PairStat)) || !ensure(m, A.raw_cnt, sizeof(int32_t) * nc) ||
-        !ensure(m, A.raw_off, sizeof(int64_t) * (nc + 1)))
+        !ensure(m, A.raw_off, sizeof(int64_t) * (nc + 1)) || !ensure(m, A.t, sizeof(double) * nc) ||
+        !ensure_more(m, A.g, sizeof(double) * (nnz > 0 ? nnz : 1)))
         return false;
     PairStat *st = ptr<PairStat>(A.stat);
     cudaMemsetAsync(st, 0, sizeof(PairStat), s);
-    k_pair_counts<<<blocks_for(nc), kThreads, 0, s>>>(nc, row_ptr, col_ptr, csc_row, ptr<int32_t>(A.raw_cnt), st);
+    k_pair_counts<<<blocks_for(nc), kThreads, 0, s>>>(nc, ptr<int64_t>(m->row_ptr), ptr<int64_t>(m->col_ptr),
+                                                      ptr<int32_t>(m->csc_row), ptr<int32_t>(A.raw_cnt), st);
     ++m->launches;
     PairStat h{};
     cudaMemcpyAsync(&h, st, sizeof h, cudaMemcpyDeviceToHost, s);
     if (cudaStreamSynchronize(s) != cudaSuccess) return true;  // the caller reads the error
     A.schur = h.most <= kBlockPairs && h.total <= static_cast<unsigned long long>(kMaxPairs * nnz) &&
               h.total < 0xffffffffull;
-    A.n0 = A.schur ? nc : 2 * nc;
-    A.capn = A.n0 * 13 / 5 + 256;
-    const size_t cn = static_cast<size_t>(A.capn);
-    Buf *dbl[] = {&A.dg, &A.ex, &A.om, &A.x, &A.b};
-    for (Buf *b : dbl)
-        if (!ensure_more(m, *b, sizeof(double) * cn)) return false;
-    Buf *i32[] = {&A.rl, &A.own, &A.gs, &A.gc, &A.agg, &A.raw};
-    for (Buf *b : i32)
-        if (!ensure_more(m, *b, sizeof(int32_t) * cn)) return false;
-    if (!ensure_more(m, A.rs, sizeof(int64_t) * cn) || !ensure_more(m, A.scratch, sizeof(int32_t) * 8 * A.n0) ||
-        !ensure_more(m, A.vec, sizeof(double) * 7 * A.n0) || !ensure_more(m, A.g, sizeof(double) * (nnz > 0 ? nnz : 1)) ||
-        !ensure(m, A.t, sizeof(double) * nc))
-        return false;
-    if (A.schur) {
-        const size_t tot = h.total > 0 ? static_cast<size_t>(h.total) : 1;
-        if (!ensure_more(m, A.raw_key, sizeof(int32_t) * tot) || !ensure_more(m, A.pair, sizeof(int2) * tot)) return false;
-        scan_i32_to_i64(m, ptr<int32_t>(A.raw_cnt), ptr<int64_t>(A.raw_off), nc);
-        k_schur_columns<<<blocks_for(nc * 32, 128), 128, 0, s>>>(
-            nc, row_ptr, col, col_ptr, csc_row, csc_src, ptr<int32_t>(A.raw_cnt), ptr<int64_t>(A.raw_off),
-            ptr<int32_t>(A.raw_key), ptr<int2>(A.pair), ptr<int32_t>(A.rl));
-        ++m->launches;
-        if (h.most > kWarpPairs) {
-            cudaFuncSetAttribute(k_schur_wide, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(kBlockPairSmem));
-            k_schur_wide<<<static_cast<int>(nc < 152 ? nc : 152), 1024, kBlockPairSmem, s>>>(
-                nc, row_ptr, col, col_ptr, csc_row, csc_src, ptr<int32_t>(A.raw_cnt), ptr<int64_t>(A.raw_off),
-                ptr<int32_t>(A.raw_key), ptr<int2>(A.pair), ptr<int32_t>(A.rl));
-            ++m->launches;
-        }
-        scan_i32_to_i64(m, ptr<int32_t>(A.rl), ptr<int64_t>(A.rs), nc);
-        int64_t e0 = 0;
-        cudaMemcpyAsync(&e0, ptr<int64_t>(A.rs) + nc, sizeof e0, cudaMemcpyDeviceToHost, s);
-        if (cudaStreamSynchronize(s) != cudaSuccess) return true;
-        A.e0 = e0;
-    } else {
-        A.e0 = 2 * nnz;
-    }
-    A.cape = 4 * A.e0 + 4096;
-    if (!ensure_more(m, A.ecol, sizeof(int32_t) * A.cape) || !ensure_more(m, A.ew, sizeof(double) * A.cape) ||
-        !ensure_more(m, A.cs, sizeof(uint32_t) * (A.schur ? A.e0 + 1 : 1)))
-        return false;
-    if (A.schur)
-        k_schur_entries<<<blocks_for(nc * 32), kThreads, 0, s>>>(nc, ptr<int32_t>(A.raw_cnt), ptr<int64_t>(A.raw_off),
-                                                                 ptr<int32_t>(A.raw_key), ptr<int64_t>(A.rs),
-                                                                 ptr<int32_t>(A.ecol), ptr<uint32_t>(A.cs));
-    else
-        k_bipartite_rows<<<blocks_for(2 * nc), kThreads, 0, s>>>(nc, nnz, row_ptr, col, col_ptr, csc_row,
-                                                                 ptr<int64_t>(A.rs), ptr<int32_t>(A.rl),
-                                                                 ptr<int32_t>(A.ecol));
-    ++m->launches;
-    return true;
+    if (A.schur && !eliminated_form(m, h)) return false;
+    return A.schur || bipartite_form(m);
 }
 
 }  // namespace bchar
