@@ -210,7 +210,7 @@ __global__ void k_bipartite_rows(int64_t nc, int64_t nnz, const int64_t *row_ptr
 // A buffer with an eighth to spare, so that the next steps' slightly larger
 // matrices do not reallocate it.
 static bool ensure_more(bchar_mesh_t m, Buf &b, size_t bytes) {
-    return (b.p && b.bytes >= bytes) || ensure(m, b, bytes + bytes / 8);
+    return (b.p && b.bytes >= bytes) || ensure(m, b, bytes + bytes / 8) || ensure(m, b, bytes);
 }
 
 // The arrays of a system of n0 nodes, its hierarchy and its conjugate gradients.
@@ -300,7 +300,12 @@ bool schur_pattern(bchar_mesh_t m) {
     if (cudaStreamSynchronize(s) != cudaSuccess) return true;  // the caller reads the error
     A.schur = h.most <= kBlockPairs && h.total <= static_cast<unsigned long long>(kMaxPairs * nnz) &&
               h.total < 0xffffffffull;
-    if (A.schur && !eliminated_form(m, h)) return false;
+    if (A.schur && !eliminated_form(m, h)) {
+        // no room for it: at ten entries per row it takes twice what rows and columns do
+        for (Buf *b : {&A.raw_key, &A.pair, &A.cs, &A.ecol, &A.ew}) release(*b);
+        A.schur = false;
+        m->err.clear();
+    }
     return A.schur || bipartite_form(m);
 }
 
