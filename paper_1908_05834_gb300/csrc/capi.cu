@@ -172,7 +172,8 @@ void bchar_destroy(bchar_mesh_t m) {
                   &m->cg_q, &m->cg_rp, &m->scan_tmp, &m->partials, &m->dinfo, &m->cg, &m->ip_f, &m->ip_u,
                   &m->ip_zl, &m->ip_zh, &m->ip_D, &m->ip_q, &m->ip_cl, &m->ip_ch, &m->ip_df, &m->ip_du,
                   &m->ip_dzl, &m->ip_dzh, &m->ip_p, &m->ip_n, &m->ip_zp, &m->ip_zn, &m->ip_cp, &m->ip_cn,
-                  &m->ip_dp, &m->ip_dn, &m->ip_dzp, &m->ip_dzn};
+                  &m->ip_dp, &m->ip_dn, &m->ip_dzp, &m->ip_dzn, &m->spill_cnt, &m->spill_off, &m->spill_col,
+                  &m->spill_val};
     for (Buf *b : all) release(*b);
     for (int a = 0; a < 3; ++a) {
         release(m->x[a]);
