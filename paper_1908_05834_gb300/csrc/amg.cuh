@@ -114,6 +114,19 @@ SolveShape solve_shape(bchar_mesh_t m);
 constexpr int64_t kSmallEntries = 40000;
 constexpr int64_t kSmallNodes = 4096;
 
+// Dynamic shared memory of a block of the solve kernel.  From kLargeEntries entries of
+// the finest level per block on (192 KB of columns and weights alone) its rows are read
+// from global memory, and the shared memory that is not asked for is L1: with 20 KB of
+// it, the sectors of the rows that a block's warps walk side by side were evicted and
+// fetched several times.  A step with 200 KB and with 128 to 144 KB, in ms: porous 48^3 (22 000
+// entries a block) 792 and 620, 64^3 3 350 and 1 890, 96^3 20 200 and 9 110, 128^3 49 000 and
+// 26 000, 1024^2 (45 000) 6 640 and 5 370; below the line 40^3 (10 600) 354 and 392,
+// 256^2 (2 600) 295 and 335, 448^2 (8 200) 856 and 878, 512^2 (10 800) 1 074 and 1 039.
+// With 112 KB the first cluster's levels do not always fit (96^3: 3 950 -> 5 020 iterations).
+constexpr size_t kSolveSmem = 200 * 1024, kLargeSmem = 144 * 1024;
+constexpr int64_t kLargeEntries = 16000;
+inline size_t solve_smem_of(int64_t e0, int blocks) { return e0 > kLargeEntries * blocks ? kLargeSmem : kSolveSmem; }
+
 inline SolveShape solve_shape_of(int64_t e0, int64_t n0, const SolveRoom &room) {
     if (room.small && e0 <= kSmallEntries && n0 <= kSmallNodes) return {kSmallCluster, kSmallCluster, 1};
     // one block per ~300 entries (two warps of rows), as many as the device holds

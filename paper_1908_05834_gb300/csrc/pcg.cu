@@ -40,7 +40,6 @@
 namespace bchar {
 
 constexpr int kNT = kSolveThreads;
-constexpr size_t kSolveSmem = 200 * 1024;  // dynamic shared memory
 // Levels of at most this many entries (and nodes) belong to the first cluster:
 // at 16 000 entries a pass of 8 blocks costs about what the grid's barrier does.
 constexpr int64_t kTierEntries = 16000;
@@ -69,6 +68,7 @@ struct PcgArgs {
     IpArgs ip;
     SolveTols tols;   // predictor (from zero), corrector (from the predictor's d)
     int vcycle;       // 1: one V-cycle only (timing)
+    unsigned smem;    // dynamic shared memory
 };
 
 // ---------------------------------------------------------------- clusters
@@ -1567,7 +1567,7 @@ template <bool ONE> __global__ void __launch_bounds__(kSolveThreads, 1) k_pcg(co
     }
     __syncthreads();
     unsigned p = 0;
-    const unsigned end = static_cast<unsigned>(kSolveSmem);
+    const unsigned end = a.smem;
     bool ok = true;
     if (b < nr && sh.t0 < sh.nlev) {
         // the vectors first: they are at the same place in every block of the cluster
@@ -1577,7 +1577,7 @@ template <bool ONE> __global__ void __launch_bounds__(kSolveThreads, 1) k_pcg(co
         if (!sh.dense) bytes += sizeof(double) * H->L[sh.nlev - 1].n;
         const int cx = (a.n0 + static_cast<int>(nr) - 1) / static_cast<int>(nr);
         if (sh.t0 == 0) bytes += sizeof(double) * 3 * cx;
-        ok = bytes <= kSolveSmem;
+        ok = bytes <= a.smem;
         if (ok) {
             for (int t = sh.t0; t < sh.nlev; ++t) {
                 const int n = H->L[t].n;
@@ -1760,7 +1760,8 @@ static void launch_pcg(bchar_mesh_t m, PcgArgs &a) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(s.grid);
     cfg.blockDim = dim3(kSolveThreads);
-    cfg.dynamicSmemBytes = kSolveSmem;
+    a.smem = static_cast<unsigned>(s.small ? kSolveSmem : solve_smem_of(a.e0, s.grid));
+    cfg.dynamicSmemBytes = a.smem;
     cfg.stream = m->stream;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;

@@ -77,3 +77,20 @@ def test_opt_ins_are_not_kept_per_process():
             assert found == ["static double *addr[256] ="]
         else:
             assert not found, (name, found)
+
+
+@needs_nvcc
+def test_shared_memory_of_large_systems_leaves_room_for_l1(tmp_path):
+    """Where the finest level's columns and weights (12 bytes an entry) cannot all be in the
+    blocks' shared memory, a block asks for less of it."""
+    for blocks, entries, smem in _run(tmp_path, r"""
+#include <cstdio>
+#include "amg.cuh"
+int main() {
+    for (int blocks : {16, 144, 152})
+        for (long long per : {1ll, 10800ll, 15999ll, 16000ll, 16001ll, 700000ll})
+            std::printf("%d %lld %zu\n", blocks, per * blocks + (per > 16000), bchar::solve_smem_of(per * blocks + (per > 16000), blocks));
+}
+"""):
+        assert smem == (200 if entries <= 16000 * blocks else 144) * 1024
+        assert smem == 144 * 1024 or entries * 12 <= smem * blocks
