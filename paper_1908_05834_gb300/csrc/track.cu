@@ -142,7 +142,7 @@ __device__ __forceinline__ void rk4(const MeshView &m, const VelView &v, int (&c
                     // the last stage moves by h/6 (k1 + 2 k2 + 2 k3 + k4), the others by their own k
                     const real k = Stage<real>::per_phi(su[p][a], phi[p]);
                     const real d = len * (s < 3 ? k : Stage<real>::add_per_phi(acc[p][a], su[p][a], phi[p]));
-                    acc[p][a] = acc[p][a] + wgt * k;
+                    acc[p][a] = s == 0 ? k : acc[p][a] + wgt * k;
                     c2[p][a] = c[p][a];
                     x2[p][a] = xi[p][a] + Stage<real>::by_width(wb[p][a], d);
                     relocate<real>(m, a, c2[p][a], x2[p][a]);
@@ -223,42 +223,73 @@ struct BallList {
 };
 static_assert(kGroupCells == 32, "a lane per cell");
 
-// phi constant: r_hat = r_K, only the centres move; a warp tracks chunks of
-// 32 kBallsPerThread balls, kBallsPerThread per lane side by side (past the end
-// of the list the last ball again).
+// phi constant: r_hat = r_K, only the centres move, kBallsPerThread per lane side by side.
+// By lists, a warp tracks chunks of 32 kBallsPerThread balls of its group (past its end the
+// last ball again).  FP64 is bound by the FP64 pipe, which takes a warp's instruction as
+// long with few lanes as with all: where the groups do not fill their chunks (stretched
+// meshes, 5 balls a cell in the mean) the incomplete last ones cost it more than equal
+// paths gain (1024^2 53.1 ms by lists, 45.4 without; 300^2 1.23 and 1.01; uniform 256^2,
+// full chunks, 0.46 and 0.55).  There a block takes consecutive balls of the mesh, lanes four
+// balls apart (cells hold four or more).  FP32: always by lists.
 constexpr int kBallsPerThread = 2;
 constexpr int kCentreThreads = 128;
+constexpr int kCentreBalls = kCentreThreads * kBallsPerThread;  // of a block at a time
+
+template <class real, int DIM>
+__device__ __forceinline__ void track_centres(const MeshView &m, const VelView &v, real h, int substeps,
+                                              const int64_t (&bs)[kBallsPerThread],
+                                              const bool (&keep)[kBallsPerThread], int32_t *out_cell, real *out_xi,
+                                              real *out_rhat) {
+    int c[kBallsPerThread][3];
+    real xi[kBallsPerThread][3];
+    int64_t Ks[kBallsPerThread];
+#pragma unroll
+    for (int p = 0; p < kBallsPerThread; ++p) ball_start<real, DIM>(m, bs[p], Ks[p], c[p], xi[p]);
+    rk4<real, DIM, kBallsPerThread>(m, v, c, xi, h, substeps, real(-1));
+#pragma unroll
+    for (int p = 0; p < kBallsPerThread; ++p) {
+        if (!keep[p]) continue;
+        const int64_t b = bs[p];
+        out_cell[b] = static_cast<int32_t>(cell_of<DIM>(m, c[p]));
+#pragma unroll
+        for (int a = 0; a < 3; ++a) out_xi[3 * b + a] = xi[p][a];
+        out_rhat[b] = Real<real>::rad(m, Ks[p]);
+    }
+}
 
 template <class real, int DIM>
 __global__ void __launch_bounds__(kCentreThreads, sizeof(real) == 4 ? 7 : 4)
-    k_track_centres(MeshView m, VelView v, real h, int substeps, int32_t *out_cell, real *out_xi, real *out_rhat) {
-    __shared__ BallList list;
-    list.build(m);
+    k_track_centres(MeshView m, VelView v, real h, int substeps, int64_t nballs, bool lists, int32_t *out_cell,
+                    real *out_xi, real *out_rhat) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    constexpr int W = kCentreThreads / 32;
-    for (int i0 = (static_cast<int>(blockIdx.y) * W + wid) * 32 * kBallsPerThread; i0 < list.total;
-         i0 += static_cast<int>(gridDim.y) * W * 32 * kBallsPerThread) {
-        int c[kBallsPerThread][3];
-        real xi[kBallsPerThread][3];
-        int64_t Ks[kBallsPerThread], bs[kBallsPerThread];
+    int64_t bs[kBallsPerThread];
+    bool keep[kBallsPerThread];
+    if (sizeof(real) == 4 || lists) {
+        __shared__ BallList list;
+        list.build(m);
+        constexpr int W = kCentreThreads / 32;
+        for (int i0 = (static_cast<int>(blockIdx.y) * W + wid) * 32 * kBallsPerThread; i0 < list.total;
+             i0 += static_cast<int>(gridDim.y) * W * 32 * kBallsPerThread) {
+#pragma unroll
+            for (int p = 0; p < kBallsPerThread; ++p) {
+                const int i = i0 + p * 32 + lane;
+                keep[p] = i < list.total;
+                bs[p] = list.ball(keep[p] ? i : list.total - 1);
+            }
+            track_centres<real, DIM>(m, v, h, substeps, bs, keep, out_cell, out_xi, out_rhat);
+        }
+    } else {
+        // two warps share 128 balls: lane l of them has 4 l .. 4 l + 3
+        const int64_t base = static_cast<int64_t>(blockIdx.x) * kCentreBalls + (wid >> 1) * 128 + 4 * lane + 2 * (wid & 1);
 #pragma unroll
         for (int p = 0; p < kBallsPerThread; ++p) {
-            const int i = i0 + p * 32 + lane;
-            bs[p] = list.ball(i < list.total ? i : list.total - 1);
-            ball_start<real, DIM>(m, bs[p], Ks[p], c[p], xi[p]);
+            keep[p] = base + p < nballs;
+            bs[p] = keep[p] ? base + p : nballs - 1;
         }
-        rk4<real, DIM, kBallsPerThread>(m, v, c, xi, h, substeps, real(-1));
-#pragma unroll
-        for (int p = 0; p < kBallsPerThread; ++p) {
-            if (i0 + p * 32 + lane >= list.total) break;
-            const int64_t b = bs[p];
-            out_cell[b] = static_cast<int32_t>(cell_of<DIM>(m, c[p]));
-#pragma unroll
-            for (int a = 0; a < 3; ++a) out_xi[3 * b + a] = xi[p][a];
-            out_rhat[b] = Real<real>::rad(m, Ks[p]);
-        }
+        track_centres<real, DIM>(m, v, h, substeps, bs, keep, out_cell, out_xi, out_rhat);
     }
 }
+static_assert(kBallsPerThread == 2 && kCentreThreads % 64 == 0, "two warps of two balls per lane share 128");
 
 // phi varying: the centre and the 2 DIM axis points C +- r e_a are tracked;
 // warp p of a block tracks point p of 32 consecutive balls (one point per lane: a
@@ -321,6 +352,12 @@ __global__ void __launch_bounds__(32 * (1 + 2 * DIM), (sizeof(real) == 4 ? 1400 
 MeshView full_view(bchar_mesh_t m);
 VelView vel_view(bchar_mesh_t m);
 
+// Every cell holds the least number of balls, and those of a group fill its chunks.
+static bool full_chunks(bchar_mesh_t m) {
+    const int64_t least = m->dim == 2 ? m->nb * m->nb : m->nb * m->nb * m->nb;
+    return m->nballs == m->nc * least && kGroupCells * least % (32 * kBallsPerThread) == 0;
+}
+
 template <class real>
 static void track_in(bchar_mesh_t m, real h, int substeps, int32_t *cell, real *xi, real *rhat) {
     MeshView mv = full_view(m);
@@ -328,14 +365,19 @@ static void track_in(bchar_mesh_t m, real h, int substeps, int32_t *cell, real *
     const int64_t most = 0x7fffffff, n32 = (m->nballs + 31) / 32;
     const unsigned chunks = static_cast<unsigned>(n32 < 1 ? 1 : (n32 > most ? most : n32));
     if (m->phi_const) {
-        // a block column per group of cells, and as many blocks per group as it has chunks in the mean
-        const unsigned groups = static_cast<unsigned>((m->nc + kGroupCells - 1) / kGroupCells);
-        const int64_t chunk = kCentreThreads * kBallsPerThread, y = ((m->nballs + groups - 1) / groups + chunk - 1) / chunk;
-        const dim3 grid(groups, static_cast<unsigned>(y < 1 ? 1 : (y > 64 ? 64 : y)));
+        dim3 grid(static_cast<unsigned>((m->nballs + kCentreBalls - 1) / kCentreBalls));
+        const bool lists = sizeof(real) == 4 || full_chunks(m);
+        if (lists) {  // a block column per group of cells, and as many blocks per group as it has chunks in the mean
+            const unsigned groups = static_cast<unsigned>((m->nc + kGroupCells - 1) / kGroupCells);
+            const int64_t y = ((m->nballs + groups - 1) / groups + kCentreBalls - 1) / kCentreBalls;
+            grid = dim3(groups, static_cast<unsigned>(y < 1 ? 1 : (y > 64 ? 64 : y)));
+        }
         if (m->dim == 2)
-            k_track_centres<real, 2><<<grid, kCentreThreads, 0, m->stream>>>(mv, vv, h, substeps, cell, xi, rhat);
+            k_track_centres<real, 2><<<grid, kCentreThreads, 0, m->stream>>>(mv, vv, h, substeps, m->nballs, lists, cell,
+                                                                               xi, rhat);
         else
-            k_track_centres<real, 3><<<grid, kCentreThreads, 0, m->stream>>>(mv, vv, h, substeps, cell, xi, rhat);
+            k_track_centres<real, 3><<<grid, kCentreThreads, 0, m->stream>>>(mv, vv, h, substeps, m->nballs, lists, cell,
+                                                                               xi, rhat);
     } else if (m->dim == 2) {
         k_track_balls<real, 2><<<chunks, 160, 0, m->stream>>>(mv, vv, h, substeps, m->nballs, cell,
                                                                                   xi, rhat);
